@@ -47,7 +47,10 @@
  *   WILSON_TUNE_CACHE=path        load tuning decisions from path, append new ones
  *   WILSON_TUNE_VERBOSE=1         report tuning candidates and decisions on stderr
  *   WILSON_HOP_VARIANT=v          pin the hop kernel variant (0..28) of every launch;
- *                                 a variant that does not fit a launch runs variant 3
+ *                                 a variant that does not fit a launch runs variant 3.
+ *                                 F64 hops run in block fixed point (no variant, not
+ *                                 tuned); on gauge handles a pinned variant takes
+ *                                 the FP64 stencil instead
  *   WILSON_HOP_BLOCK=n            block size with WILSON_HOP_VARIANT (64, 128, 256)
  *   WILSON_TEST_STAGE_TIMEOUT=1   failure-detection test only: the t-slab hop's
  *                                 staged slices never complete, so its bounded

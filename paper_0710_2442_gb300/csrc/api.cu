@@ -132,9 +132,7 @@ SolveStream& solve_stream() {
 // has passed the release (a later call on another stream gets other memory
 // or an ordering dependency the pool inserts).  Only the first call of a new
 // size grows the pool.
-cudaMemPool_t stateless_pool() {
-    static std::mutex m;
-    static cudaMemPool_t pools[64] = {};
+cudaMemPool_t device_pool(std::mutex& m, cudaMemPool_t (&pools)[64]) {
     int dev = 0;
     WL_CUDA(cudaGetDevice(&dev));
     WL_REQUIRE(dev >= 0 && dev < 64, "device ordinal out of range");
@@ -153,6 +151,18 @@ cudaMemPool_t stateless_pool() {
     }
     return pools[dev];
 }
+cudaMemPool_t stateless_pool() {
+    static std::mutex m;
+    static cudaMemPool_t pools[64] = {};
+    return device_pool(m, pools);
+}
+// The same for the fixed-point inputs of F64 handle hops; what is unused goes
+// back to the device when an F64 gauge handle is destroyed.
+cudaMemPool_t hop_pool() {
+    static std::mutex m;
+    static cudaMemPool_t pools[64] = {};
+    return device_pool(m, pools);
+}
 
 // Stream-ordered allocations of one call, released on the stream when the
 // call's scope ends (also when it throws).
@@ -164,6 +174,18 @@ struct StreamAllocs {
     void* get(size_t bytes) {
         void* q = nullptr;
         WL_CUDA(cudaMallocFromPoolAsync(&q, bytes, stateless_pool(), st));
+        p[n++] = q;
+        return q;
+    }
+    // Null where there is no memory, or the stream is being captured.
+    void* try_get(cudaMemPool_t pool, size_t bytes) {
+        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+        void* q = nullptr;
+        if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone ||
+            cudaMallocFromPoolAsync(&q, bytes, pool, st) != cudaSuccess) {
+            (void)cudaGetLastError();
+            return nullptr;
+        }
         p[n++] = q;
         return q;
     }
@@ -511,6 +533,7 @@ int wilson_gauge_create(wilson_gauge** out, const double* canon, const wilson_la
         h->f.recon = recon;
         h->f.g = g;
         h->f.buf.alloc(gauge_bytes(p, recon, g.stride));
+        if (p == P_F64) h->f.fx.alloc(gauge_bytes(P_F64, 18, g.stride));
         DevBuf tmp;
         const double* d = device_view(canon, sizeof(double) * 72 * 2 * (size_t)g.Vh, tmp, st);
         pack_gauge(h->f, d, st);
@@ -520,7 +543,11 @@ int wilson_gauge_create(wilson_gauge** out, const double* canon, const wilson_la
 }
 
 int wilson_gauge_destroy(wilson_gauge* g) {
-    return guarded([&] { delete g; });
+    return guarded([&] {
+        const bool trim = g && g->f.fx.p;
+        delete g;
+        if (trim) WL_CUDA(cudaMemPoolTrimTo(hop_pool(), 0));
+    });
 }
 
 int wilson_spinor_create(wilson_spinor** out, const wilson_lattice* L, int subset, int nrhs, int prec) {
@@ -651,6 +678,15 @@ int wilson_dslash_h(wilson_spinor* out, const wilson_gauge* gh, const wilson_spi
         h.in_rstep = a.rstep();
         h.x_rstep = a.rstep();
         h.a = 1.0;
+        // F64 on fixed-point fields: room for the input from the stream's pool
+        StreamAllocs mem(st);
+        bool fx = a.prec == P_F64 && fx_hops(gf) && fx_site_kernel(a.g, a.nrhs, a.subset == 2);
+        if (fx) {
+            h.fx_pstep = fx_spinor_bytes(a.g.stride);
+            h.fx_rstep = h.fx_pstep * a.nparity();
+            h.fx_tmp = mem.try_get(hop_pool(), (size_t)h.fx_rstep * a.nrhs);
+            fx = h.fx_tmp != nullptr;
+        }
         if (op == WILSON_OP_HOP || op == WILSON_OP_M) {
             if (a.subset == 2) {
                 WL_REQUIRE(b.subset == 2, "full input needs a full output");
@@ -676,8 +712,10 @@ int wilson_dslash_h(wilson_spinor* out, const wilson_gauge* gh, const wilson_spi
             // the intermediate field of the other parity lives with the gauge handle
             std::lock_guard<std::mutex> lk(gh->m);
             SpinorField& t = gh->tmp;
-            if (!t.buf.p || t.prec != a.prec || t.nrhs < a.nrhs || t.subset != 1 - a.subset)
-                t.alloc(a.prec, 1 - a.subset, a.nrhs, a.g);
+            if (!t.buf.p || t.prec != a.prec || t.nrhs < a.nrhs || t.subset != 1 - a.subset) {
+                if (a.prec == P_F64) t.alloc_fx(1 - a.subset, a.nrhs, a.g, 1);
+                else t.alloc(a.prec, 1 - a.subset, a.nrhs, a.g);
+            }
             const int dag = op == WILSON_OP_SCHUR_DAG;
             HopLaunch h1 = h;
             h1.out = t.block(1 - a.subset);
@@ -685,11 +723,16 @@ int wilson_dslash_h(wilson_spinor* out, const wilson_gauge* gh, const wilson_spi
             h1.out_rstep = t.rstep();
             h1.out_parity = 1 - a.subset;
             h1.dagger = dag;
+            h1.fx_out = fx;
             launch_hop(h1, st);
             HopLaunch h2 = h;
             h2.out = b.block(b.subset);
             h2.in = t.block(1 - a.subset);
             h2.in_rstep = t.rstep();
+            if (fx) {
+                h2.fx_in = t.block(1 - a.subset);
+                h2.fx_rstep = t.rstep();
+            }
             h2.x = a.block(a.subset);
             h2.xpay = 1;
             h2.a = -kappa * kappa;

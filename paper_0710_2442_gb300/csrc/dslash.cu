@@ -52,8 +52,18 @@ static void dispatch(const HopParams& P, Prec sp, Prec gp, int R, int block, int
     else throw Error(7, "unsupported spinor/gauge precision and link-storage combination");
 }
 
+bool fx_hops(const GaugeField& gf) {
+    if (gf.prec != P_F64 || !gf.fx.p) return false;
+    const char* forced = std::getenv("WILSON_HOP_VARIANT");
+    return !(forced && *forced && gf.buf.p);
+}
+
 void launch_hop(const HopLaunch& L, cudaStream_t st) {
     const GaugeField& gf = *L.gauge;
+    if (L.sprec == P_F64 && fx_hops(gf)) {
+        if (!L.tune_only) launch_hop_fx(L, st);
+        return;
+    }
     HopParams P;
     P.out = static_cast<char*>(L.out);
     P.in = static_cast<const char*>(L.in);

@@ -1,0 +1,169 @@
+// fx.cuh -- FP64 products on the integer pipe: block fixed point.
+//
+// GB300 runs two FP64 operations per SM and clock (measured 1.88 DFMA lanes
+// per clock), but 64 lanes of IMAD.WIDE (32 x 32 + 64 -> 64 bits).  A link times
+// a half spinor needs no exponent per term: the terms of one row are all
+// below |U| |h|, so the half spinor is scaled by its own largest exponent,
+// the link by 1 (SU(3): |U_ij| <= 1), and both become integers of 58 bits
+// below the scale, in two limbs of one sign, v = h 2^30 + l.  A real product is
+// three IMAD.WIDE: hh += u.h v.h and mid += u.h v.l + u.l v.h; the l l term is
+// below 2^-56 of the scale and is dropped (it vanishes where the link is exact
+// in one limb).
+//
+// Precision.  A term is exact to about 2^-57 of the row's scale, and the sum
+// of the eight hops is kept in 64-bit integers and rounded to FP64 once; the
+// FP64 stencil rounds every partial sum to 2^-53 of itself.  Measured against
+// 64-bit references the error of a hop is not larger than the FP64 stencil's
+// (mostly its final rounding).
+//
+// Ranges, with the unit of a term at 2^56 = scale: |v.h| <= 2^28, v.l < 2^30 for
+// a component, twice that after the projection's one addition; link entries
+// |u.h| <= 2^28, |u.l| < 2^30.  Six terms: |hh| <= 6 2^57 < 2^60,
+// |mid| <= 12 2^59 < 2^63; eight hops of at most 12 2^56: below 2^63.
+// Fields outside the ranges (a link entry above 1 or a link with no entry above
+// 1/4, exponents below 2^-423 or above 2^477, Inf, NaN) are reported to the caller, who
+// takes the FP64 stencil for that site.
+#pragma once
+
+#include "common.cuh"
+
+namespace wl {
+
+// exponents (biased) of half spinors that the fixed-point path takes
+constexpr int kFxEmin = 600, kFxEmax = 1500;
+// |hi word| << 1 of a link's largest entry: 0.25 <= max |U_ij| < 1 + 2^-20
+constexpr unsigned kFxLinkLo = 0x3FD00000u << 1, kFxLinkHi = 0x3FF00000u << 1 | 1u;
+
+// Right shifts that give 0 for counts of the word length and more.
+__host__ __device__ __forceinline__ unsigned fx_shr32(unsigned v, unsigned s) {
+#ifdef __CUDA_ARCH__
+    unsigned r;
+    asm("shr.u32 %0, %1, %2;" : "=r"(r) : "r"(v), "r"(s));
+    return r;
+#else
+    return s >= 32 ? 0u : v >> s;
+#endif
+}
+__host__ __device__ __forceinline__ unsigned fx_shr64_lo(unsigned long long v, unsigned s) {
+#ifdef __CUDA_ARCH__
+    unsigned long long r;
+    asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(s));
+    return (unsigned)r;
+#else
+    return s >= 64 ? 0u : (unsigned)(v >> s);
+#endif
+}
+// arithmetic, d in 0..63
+__host__ __device__ __forceinline__ long long fx_sar(long long v, int d) { return v >> d; }
+
+struct FxMag {
+    int h, l;  // magnitude, h 2^30 + l, 0 <= l < 2^30
+};
+struct FxReal {
+    int h, l;  // signed limbs
+};
+struct FxCplx {
+    FxReal re, im;
+};
+
+// A double's exponent against a scale: both come as |hi word| << 1, the scale
+// word with ones below its exponent e, so that the difference is that of the
+// exponents.  fx_scale_word(e + OFF) gives the right shift of fx_mag.
+__host__ __device__ __forceinline__ unsigned fx_scale_word(int e) { return (unsigned)e << 21 | 0x1FFFFFu; }
+__host__ __device__ __forceinline__ unsigned fx_shift(unsigned scale, unsigned hi2) { return (scale - hi2) >> 21; }
+
+// The magnitude of the double (hi, lo), its mantissa shifted right by t >= 5
+// from the top of 64 bits.  t = 6 + e - exponent puts an exponent equal to the
+// scale's below 2^58 (spinors), t = 5 + 1023 - exponent puts 1.0 at 2^58 (links).
+// Zeros and denormals have t so large that nothing is left.
+constexpr int kFxOffSpinor = 6, kFxOffLink = 5;
+__host__ __device__ __forceinline__ FxMag fx_mag(unsigned hi, unsigned lo, unsigned t) {
+    const unsigned mh = (hi & 0xFFFFFu) | 0x100000u;
+    const unsigned long long M = ((unsigned long long)mh << 32 | lo) << 11;
+    return FxMag{(int)fx_shr32((unsigned)(M >> 32), t - 2), (int)(fx_shr64_lo(M, t) & 0x3FFFFFFFu)};
+}
+// sg times the double's sign
+__host__ __device__ __forceinline__ int fx_sign(unsigned hi, int sg) { return sg - 2 * sg * (int)(hi >> 31); }
+
+// A link entry.
+__host__ __device__ __forceinline__ FxReal fx_link(unsigned hi, unsigned lo) {
+    const FxMag m = fx_mag(hi, lo, fx_shift(fx_scale_word(1023 + kFxOffLink), hi << 1));
+    const int s = fx_sign(hi, 1);
+    return FxReal{m.h * s, m.l * s};
+}
+
+// One accumulating sum of products; hh 2^60 + mid 2^30 in units of the product
+// of the two 2^58 scales.  mid starts at half of its last kept bit.
+struct FxAcc {
+    long long hh, mid;
+};
+__host__ __device__ __forceinline__ FxAcc fx_zero() { return FxAcc{0, 1LL << 29}; }
+__host__ __device__ __forceinline__ void fx_mac(FxAcc& a, const FxReal& u, const FxReal& v) {
+    a.hh += (long long)u.h * v.h;
+    a.mid += (long long)u.h * v.l;
+    a.mid += (long long)u.l * v.h;
+}
+// The sum with the scale at 2^56.
+__host__ __device__ __forceinline__ long long fx_sum(const FxAcc& a) { return a.hh + (a.mid >> 30); }
+__host__ __device__ __forceinline__ FxReal fx_neg(const FxReal& a) { return FxReal{-a.h, -a.l}; }
+
+// Links stored in this form (four 32-bit words an entry: re.h, re.l, im.h,
+// im.l) mark a link out of range by re.h of their first entry.
+constexpr unsigned kFxBadLink = 0x80000000u;
+
+#ifdef __CUDACC__
+// v 2^k as a double, rounded once, with two FP64 additions (the conversion
+// instruction takes five): v = h 2^32 + l; the words of h (biased to unsigned)
+// and l under the exponents of 2^84 and 2^52 are 2^84 + 2^63 + h 2^32 and
+// 2^52 + l, and the exponent fields take k.  bias = fx_bias(k).
+struct FxBias {
+    int a, b;   // high words of 2^(84 + k), 2^(52 + k)
+    double c;   // (2^84 + 2^63 + 2^52) 2^k
+};
+__device__ __forceinline__ FxBias fx_bias(int k) {
+    const int s = k * (1 << 20);
+    return FxBias{0x45300000 + s, 0x43300000 + s, __hiloint2double(0x45300000 + s, (int)0x80100000)};
+}
+__device__ __forceinline__ double fx_double(long long v, const FxBias& b) {
+    const int h = (int)((unsigned)(v >> 32) ^ 0x80000000u), l = (int)(unsigned)v;
+    return (__hiloint2double(b.a, h) - b.c) + __hiloint2double(b.b, l);
+}
+#endif
+
+// A sum of products of link-like numbers back to limbs at 2^58, l in [0, 2^30).
+__host__ __device__ __forceinline__ FxReal fx_requant(long long hh, long long mid) {
+    const long long n = hh * 4 + ((mid + (1LL << 27)) >> 28);
+    return FxReal{(int)(n >> 30), (int)(n & 0x3FFFFFFF)};
+}
+// re, im of a b - c d, for the third row of a 12-real link (conjugated by the caller)
+__host__ __device__ __forceinline__ FxCplx fx_cross(const FxCplx& a, const FxCplx& b, const FxCplx& c, const FxCplx& d) {
+    FxAcc r{0, 0}, i{0, 0};
+    fx_mac(r, a.re, b.re);
+    fx_mac(r, fx_neg(a.im), b.im);
+    fx_mac(r, fx_neg(c.re), d.re);
+    fx_mac(r, c.im, d.im);
+    fx_mac(i, a.re, b.im);
+    fx_mac(i, a.im, b.re);
+    fx_mac(i, fx_neg(c.re), d.im);
+    fx_mac(i, fx_neg(c.im), d.re);
+    return FxCplx{fx_requant(r.hh, r.mid), fx_requant(i.hh, i.mid)};
+}
+__host__ __device__ __forceinline__ void fx_recon_row2(FxCplx U[3][3]) {
+#pragma unroll
+    for (int q = 0; q < 3; q++) {
+        const int a = (q + 1) % 3, b = (q + 2) % 3;
+        U[2][q] = fx_cross(U[0][a], U[1][b], U[0][b], U[1][a]);
+        U[2][q].im = fx_neg(U[2][q].im);
+    }
+}
+// eta h (a boundary phase on a projected component)
+__host__ __device__ __forceinline__ FxCplx fx_phase(const FxCplx& eta, const FxCplx& h) {
+    FxAcc r{0, 0}, i{0, 0};
+    fx_mac(r, eta.re, h.re);
+    fx_mac(r, fx_neg(eta.im), h.im);
+    fx_mac(i, eta.re, h.im);
+    fx_mac(i, eta.im, h.re);
+    return FxCplx{fx_requant(r.hh, r.mid), fx_requant(i.hh, i.mid)};
+}
+
+}  // namespace wl

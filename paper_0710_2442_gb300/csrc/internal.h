@@ -150,6 +150,7 @@ struct SpinorField {
     // bytes from one right-hand side's blocks to the next one's
     long long rstep() const { return (long long)nparity() * pbytes; }
     void alloc(Prec p, int sub, int nr, const Geom& geom);
+    void alloc_fx(int sub, int nr, const Geom& geom, int fields);  // F64, or `fields` fixed-point fields a block
 };
 
 struct GaugeField {
@@ -157,6 +158,11 @@ struct GaugeField {
     int recon = 12;
     Geom g{};
     DevBuf buf;
+    // F64 links of the fixed-point hops (dslash_fx.cuh), 18 reals for either
+    // recon; links out of their range are read from buf, or where there is
+    // none from canon (canonical links the caller keeps).
+    DevBuf fx;
+    const double* canon = nullptr;
 };
 
 // Per-device scratch: reduction partials and counters.
@@ -208,8 +214,29 @@ struct HopLaunch {
     int grid_cap;          // max blocks of a reducing launch (0 = no cap)
     int tune_only;         // 1: tune the launch configuration if it is not known yet, launch nothing else
     int no_tune;           // 1: take a cached decision or the default configuration, never time candidates
+    // F64 on the fixed-point hops (fx_hops(*gauge)); fields of fx_spinor_bytes per parity
+    const void* fx_in;     // the input as a fixed-point field, or null
+    void* fx_tmp;          // else room to convert it (null: the kernel that takes doubles)
+    long long fx_pstep;    // steps of either
+    long long fx_rstep;
+    int fx_out;            // out is a fixed-point field (plain hop, fx_site_kernel only)
 };
 void launch_hop(const HopLaunch& L, cudaStream_t st);
+
+// FP64 hops on the integer pipe (dslash_fx.cu).  They run wherever the links
+// have a fixed-point form, unless WILSON_HOP_VARIANT pins the FP64 stencil and the
+// links are there as doubles.
+bool fx_hops(const GaugeField& gf);
+void launch_hop_fx(const HopLaunch& L, cudaStream_t st);
+long long fx_spinor_bytes(int stride);  // one parity, one rhs
+// Whether the kernel on fixed-point fields is taken, given room for them: below
+// kFxSiteMin output sites the conversion costs more than it saves (12^4: 14 against 12.3 + 4.2 us
+// a hop; 16^3 x 32: 43 against 27.6 + 6.2 us).
+constexpr long long kFxSiteMin = 20000;
+bool fx_site_kernel(const Geom& g, int nrhs, int full);
+void fx_convert(void* dst, long long dst_pstep, long long dst_rstep, const void* src, long long src_pstep,
+                long long src_rstep, int nrhs, int full, const Geom& g, const int* skip, int skip_stride,
+                cudaStream_t st);
 int hop_grid_blocks(const Geom& g, int block, int grid_cap);
 
 // canonical <-> SoA

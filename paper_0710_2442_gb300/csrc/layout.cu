@@ -9,6 +9,7 @@
 // component / scale rounded to nearest even).  Links: rows 0 and 1 only for
 // 12-real storage (row 2 is rebuilt in the kernels, exact for SU(3)); links
 // are never scaled (|U_ij| <= 1).
+#include "fx.cuh"
 #include "internal.h"
 
 namespace wl {
@@ -49,6 +50,15 @@ void SpinorField::alloc(Prec p, int sub, int nr, const Geom& geom) {
     nrhs = nr;
     g = geom;
     pbytes = (spinor_field_bytes(p, g.stride) + 255) / 256 * 256;
+    buf.alloc((size_t)pbytes * nparity() * nrhs);
+}
+
+void SpinorField::alloc_fx(int sub, int nr, const Geom& geom, int fields) {
+    prec = P_F64;
+    subset = sub;
+    nrhs = nr;
+    g = geom;
+    pbytes = fx_spinor_bytes(g.stride) * fields;
     buf.alloc((size_t)pbytes * nparity() * nrhs);
 }
 
@@ -221,6 +231,45 @@ __global__ void pack_gauge_kernel(const double2* __restrict__ canon, char* base,
     }
 }
 
+// F64 links in fixed point (fx.cuh): nine words per link whatever R, the third row
+// rebuilt for R = 12; a link out of range is marked.  DBL: the doubles too.
+template <int R, bool DBL>
+__global__ void pack_gauge_fx_kernel(const double2* __restrict__ canon, char* base, uint4* fx, Geom g) {
+    const long long V = 2LL * g.Vh;
+    for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < V; s += (long long)gridDim.x * blockDim.x) {
+        int c[4];
+        site_coords_full(s, g, c);
+        const int p = (c[0] + c[1] + c[2] + c[3]) & 1;
+        const int h = (int)(s >> 1);
+#pragma unroll
+        for (int mu = 0; mu < 4; mu++) {
+            double2 u[9];
+            const double2* src = canon + (s * 4 + mu) * 9;
+#pragma unroll
+            for (int k = 0; k < R / 2; k++) u[k] = src[k];
+            if (DBL) store_link<P_F64, R>(base, g.stride, p * 4 + mu, h, u);
+            FxCplx f[3][3];
+            unsigned mx = 0;
+#pragma unroll
+            for (int k = 0; k < R / 2; k++) {
+                const unsigned rh = (unsigned)__double2hiint(u[k].x), ih = (unsigned)__double2hiint(u[k].y);
+                mx = max(mx, max(rh << 1, ih << 1));
+                f[k / 3][k % 3] = FxCplx{fx_link(rh, (unsigned)__double2loint(u[k].x)),
+                                         fx_link(ih, (unsigned)__double2loint(u[k].y))};
+            }
+            if (R == 12) fx_recon_row2(f);
+            if (mx < kFxLinkLo || mx > kFxLinkHi) f[0][0].re.h = (int)kFxBadLink;
+            uint4* b = fx + (size_t)(p * 4 + mu) * 9 * g.stride + h;
+#pragma unroll
+            for (int k = 0; k < 9; k++) {
+                const FxCplx& z = f[k / 3][k % 3];
+                b[(size_t)k * g.stride] =
+                    make_uint4((unsigned)z.re.h, (unsigned)z.re.l, (unsigned)z.im.h, (unsigned)z.im.l);
+            }
+        }
+    }
+}
+
 void pack_gauge(GaugeField& gf, const double* canon, cudaStream_t st) {
     const long long V = 2LL * gf.g.Vh;
     const int block = 256, grid = grid_for(V, block);
@@ -228,6 +277,15 @@ void pack_gauge(GaugeField& gf, const double* canon, cudaStream_t st) {
     char* base = gf.buf.as<char>();
     const Prec p = gf.prec;
     const int R = gf.recon;
+    if (p == P_F64 && gf.fx.p) {
+        uint4* fx = gf.fx.as<uint4>();
+        if (R == 18 && base) pack_gauge_fx_kernel<18, true><<<grid, block, 0, st>>>(src, base, fx, gf.g);
+        else if (R == 18) pack_gauge_fx_kernel<18, false><<<grid, block, 0, st>>>(src, base, fx, gf.g);
+        else if (base) pack_gauge_fx_kernel<12, true><<<grid, block, 0, st>>>(src, base, fx, gf.g);
+        else pack_gauge_fx_kernel<12, false><<<grid, block, 0, st>>>(src, base, fx, gf.g);
+        WL_LAUNCH_CHECK();
+        return;
+    }
     if (p == P_F64 && R == 18) pack_gauge_kernel<P_F64, 18><<<grid, block, 0, st>>>(src, base, gf.g);
     else if (p == P_F64 && R == 12) pack_gauge_kernel<P_F64, 12><<<grid, block, 0, st>>>(src, base, gf.g);
     else if (p == P_F32 && R == 18) pack_gauge_kernel<P_F32, 18><<<grid, block, 0, st>>>(src, base, gf.g);

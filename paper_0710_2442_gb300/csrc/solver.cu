@@ -52,7 +52,15 @@ namespace {
 void schur_launch(const GaugeField& gf, Prec sp, Vec out, Vec in, Vec tmp, int nrhs, double kappa, int dag,
                   const RedArgs* red, const int* skip, int skip_stride, int grid_cap, bool tune_only,
                   cudaStream_t st) {
+    // F64 on fixed-point fields: the input is converted, the intermediate field
+    // stays in that form (F64 tmp blocks have room for both, SpinorField::alloc_fx)
+    const bool site = sp == P_F64 && fx_hops(gf) && fx_site_kernel(gf.g, nrhs, 0);
     HopLaunch a{};
+    if (site) {
+        a.fx_tmp = static_cast<char*>(tmp.p) + fx_spinor_bytes(gf.g.stride);
+        a.fx_rstep = tmp.rstep;
+        a.fx_out = 1;
+    }
     a.tune_only = tune_only;
     a.out = tmp.p;
     a.in = in.p;
@@ -68,6 +76,10 @@ void schur_launch(const GaugeField& gf, Prec sp, Vec out, Vec in, Vec tmp, int n
     a.skip_stride = skip_stride;
     launch_hop(a, st);
     HopLaunch b{};
+    if (site) {
+        b.fx_in = tmp.p;
+        b.fx_rstep = tmp.rstep;
+    }
     b.tune_only = tune_only;
     b.out = out.p;
     b.in = tmp.p;
@@ -123,7 +135,8 @@ struct Inner {
         p.alloc(ip, 0, nr, g);
         q.alloc(ip, 0, nr, g);
         r.alloc(ip, 0, nr, g);
-        t.alloc(ip, 1, nr, g);
+        if (ip == P_F64) t.alloc_fx(1, nr, g, 2);
+        else t.alloc(ip, 1, nr, g);
     }
     Vec s_in() const { return has_slow ? vec(slow, 0) : vec(s, 0); }
 };
@@ -157,7 +170,8 @@ std::vector<SolveStats> cg_solve_prepared(SpinorField& x, const SpinorField& b, 
     bhat.alloc(P_F64, 0, nr, g);
     r64.alloc(P_F64, 0, nr, g);
     q64.alloc(P_F64, 0, nr, g);
-    t64.alloc(P_F64, 1, nr, g);
+    t64.alloc_fx(1, nr, g, 2);
+    const long long fx_step = fx_spinor_bytes(g.stride);  // t64: room for two fixed-point fields
 
     // |b_k|^2 over both parities
     norm2(P_F64, vec(b, 0), g, nr, red.args(slot(0), FIN_STORE, d_res, nullptr), grid_cap, st);
@@ -177,6 +191,8 @@ std::vector<SolveStats> cg_solve_prepared(SpinorField& x, const SpinorField& b, 
         h.gauge = &g64;
         h.sprec = P_F64;
         h.out_parity = 0;
+        h.fx_tmp = t64.buf.p;
+        h.fx_rstep = t64.rstep();
         launch_hop(h, st);
         hops += 1;
     }
@@ -471,6 +487,8 @@ std::vector<SolveStats> cg_solve_prepared(SpinorField& x, const SpinorField& b, 
         h.gauge = &g64;
         h.sprec = P_F64;
         h.out_parity = 1;
+        h.fx_tmp = t64.buf.p;
+        h.fx_rstep = t64.rstep();
         launch_hop(h, st);
         hops += 1;
     }
@@ -494,6 +512,9 @@ std::vector<SolveStats> cg_solve_prepared(SpinorField& x, const SpinorField& b, 
         h.a = -kappa;
         h.gauge = &g64;
         h.sprec = P_F64;
+        h.fx_tmp = t64.buf.p;
+        h.fx_pstep = fx_step;
+        h.fx_rstep = t64.rstep();
         launch_hop(h, st);
         hops += 2;
         xmy_norm64(Vec{nullptr, 0}, vec(b, 0), vec(mx, 0), g, nr,
@@ -526,7 +547,8 @@ std::vector<SolveStats> cg_solve(double* xc, const double* gauge_canon, const do
     g64.prec = P_F64;
     g64.recon = 18;
     g64.g = g;
-    g64.buf.alloc(gauge_bytes(P_F64, 18, g.stride));
+    g64.fx.alloc(gauge_bytes(P_F64, 18, g.stride));
+    g64.canon = gauge_canon;
     pack_gauge(g64, gauge_canon, st);
     GaugeField glo;
     const GaugeField* inner_gauge = &g64;
@@ -534,7 +556,12 @@ std::vector<SolveStats> cg_solve(double* xc, const double* gauge_canon, const do
         glo.prec = prm.inner;
         glo.recon = prm.recon;
         glo.g = g;
-        glo.buf.alloc(gauge_bytes(prm.inner, prm.recon, g.stride));
+        if (prm.inner == P_F64) {
+            glo.fx.alloc(gauge_bytes(P_F64, 18, g.stride));
+            glo.canon = gauge_canon;
+        } else {
+            glo.buf.alloc(gauge_bytes(prm.inner, prm.recon, g.stride));
+        }
         pack_gauge(glo, gauge_canon, st);
         inner_gauge = &glo;
     }
