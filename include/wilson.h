@@ -113,13 +113,12 @@ typedef struct {
 
 /* ---------------------------------------------------------------------- */
 /* Stateless calls on canonical complex128 device fields (Sec. 5, Eq. 3).  */
-/* Computed in FP64 with 18-real links.  Each call packs its inputs into   */
-/* workspace taken from a per-device memory pool of the library with       */
-/* stream-ordered allocation on the caller's stream (the pool keeps its    */
-/* memory, so only the first call of a size grows it).  The calls do not   */
-/* synchronise, except that the first call for a new lattice, operator    */
-/* and dagger flag times the kernel's launch configurations (autotuning)   */
-/* and so synchronises the stream once; WILSON_TUNE=0 turns that off.      */
+/* FP64 results from 18-real links (computed in block fixed point, where    */
+/* that is at least as accurate, else in FP64).  Small lattices read links  */
+/* and fields as they are; larger ones convert them into workspace taken    */
+/* from a per-device memory pool of the library with stream-ordered         */
+/* allocation on the caller's stream (the pool keeps its memory, so only    */
+/* the first call of a size grows it).  The calls do not synchronise.       */
 /* ---------------------------------------------------------------------- */
 
 /* out = D_h in (op = HOP) or M in (op = M), full lattice.
@@ -366,17 +365,14 @@ int wilson_dd_hop(wilson_spinor* out, const wilson_gauge* g, const wilson_spinor
 #define WILSON_NOALLOC_SCRATCH_BYTES (32u << 20)
 
 /* Same arguments, result and precision (FP64, 18-real links) as
- * wilson_dslash_eo, but the packed fields live in one fixed device array of
+ * wilson_dslash_eo, but the workspace lies in one fixed device array of
  * WILSON_NOALLOC_SCRATCH_BYTES (32 MiB) that every GPU loading the library
  * holds until exit; nothing is allocated or freed.  Fits lattices with
  * V/2 up to about 19,000 sites (8^4, 12^4, 8^3 x 32, 12^3 x 22); larger ones
  * return WILSON_ERR_ARG before any work.  The first call in a CUDA context
  * resolves the array's device address in that context (cudaGetSymbolAddress)
- * and caches it under the context's unique ID.  The call never times launch
- * configurations: it uses the one an earlier wilson_dslash_eo call on the
- * same lattice and operator chose (or the WILSON_TUNE_CACHE file holds), else
- * a fixed default; it neither allocates nor synchronises and is
- * asynchronous on the stream.  All calls on a device share the array (it
+ * and caches it under the context's unique ID.  The call neither allocates nor
+ * synchronises and is asynchronous on the stream.  All calls on a device share the array (it
  * keeps the last call's contents; nothing in it needs clearing): calls whose
  * GPU work overlaps race on it and must be serialised by the caller. */
 int wilson_dslash_eo_noalloc(double* out, const double* gauge, const double* in, const wilson_lattice* L,

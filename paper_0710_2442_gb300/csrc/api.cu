@@ -194,22 +194,10 @@ struct StreamAllocs {
     }
 };
 
-// A packed FP64 field of one parity subset (0, 1 or 2 = both) in pool memory.
-void borrow_spinor(SpinorField& f, int subset, const Geom& g, StreamAllocs& a, BorrowGuard& guard) {
-    f.prec = P_F64;
-    f.subset = subset;
-    f.nrhs = 1;
-    f.g = g;
-    f.pbytes = spinor_field_bytes(P_F64, g.stride);
-    const size_t bytes = (size_t)f.pbytes * f.nparity();
-    guard.borrow(f.buf, a.get(bytes), bytes);
-}
-void borrow_gauge(GaugeField& gf, const Geom& g, StreamAllocs& a, BorrowGuard& guard) {
-    gf.prec = P_F64;
-    gf.recon = 18;
-    gf.g = g;
-    const size_t bytes = (size_t)gauge_bytes(P_F64, 18, g.stride);
-    guard.borrow(gf.buf, a.get(bytes), bytes);
+// Whether two ranges of device memory overlap.
+bool overlap(const void* a, size_t na, const void* b, size_t nb) {
+    const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
+    return x < y + nb && y < x + na;
 }
 
 }  // namespace
@@ -255,6 +243,76 @@ bool wl::is_device_ptr(const void* p) {
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
+// An operator on canonical F64 fields (arguments checked by the callers): of a
+// full field (parity 2: HOP, M) or onto one parity (HOP, SCHUR, SCHUR_DAG).
+// Small lattices (fx_site_kernel) take the kernel that reads canonical links and
+// fields as they are: one launch a hop and nothing packed.  Larger ones convert the links
+// and the input to fixed point first.  Workspace: scratch (of the given size), or
+// the stateless pool where there is none; with scratch nothing is allocated.
+void wl::stateless_op(double* out, const double* gauge, const double* in, const Geom& g, int parity, double kappa, int op,
+                      cudaStream_t st, void* scratch, size_t scratch_bytes) {
+    const bool full = parity == 2, schur = op == WILSON_OP_SCHUR || op == WILSON_OP_SCHUR_DAG;
+    StreamAllocs mem(st);
+    size_t used = 0;
+    auto room = [&](size_t bytes) -> void* {
+        if (!scratch) return mem.get(bytes);
+        bytes = (bytes + 255) / 256 * 256;
+        WL_REQUIRE(used + bytes <= scratch_bytes, "scratch too small");
+        used += bytes;
+        return static_cast<char*>(scratch) + used - bytes;
+    };
+    const size_t field = sizeof(double) * 24 * (size_t)g.Vh * (full ? 2 : 1);
+    // the kernels read the inputs while they write the output: one that overlaps
+    // them (not in by contract, but accepted) is written elsewhere first
+    double* dst = out;
+    if (overlap(out, field, in, field) || overlap(out, field, gauge, sizeof(double) * 144 * (size_t)g.Vh))
+        dst = static_cast<double*>(room(field));
+    GaugeField gf;
+    BorrowGuard guard;  // declared after gf: detaches its view first
+    gf.prec = P_F64;
+    gf.recon = 18;
+    gf.g = g;
+    gf.canon = gauge;
+    HopLaunch h{};
+    h.gauge = &gf;
+    h.sprec = P_F64;
+    h.out = dst;
+    h.in = in;
+    h.x = in;
+    h.full = full;
+    h.out_parity = full ? 0 : parity;
+    h.dagger = op == WILSON_OP_SCHUR_DAG;
+    h.xpay = op != WILSON_OP_HOP;
+    h.a = op == WILSON_OP_HOP ? 1.0 : op == WILSON_OP_M ? -kappa : -kappa * kappa;
+    h.canon = kCanonIn | kCanonX | kCanonOut;
+    const bool site = !scratch && fx_site_kernel(g, 1, full);
+    const size_t fx = (size_t)fx_spinor_bytes(g.stride);
+    if (site) {
+        const size_t bytes = (size_t)gauge_bytes(P_F64, 18, g.stride);
+        guard.borrow(gf.fx, mem.get(bytes), bytes);
+        pack_gauge(gf, gauge, st);
+        h.fx_tmp = mem.get(fx * (full ? 2 : 1));
+        h.fx_pstep = (long long)fx;
+    }
+    if (schur) {
+        // Mhat_p = 1 - kappa^2 D_{p,1-p} D_{1-p,p}
+        void* t = room(site ? fx : (size_t)spinor_field_bytes(P_F64, g.stride));
+        HopLaunch h1 = h;
+        h1.out = t;
+        h1.out_parity = 1 - parity;
+        h1.xpay = 0;
+        h1.a = 1.0;
+        h1.canon = kCanonIn;
+        h1.fx_out = site;
+        launch_hop_fx(h1, st);
+        h.in = t;
+        h.canon = kCanonX | kCanonOut;
+        if (site) h.fx_in = t;
+    }
+    launch_hop_fx(h, st);
+    if (dst != out) WL_CUDA(cudaMemcpyAsync(out, dst, field, cudaMemcpyDeviceToDevice, st));
+}
+
 // ---------------------------------------------------------------------------
 extern "C" {
 
@@ -289,30 +347,7 @@ int wilson_dslash(double* out, const double* gauge, const double* in, const wils
         check_device();
         WL_REQUIRE(is_device_ptr(out) && is_device_ptr(in) && is_device_ptr(gauge),
                    "wilson_dslash takes device pointers");
-        cudaStream_t st = static_cast<cudaStream_t>(stream);
-        StreamAllocs mem(st);
-        GaugeField gf;
-        SpinorField a, b;
-        BorrowGuard guard;  // declared last: detaches the views first, and mem releases the memory last
-        borrow_gauge(gf, g, mem, guard);
-        borrow_spinor(a, 2, g, mem, guard);
-        borrow_spinor(b, 2, g, mem, guard);
-        pack_gauge(gf, gauge, st);
-        pack_spinor(a, 0, in, st);
-        HopLaunch h{};
-        h.out = b.block(0);
-        h.in = a.block(0);
-        h.x = a.block(0);
-        h.out_pstep = b.pbytes;
-        h.in_pstep = a.pbytes;
-        h.x_pstep = a.pbytes;
-        h.full = 1;
-        h.gauge = &gf;
-        h.sprec = P_F64;
-        h.xpay = op == WILSON_OP_M;
-        h.a = op == WILSON_OP_M ? -kappa : 1.0;
-        launch_hop(h, st);
-        unpack_spinor(b, 0, out, st);
+        stateless_op(out, gauge, in, g, 2, kappa, op, static_cast<cudaStream_t>(stream), nullptr, 0);
     });
 }
 
@@ -331,52 +366,7 @@ int wilson_dslash_eo(double* out, const double* gauge, const double* in, const w
         check_device();
         WL_REQUIRE(is_device_ptr(out) && is_device_ptr(in) && is_device_ptr(gauge),
                    "wilson_dslash_eo takes device pointers");
-        cudaStream_t st = static_cast<cudaStream_t>(stream);
-        StreamAllocs mem(st);
-        const int pin = op == WILSON_OP_HOP ? 1 - out_parity : out_parity;
-        GaugeField gf;
-        SpinorField a, b, t;
-        BorrowGuard guard;  // declared last: detaches the views first, and mem releases the memory last
-        borrow_gauge(gf, g, mem, guard);
-        borrow_spinor(a, pin, g, mem, guard);
-        borrow_spinor(b, out_parity, g, mem, guard);
-        pack_gauge(gf, gauge, st);
-        pack_spinor(a, 0, in, st);
-        if (op == WILSON_OP_HOP) {
-            HopLaunch h{};
-            h.out = b.block(out_parity);
-            h.in = a.block(pin);
-            h.gauge = &gf;
-            h.sprec = P_F64;
-            h.out_parity = out_parity;
-            h.a = 1.0;
-            launch_hop(h, st);
-        } else {
-            // Mhat_p = 1 - kappa^2 D_{p,1-p} D_{1-p,p}
-            borrow_spinor(t, 1 - out_parity, g, mem, guard);
-            const int dag = op == WILSON_OP_SCHUR_DAG;
-            HopLaunch h1{};
-            h1.out = t.block(1 - out_parity);
-            h1.in = a.block(pin);
-            h1.gauge = &gf;
-            h1.sprec = P_F64;
-            h1.out_parity = 1 - out_parity;
-            h1.dagger = dag;
-            h1.a = 1.0;
-            launch_hop(h1, st);
-            HopLaunch h2{};
-            h2.out = b.block(out_parity);
-            h2.in = t.block(1 - out_parity);
-            h2.x = a.block(pin);
-            h2.xpay = 1;
-            h2.a = -kappa * kappa;
-            h2.gauge = &gf;
-            h2.sprec = P_F64;
-            h2.out_parity = out_parity;
-            h2.dagger = dag;
-            launch_hop(h2, st);
-        }
-        unpack_spinor(b, 0, out, st);
+        stateless_op(out, gauge, in, g, out_parity, kappa, op, static_cast<cudaStream_t>(stream), nullptr, 0);
     });
 }
 

@@ -53,7 +53,7 @@ static void dispatch(const HopParams& P, Prec sp, Prec gp, int R, int block, int
 }
 
 bool fx_hops(const GaugeField& gf) {
-    if (gf.prec != P_F64 || !gf.fx.p) return false;
+    if (gf.prec != P_F64 || !(gf.fx.p || gf.canon)) return false;
     const char* forced = std::getenv("WILSON_HOP_VARIANT");
     return !(forced && *forced && gf.buf.p);
 }

@@ -15,6 +15,10 @@ constexpr int kSplitBlocks = 4;
 FxField soa(const void* p, long long pstep, long long rstep, int stride) {
     return FxField{static_cast<char*>(const_cast<void*>(p)), pstep, rstep, 1, stride, 0};
 }
+// A canonical field: half fields by half-site index, full ones by site.
+FxField canonical(const void* p, int full) {
+    return FxField{static_cast<char*>(const_cast<void*>(p)), 0, 0, 12, 1, full};
+}
 
 template <bool OUTFX, bool RED>
 void launch_site(const FxParams& P, int blocks, int ny, cudaStream_t st) {
@@ -41,15 +45,6 @@ bool fx_site_kernel(const Geom& g, int nrhs, int full) {
     return (long long)g.Vh * std::max(nrhs, 1) * (full ? 2 : 1) >= kFxSiteMin;
 }
 
-void fx_convert(void* dst, long long dst_pstep, long long dst_rstep, const void* src, long long src_pstep,
-                long long src_rstep, int nrhs, int full, const Geom& g, const int* skip, int skip_stride,
-                cudaStream_t st) {
-    const FxField f = soa(src, full ? src_pstep : 0, src_rstep, g.stride);
-    const int n = nrhs > 1 ? nrhs : 1;
-    launch_dep(fx_pack_kernel, dim3((g.Vh + 127) / 128 * n, full ? 2 : 1), dim3(128), st, f, static_cast<char*>(dst),
-               dst_pstep, dst_rstep, n, 0, full ? 2 : 1, g, skip, skip_stride);
-}
-
 void launch_hop_fx(const HopLaunch& L, cudaStream_t st) {
     const GaugeField& gf = *L.gauge;
     const Geom& g = gf.g;
@@ -58,13 +53,15 @@ void launch_hop_fx(const HopLaunch& L, cudaStream_t st) {
     WL_REQUIRE(!L.xpay || L.x, "xpay needs a field");
     WL_REQUIRE(!L.red || !L.full, "reducing hop launches are single-parity");
     FxParams P;
-    P.out = soa(L.out, L.full ? L.out_pstep : 0, L.out_rstep, g.stride);
-    P.in = soa(L.in, L.full ? L.in_pstep : 0, L.in_rstep, g.stride);
-    P.x = soa(L.x, L.full ? L.x_pstep : 0, L.x_rstep, g.stride);
+    WL_REQUIRE(!L.canon || nrhs == 1, "canonical fields: one right-hand side");
+    P.out = L.canon & kCanonOut ? canonical(L.out, L.full) : soa(L.out, L.full ? L.out_pstep : 0, L.out_rstep, g.stride);
+    P.in = L.canon & kCanonIn ? canonical(L.in, L.full) : soa(L.in, L.full ? L.in_pstep : 0, L.in_rstep, g.stride);
+    P.x = L.canon & kCanonX ? canonical(L.x, L.full) : soa(L.x, L.full ? L.x_pstep : 0, L.x_rstep, g.stride);
     P.u = FxLinks{gf.fx.as<const char>(), 36 * s, 9 * s, 1, g.stride, 0};
     P.un_recon = gf.recon;
     if (gf.canon) {
         P.un = FxLinks{reinterpret_cast<const char*>(gf.canon), 0, 9, 36, 1, 1};
+        if (!gf.fx.p) P.u = P.un;
     } else {
         const long long w = gf.recon / 2 * s;
         P.un = FxLinks{gf.buf.as<const char>(), 4 * w, w, 1, g.stride, 0};
@@ -80,7 +77,7 @@ void launch_hop_fx(const HopLaunch& L, cudaStream_t st) {
     P.scaled = !L.xpay && L.a != 1.0;
     P.red = L.red ? *L.red : RedArgs{};
     P.skip = L.skip;
-    const bool site = L.fx_in || (L.fx_tmp && fx_site_kernel(g, nrhs, L.full));
+    const bool site = gf.fx.p && (L.fx_in || (L.fx_tmp && fx_site_kernel(g, nrhs, L.full)));
     WL_REQUIRE(site || !L.fx_out, "a fixed-point output needs the site kernel");
     const int sites = site ? kSiteThreads / 2 : 32;
     int cap = 0;
@@ -88,15 +85,21 @@ void launch_hop_fx(const HopLaunch& L, cudaStream_t st) {
     const int blocks = hop_grid_blocks(g, sites, cap);
     WL_REQUIRE(!L.red || blocks <= L.red->slot_cap, "reduction capacity below the grid size");
     if (!site) {
-        if (L.red) launch_split<true, true>(P, blocks, ny, st);
-        else launch_split<true, false>(P, blocks, ny, st);
+        if (!gf.fx.p) {
+            WL_REQUIRE(gf.recon == 18 && !L.red, "links as doubles: 18 reals, no reduction");
+            launch_split<false, false>(P, blocks, ny, st);
+        } else if (L.red) {
+            launch_split<true, true>(P, blocks, ny, st);
+        } else {
+            launch_split<true, false>(P, blocks, ny, st);
+        }
         return;
     }
     if (L.fx_in) {
         P.in = soa(L.fx_in, L.full ? L.fx_pstep : 0, L.fx_rstep, g.stride);
     } else {
-        fx_convert(L.fx_tmp, L.fx_pstep, L.fx_rstep, L.in, L.in_pstep, L.in_rstep, nrhs, L.full, g, L.skip,
-                   L.skip_stride, st);
+        launch_dep(fx_pack_kernel, dim3((g.Vh + 127) / 128 * nrhs, ny), dim3(128), st, P.in,
+                   static_cast<char*>(L.fx_tmp), L.fx_pstep, L.fx_rstep, nrhs, 0, ny, g, L.skip, L.skip_stride);
         P.in = soa(L.fx_tmp, L.full ? L.fx_pstep : 0, L.fx_rstep, g.stride);
     }
     if (L.fx_out) {

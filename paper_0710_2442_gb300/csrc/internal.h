@@ -160,7 +160,8 @@ struct GaugeField {
     DevBuf buf;
     // F64 links of the fixed-point hops (dslash_fx.cuh), 18 reals for either
     // recon; links out of their range are read from buf, or where there is
-    // none from canon (canonical links the caller keeps).
+    // none from canon (canonical links the caller keeps).  canon alone: the
+    // kernel for small lattices, which converts the links itself.
     DevBuf fx;
     const double* canon = nullptr;
 };
@@ -220,7 +221,9 @@ struct HopLaunch {
     long long fx_pstep;    // steps of either
     long long fx_rstep;
     int fx_out;            // out is a fixed-point field (plain hop, fx_site_kernel only)
+    int canon;             // bits kCanonIn, kCanonX, kCanonOut: that field is canonical (one rhs)
 };
+constexpr int kCanonIn = 1, kCanonX = 2, kCanonOut = 4;
 void launch_hop(const HopLaunch& L, cudaStream_t st);
 
 // FP64 hops on the integer pipe (dslash_fx.cu).  They run wherever the links
@@ -234,9 +237,6 @@ long long fx_spinor_bytes(int stride);  // one parity, one rhs
 // a hop; 16^3 x 32: 43 against 27.6 + 6.2 us).
 constexpr long long kFxSiteMin = 20000;
 bool fx_site_kernel(const Geom& g, int nrhs, int full);
-void fx_convert(void* dst, long long dst_pstep, long long dst_rstep, const void* src, long long src_pstep,
-                long long src_rstep, int nrhs, int full, const Geom& g, const int* skip, int skip_stride,
-                cudaStream_t st);
 int hop_grid_blocks(const Geom& g, int block, int grid_cap);
 
 // canonical <-> SoA
@@ -251,6 +251,10 @@ struct NvtxRange {
     explicit NvtxRange(const char* name) { nvtxRangePushA(name); }
     ~NvtxRange() { nvtxRangePop(); }
 };
+
+// The stateless operators (api.cu).
+void stateless_op(double* out, const double* gauge, const double* in, const Geom& g, int parity, double kappa, int op,
+                  cudaStream_t st, void* scratch, size_t scratch_bytes);
 
 // Set the calling thread's message returned by wilson_last_error().
 void record_error(const std::string& msg);

@@ -1,21 +1,22 @@
 // noalloc.cu -- wilson_dslash_eo_noalloc: the even-odd hopping term and the
 // Schur operator on canonical FP64 device fields, with no device allocation.
 //
-// Why it exists.  wilson_dslash_eo packs its canonical inputs into the
-// kernels' SoA layout in memory it takes from a device memory pool.  Some
-// callers cannot let a library allocate device memory at all: hosts whose
-// memory manager owns the whole device (a framework's caching allocator, a
-// fixed arena sized to the card), and latency-critical loops that must never
-// block in the allocator or grow a pool behind the caller's back.  This entry
-// point runs the same kernels with the packed fields placed in one file-scope
-// device array of fixed size instead.
+// Why it exists.  wilson_dslash_eo takes its workspace (a Schur operator's
+// intermediate field; larger lattices' converted links and input) from a device memory
+// pool.  Some callers cannot let a library allocate device memory at all: hosts whose memory manager
+// owns the whole device (a framework's caching allocator, a fixed arena sized to
+// the card), and latency-critical loops that must never block in the allocator or
+// grow a pool behind the caller's back.  This entry point runs the same kernels
+// with that workspace placed in one file-scope device array of fixed size instead.
 //
 // The scratch array.  WILSON_NOALLOC_SCRATCH_BYTES (32 MiB) of device memory
 // declared below; every GPU that loads the library holds it until the
-// process exits.  It holds the packed FP64 links (1152 B per half-lattice
-// site) and up to three packed FP64 half fields (192 B per site each), so
-// lattices with V/2 up to about 19,000 sites fit (8^4, 12^4, 12^3 x 22, ...).
-// Larger lattices are rejected with WILSON_ERR_ARG before anything runs.
+// process exits.  Its size sets the largest lattice: packed FP64 links (1152 B per
+// half-lattice site) and three packed FP64 half fields (192 B per site each) have to
+// fit, V/2 up to about 19,000 sites (8^4, 12^4, 12^3 x 22, ...).
+// Larger lattices are rejected with WILSON_ERR_ARG before anything runs.  (The
+// kernel of these sizes reads canonical links and fields as they are; only the Schur
+// operator's intermediate field lies in the array.)
 //
 // Host code cannot use the array's name as a device address: in host code
 // the name denotes a host-side stand-in.  The first call in each CUDA
@@ -23,10 +24,8 @@
 // with cudaGetSymbolAddress and caches it under the context's unique ID, so
 // a context torn down and created again (cudaDeviceReset) resolves it anew.
 //
-// No tuning, no synchronisation.  The call never times launch
-// configurations: it takes the one an earlier wilson_dslash_eo call on the
-// same lattice chose (or the WILSON_TUNE_CACHE file holds), else a fixed
-// default.  It neither allocates nor synchronises.
+// No tuning, no synchronisation.  The call neither times launch configurations nor
+// allocates nor synchronises.
 //
 // Sharing.  All calls on a device use the same array, and it keeps whatever
 // the previous call left there.  Nothing here needs it cleared: every byte a
@@ -135,66 +134,8 @@ extern "C" int wilson_dslash_eo_noalloc(double* out, const double* gauge, const 
         WL_REQUIRE(is_device_ptr(out) && is_device_ptr(in) && is_device_ptr(gauge),
                    "wilson_dslash_eo_noalloc takes device pointers");
         char* base = static_cast<char*>(scratch_address());
-        cudaStream_t st = static_cast<cudaStream_t>(stream);
-
-        const int pin = op == WILSON_OP_HOP ? 1 - out_parity : out_parity;
-        GaugeField gf;
-        SpinorField a, b, t;
-        BorrowGuard guard;  // the views never free the array
-        gf.prec = P_F64;
-        gf.recon = 18;
-        gf.g = g;
-        guard.borrow(gf.buf, base, gbytes);
-        auto view = [&](SpinorField& f, int subset, size_t off) {
-            f.prec = P_F64;
-            f.subset = subset;
-            f.nrhs = 1;
-            f.g = g;
-            f.pbytes = (long long)pbytes;
-            guard.borrow(f.buf, base + off, pbytes);
-        };
-        view(a, pin, gbytes);
-        view(b, out_parity, gbytes + pbytes);
-        view(t, 1 - out_parity, gbytes + 2 * pbytes);
-
-        pack_gauge(gf, gauge, st);
-        pack_spinor(a, 0, in, st);
-        if (op == WILSON_OP_HOP) {
-            HopLaunch h{};
-            h.out = b.block(out_parity);
-            h.in = a.block(pin);
-            h.gauge = &gf;
-            h.sprec = P_F64;
-            h.no_tune = 1;
-            h.out_parity = out_parity;
-            h.a = 1.0;
-            launch_hop(h, st);
-        } else {
-            const int dag = op == WILSON_OP_SCHUR_DAG;
-            HopLaunch h1{};
-            h1.out = t.block(1 - out_parity);
-            h1.in = a.block(pin);
-            h1.gauge = &gf;
-            h1.sprec = P_F64;
-            h1.no_tune = 1;
-            h1.out_parity = 1 - out_parity;
-            h1.dagger = dag;
-            h1.a = 1.0;
-            launch_hop(h1, st);
-            HopLaunch h2{};
-            h2.out = b.block(out_parity);
-            h2.in = t.block(1 - out_parity);
-            h2.x = a.block(pin);
-            h2.xpay = 1;
-            h2.a = -kappa * kappa;
-            h2.gauge = &gf;
-            h2.sprec = P_F64;
-            h2.no_tune = 1;
-            h2.out_parity = out_parity;
-            h2.dagger = dag;
-            launch_hop(h2, st);
-        }
-        unpack_spinor(b, 0, out, st);
+        stateless_op(out, gauge, in, g, out_parity, kappa, op, static_cast<cudaStream_t>(stream), base,
+                     WILSON_NOALLOC_SCRATCH_BYTES);
         record_error("");
         return WILSON_OK;
     } catch (const Error& e) {

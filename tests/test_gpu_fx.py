@@ -93,3 +93,25 @@ def test_out_of_range(w, monkeypatch, dims, case):
                 assert np.all(a == 0)
             else:
                 assert np.max(np.abs(a[f] - b[f])) <= TOL * np.max(np.abs(b[f]))
+
+
+@pytest.mark.parametrize("dims", [(4, 4, 4, 6), (14, 14, 12, 18)])
+def test_output_over_an_input(w, dims):
+    """An output that overlaps the links or part of the input is what it is in
+    memory of its own (the kernels read their inputs while they write)."""
+    import torch
+    L = w.lattice(dims, PHASES)
+    V = inputs.volume(dims)
+    U = torch.from_numpy(inputs.gauge_field(dims, "random", seed=409)).cuda()
+    src = torch.from_numpy(inputs.gaussian_spinor(V // 2, seed=410)).cuda()
+    want = torch.empty_like(src)
+    for op in (w.WILSON_OP_HOP, w.WILSON_OP_SCHUR):
+        w.wilson_dslash_eo(want, U, src, L, 0, 0.13, op)
+        links = U.clone()
+        out = links.reshape(-1)[: src.numel()].view_as(src)
+        w.wilson_dslash_eo(out, links, src, L, 0, 0.13, op)
+        assert torch.equal(out, want)
+        both = torch.cat([src.reshape(-1), torch.zeros(1200, dtype=src.dtype, device="cuda")])
+        out = both[1200:].view_as(src)
+        w.wilson_dslash_eo(out, U, both[: src.numel()].view_as(src), L, 0, 0.13, op)
+        assert torch.equal(out, want)
