@@ -570,7 +570,7 @@ int wilson_spinor_import(wilson_spinor* s, const double* canon, void* stream) {
         cudaStream_t st = static_cast<cudaStream_t>(stream);
         const size_t per = sizeof(double) * 24 * (size_t)s->g.Vh * (s->f.subset == 2 ? 2 : 1);
         if (is_device_ptr(canon)) {
-            for (int k = 0; k < s->f.nrhs; k++) pack_spinor(s->f, k, canon + (per / sizeof(double)) * k, st);
+            pack_spinor(s->f, 0, s->f.nrhs, canon, st);
             return;
         }
         AsyncStaging& as = async_staging();
@@ -582,8 +582,7 @@ int wilson_spinor_import(wilson_spinor* s, const double* canon, void* stream) {
             WL_CUDA(cudaMemcpyAsync(as.in.p, canon, bytes, cudaMemcpyHostToDevice, as.copy_in));
             WL_CUDA(cudaEventRecord(as.in_ready, as.copy_in));
             WL_CUDA(cudaStreamWaitEvent(st, as.in_ready, 0));
-            for (int k = 0; k < s->f.nrhs; k++)
-                pack_spinor(s->f, k, as.in.as<const double>() + (per / sizeof(double)) * k, st);
+            pack_spinor(s->f, 0, s->f.nrhs, as.in.as<const double>(), st);
             WL_CUDA(cudaEventRecord(as.in_free, st));
             return;
         }
@@ -593,8 +592,7 @@ int wilson_spinor_import(wilson_spinor* s, const double* canon, void* stream) {
             std::lock_guard<std::mutex> lk(sg.m);
             sg.buf.ensure(per * s->f.nrhs);
             WL_CUDA(cudaMemcpyAsync(sg.buf.p, canon, per * s->f.nrhs, cudaMemcpyHostToDevice, st));
-            for (int k = 0; k < s->f.nrhs; k++)
-                pack_spinor(s->f, k, sg.buf.as<const double>() + (per / sizeof(double)) * k, st);
+            pack_spinor(s->f, 0, s->f.nrhs, sg.buf.as<const double>(), st);
             // the staging buffer is reused by the next call: finish with it first
             WL_CUDA(cudaStreamSynchronize(st));
         }
@@ -608,7 +606,7 @@ int wilson_spinor_export(const wilson_spinor* s, double* canon, void* stream) {
         cudaStream_t st = static_cast<cudaStream_t>(stream);
         const size_t per = sizeof(double) * 24 * (size_t)s->g.Vh * (s->f.subset == 2 ? 2 : 1);
         if (is_device_ptr(canon)) {
-            for (int k = 0; k < s->f.nrhs; k++) unpack_spinor(s->f, k, canon + (per / sizeof(double)) * k, st);
+            unpack_spinor(s->f, 0, s->f.nrhs, canon, st);
             return;
         }
         AsyncStaging& as = async_staging();
@@ -623,8 +621,7 @@ int wilson_spinor_export(const wilson_spinor* s, double* canon, void* stream) {
                 ob.ensure(bytes);
             }
             WL_CUDA(cudaStreamWaitEvent(st, as.out_free[i], 0));  // its last copy-out is done
-            for (int k = 0; k < s->f.nrhs; k++)
-                unpack_spinor(s->f, k, ob.as<double>() + (per / sizeof(double)) * k, st);
+            unpack_spinor(s->f, 0, s->f.nrhs, ob.as<double>(), st);
             WL_CUDA(cudaEventRecord(as.out_ready, st));
             WL_CUDA(cudaStreamWaitEvent(as.copy_out, as.out_ready, 0));
             WL_CUDA(cudaMemcpyAsync(canon, ob.p, bytes, cudaMemcpyDeviceToHost, as.copy_out));
@@ -637,8 +634,7 @@ int wilson_spinor_export(const wilson_spinor* s, double* canon, void* stream) {
             Staging& sg = staging();
             std::lock_guard<std::mutex> lk(sg.m);
             sg.buf.ensure(per * s->f.nrhs);
-            for (int k = 0; k < s->f.nrhs; k++)
-                unpack_spinor(s->f, k, sg.buf.as<double>() + (per / sizeof(double)) * k, st);
+            unpack_spinor(s->f, 0, s->f.nrhs, sg.buf.as<double>(), st);
             WL_CUDA(cudaMemcpyAsync(canon, sg.buf.p, per * s->f.nrhs, cudaMemcpyDeviceToHost, st));
             WL_CUDA(cudaStreamSynchronize(st));
         }

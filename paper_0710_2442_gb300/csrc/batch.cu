@@ -403,8 +403,8 @@ void build_problem(HostProb& P, const wilson_problem& in, Prec ip, const SolvePa
         P.f[BF_T32].alloc(P_F32, 1, 1, P.g);
         WL_CUDA(cudaMemsetAsync(P.f[BF_X32].buf.p, 0, P.f[BF_X32].buf.bytes, st));  // read by tuning launches
     }
-    pack_spinor(P.f[BF_B], 0, in.b, st);
-    if (prm.use_initial_guess) pack_spinor(P.f[BF_X], 0, in.x, st);
+    pack_spinor(P.f[BF_B], 0, 1, in.b, st);
+    if (prm.use_initial_guess) pack_spinor(P.f[BF_X], 0, 1, in.x, st);
 }
 
 // Device descriptors, states and the tile table of one run.
@@ -889,7 +889,7 @@ void batch_solve(int n, const wilson_problem* probs, const SolveParams& prm, wil
         WL_CUDA(cudaMemcpy(hs.data(), R.state.p, sizeof(BatchState) * R.nprob, cudaMemcpyDeviceToHost));
         for (int j = 0; j < R.nprob; j++) {
             const int i = R.members[j];
-            unpack_spinor(hp[i].f[BF_X], 0, probs[i].x, st);
+            unpack_spinor(hp[i].f[BF_X], 0, 1, probs[i].x, st);
             const BatchState& S = hs[j];
             wilson_solve_stats& o = stats[i];
             const double bn = std::sqrt(S.bnorm2);

@@ -240,8 +240,9 @@ bool fx_site_kernel(const Geom& g, int nrhs, int full);
 int hop_grid_blocks(const Geom& g, int block, int grid_cap);
 
 // canonical <-> SoA
-void pack_spinor(const SpinorField& f, int rhs, const double* canon, cudaStream_t st);
-void unpack_spinor(const SpinorField& f, int rhs, double* canon, cudaStream_t st);
+// n_rhs right-hand sides from rhs on, canonical fields back to back
+void pack_spinor(const SpinorField& f, int rhs, int n_rhs, const double* canon, cudaStream_t st);
+void unpack_spinor(const SpinorField& f, int rhs, int n_rhs, double* canon, cudaStream_t st);
 void pack_gauge(GaugeField& gf, const double* canon, cudaStream_t st);
 
 int device_sm_count();

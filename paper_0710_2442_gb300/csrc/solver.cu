@@ -581,13 +581,10 @@ std::vector<SolveStats> cg_solve(double* xc, const double* gauge_canon, const do
     SpinorField b, x;
     b.alloc(P_F64, 2, nrhs, g);
     x.alloc(P_F64, 2, nrhs, g);
-    const size_t per = (size_t)24 * 2 * g.Vh;  // doubles per canonical full field
-    for (int k = 0; k < nrhs; k++) {
-        pack_spinor(b, k, bc + per * k, st);
-        if (prm.use_initial_guess) pack_spinor(x, k, xc + per * k, st);
-    }
+    pack_spinor(b, 0, nrhs, bc, st);
+    if (prm.use_initial_guess) pack_spinor(x, 0, nrhs, xc, st);
     std::vector<SolveStats> stats = cg_solve_prepared(x, b, g64, *inner_gauge, kappa, prm, st, g32);
-    for (int k = 0; k < nrhs; k++) unpack_spinor(x, k, xc + per * k, st);
+    unpack_spinor(x, 0, nrhs, xc, st);
     WL_CUDA(cudaStreamSynchronize(st));
     return stats;
 }
