@@ -138,15 +138,38 @@ def _ptr(t) -> int:
     return t.data_ptr()  # torch tensor
 
 
+_torch_cuda = None  # (is_initialized, current device, current raw stream of a device) of torch
+
+
+def _current_stream() -> int:
+    """torch's current stream on the current device (0 without torch or CUDA).
+
+    By torch's own accessors for the two integers: building the Stream object
+    that torch.cuda.current_stream returns costs 2.9 us a call and asking
+    whether CUDA is there 0.8 us, of the 9 us that a small operator call
+    took on the host."""
+    global _torch_cuda
+    try:
+        if _torch_cuda is None:
+            import torch
+            _torch_cuda = (torch.cuda.is_initialized, torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream)
+        initialized, device, raw_stream = _torch_cuda
+        if initialized():
+            return raw_stream(device())
+    except Exception:
+        pass
+    try:
+        import torch
+        if torch.cuda.is_available():
+            return torch.cuda.current_stream().cuda_stream
+    except Exception:
+        pass
+    return 0
+
+
 def _stream(stream) -> int:
     if stream is None:
-        try:
-            import torch
-            if torch.cuda.is_available():
-                return torch.cuda.current_stream().cuda_stream
-        except Exception:
-            pass
-        return 0
+        return _current_stream()
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream

@@ -40,3 +40,12 @@ def test_multi_rhs_round_trip(w, dims, prec, subset):
     else:  # one rounding of a value below its site's largest component
         top = np.abs(src.view(np.float64)).reshape(3, n, -1).max(axis=2)[..., None, None]
         assert np.max(np.abs((got - src).view(np.float64).reshape(3, n, 4, 6)) / top) <= (2.0 ** -11 if prec == "f16" else 2.0 ** -8)
+
+
+def test_default_stream_is_torchs_current_one(w):
+    import torch
+    side = torch.cuda.Stream()
+    assert w._stream(None) == torch.cuda.current_stream().cuda_stream
+    with torch.cuda.stream(side):
+        assert w._stream(None) == side.cuda_stream == w._stream(side)
+    assert w._stream(None) == torch.cuda.current_stream().cuda_stream
