@@ -92,6 +92,7 @@ struct Geom {
     int Vh;            // sites per parity
     int stride;        // SoA row length (chunks) of a parity-field row, >= Vh
     double ph[4][2];   // boundary phases (re, im)
+    float pf[4][2];    // the same rounded to FP32 (a conversion from FP64 takes the FP64 pipe 64 cycles)
     unsigned int dm[3];  // division by Lx, Ly, Lz: n / L = umulhi(n, dm) >> ds, exact for n < 2^31
     int ds[3];
 };
@@ -125,6 +126,13 @@ __device__ __forceinline__ void site_of_half(int h, int p, const Geom& g, int c[
     int odd = (c[1] + c[2] + c[3] + p) & 1;
     c[0] = x0 + odd;
     s = s0 + odd;
+}
+
+// Boundary phase component z of direction mu in the arithmetic's type.
+template <class T>
+__device__ __forceinline__ T phase_of(const Geom& g, int mu, int z) {
+    if constexpr (sizeof(T) == 4) return g.pf[mu][z];
+    else return g.ph[mu][z];
 }
 
 // Read-only loads go through the non-coherent path (__ldg) by default.  A

@@ -82,6 +82,8 @@ void launch_hop(const HopLaunch& L, cudaStream_t st) {
     P.full = L.full;
     P.xpay = L.xpay;
     P.a = L.a;
+    P.af = (float)L.a;
+    P.scaled = L.a != 1.0;
     P.reduce = 0;
     P.red = RedArgs{};
     P.skip = L.skip;

@@ -168,7 +168,7 @@ __global__ void __launch_bounds__(256, 2) dd_hop_kernel(const HopParams P, const
             if (c[3] == Lt - 1) {
                 HaloFmt<SP>::load(A.recv_next, A.fst, h - (Lt - 1) * A.nface, hs);
                 if (A.last) {
-                    const cpx<T> eta = {(T)g.ph[3][0], (T)g.ph[3][1]};
+                    const cpx<T> eta = {phase_of<T>(g, 3, 0), phase_of<T>(g, 3, 1)};
 #pragma unroll
                     for (int k = 0; k < 6; k++) hs[k] = cmul(eta, hs[k]);
                 }
@@ -187,7 +187,7 @@ __global__ void __launch_bounds__(256, 2) dd_hop_kernel(const HopParams P, const
             if (c[3] == 0) {
                 HaloFmt<SP>::load(A.recv_prev, A.fst, h, w);
                 if (A.first) {
-                    const cpx<T> eta = {(T)g.ph[3][0], -(T)g.ph[3][1]};
+                    const cpx<T> eta = {phase_of<T>(g, 3, 0), -phase_of<T>(g, 3, 1)};
 #pragma unroll
                     for (int k = 0; k < 6; k++) w[k] = cmul(eta, w[k]);
                 }

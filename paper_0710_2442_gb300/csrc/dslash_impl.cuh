@@ -157,6 +157,8 @@ struct HopParams {
     int full;
     int xpay;
     double a;
+    float af;    // a in FP32
+    int scaled;  // a != 1
     RedArgs red;
     int reduce;
     const int* skip;
@@ -183,7 +185,7 @@ __device__ __forceinline__ void hop_dir(cpx<typename SpinorFmt<SP>::real> acc[12
         GF::load(P.gauge, g.stride, p * 4 + MU, h, U);
         project<MU, SF_>(v, hs);
         if (wrap) {
-            const cpx<T> eta = {(T)g.ph[MU][0], (T)g.ph[MU][1]};
+            const cpx<T> eta = {phase_of<T>(g, MU, 0), phase_of<T>(g, MU, 1)};
 #pragma unroll
             for (int k = 0; k < 6; k++) hs[k] = cmul(eta, hs[k]);
         }
@@ -201,7 +203,7 @@ __device__ __forceinline__ void hop_dir(cpx<typename SpinorFmt<SP>::real> acc[12
         GF::load(P.gauge, g.stride, (1 - p) * 4 + MU, hn, U);
         project<MU, -SF_>(v, hs);
         if (wrap) {
-            const cpx<T> eta = {(T)g.ph[MU][0], -(T)g.ph[MU][1]};
+            const cpx<T> eta = {phase_of<T>(g, MU, 0), -phase_of<T>(g, MU, 1)};
 #pragma unroll
             for (int k = 0; k < 6; k++) hs[k] = cmul(eta, hs[k]);
         }
@@ -257,7 +259,9 @@ __global__ void __launch_bounds__(256, MINB) hop_kernel(const HopParams P) {
     const char* in = P.in + (P.full ? pin * P.in_pstep : 0) + k * P.in_rstep;
     const char* x = P.x ? P.x + (P.full ? p * P.x_pstep : 0) + k * P.x_rstep : nullptr;
     const Geom& g = P.g;
-    const T a = (T)P.a;
+    T a;
+    if constexpr (sizeof(T) == 4) a = P.af;
+    else a = P.a;
     double nrm = 0.0;
     // The whole block iterates while its tile starts inside the lattice (a
     // block-uniform trip count); this form compiles to faster code than the
@@ -280,7 +284,7 @@ __global__ void __launch_bounds__(256, MINB) hop_kernel(const HopParams P) {
                 acc[k].re = fma(a, acc[k].re, xv[k].re);
                 acc[k].im = fma(a, acc[k].im, xv[k].im);
             }
-        } else if (P.a != 1.0) {
+        } else if (P.scaled) {
 #pragma unroll
             for (int k = 0; k < 12; k++) acc[k] = cscale(a, acc[k]);
         }
@@ -454,7 +458,7 @@ __device__ __forceinline__ void hop_dir_p(PSpinor& acc, const HopParams& P, cons
         GF::load(P.gauge, g.stride, p * 4 + MU, h, U);
         project_p<MU, SF_>(q, hh);
         if (wrap) {
-            const float er = (float)g.ph[MU][0], ei = (float)g.ph[MU][1];
+            const float er = g.pf[MU][0], ei = g.pf[MU][1];
 #pragma unroll
             for (int k = 0; k < 3; k++) {
                 const float2 r = hh.re[k], m = hh.im[k];
@@ -477,7 +481,7 @@ __device__ __forceinline__ void hop_dir_p(PSpinor& acc, const HopParams& P, cons
         GF::load(P.gauge, g.stride, (1 - p) * 4 + MU, hn, U);
         project_p<MU, -SF_>(q, hh);
         if (wrap) {
-            const float er = (float)g.ph[MU][0], ei = -(float)g.ph[MU][1];
+            const float er = g.pf[MU][0], ei = -g.pf[MU][1];
 #pragma unroll
             for (int k = 0; k < 3; k++) {
                 const float2 r = hh.re[k], m = hh.im[k];
@@ -504,7 +508,7 @@ __global__ void __launch_bounds__(256, MINB) hop_kernel_p(const HopParams P) {
     const char* in = P.in + (P.full ? pin * P.in_pstep : 0) + k * P.in_rstep;
     const char* x = P.x ? P.x + (P.full ? p * P.x_pstep : 0) + k * P.x_rstep : nullptr;
     const Geom& g = P.g;
-    const float a = (float)P.a;
+    const float a = P.af;
     double nrm = 0.0;
     for (int h = sb * blockDim.x + threadIdx.x; h - (int)threadIdx.x < g.Vh; h += nb * blockDim.x) {
         if (h >= g.Vh) continue;
@@ -528,7 +532,7 @@ __global__ void __launch_bounds__(256, MINB) hop_kernel_p(const HopParams P) {
                 acc.re23[cc] = fma2(A, acc.re23[cc], mul2(X, xq.re23[cc]));
                 acc.im23[cc] = fma2(A, acc.im23[cc], mul2(X, xq.im23[cc]));
             }
-        } else if (P.a != 1.0) {
+        } else if (P.scaled) {
             const float2 A = bc2(a);
 #pragma unroll
             for (int cc = 0; cc < 3; cc++) {
@@ -615,7 +619,7 @@ __device__ __forceinline__ void hop_dir_pm(PSpinor (&acc)[NB], const HopParams& 
             PHalf hh, w;
             float sc;
             load_project<SP, MU, SF_, HP>(in + r * P.in_rstep, g.stride, hn, hh, sc);
-            if (wrap) apply_phase_p(hh, (float)g.ph[MU][0], (float)g.ph[MU][1]);
+            if (wrap) apply_phase_p(hh, g.pf[MU][0], g.pf[MU][1]);
             su3_mul_p<false>(U, hh, w);
             expand_p<MU, SF_, FIRST>(acc[r], w, sc);
         }
@@ -630,7 +634,7 @@ __device__ __forceinline__ void hop_dir_pm(PSpinor (&acc)[NB], const HopParams& 
             PHalf hh, w;
             float sc;
             load_project<SP, MU, -SF_, HP>(in + r * P.in_rstep, g.stride, hn, hh, sc);
-            if (wrap) apply_phase_p(hh, (float)g.ph[MU][0], -(float)g.ph[MU][1]);
+            if (wrap) apply_phase_p(hh, g.pf[MU][0], -g.pf[MU][1]);
             su3_mul_p<true>(U, hh, w);
             expand_p<MU, -SF_, false>(acc[r], w, sc);
         }
@@ -657,7 +661,7 @@ __global__ void __launch_bounds__(256, MINB) hop_kernel_pm(const HopParams P) {
     const char* in = P.in + (P.full ? pin * P.in_pstep : 0) + k0 * P.in_rstep;
     const char* x = P.x ? P.x + (P.full ? p * P.x_pstep : 0) + k0 * P.x_rstep : nullptr;
     const Geom& g = P.g;
-    const float a = (float)P.a;
+    const float a = P.af;
     double nrm[NB];
 #pragma unroll
     for (int r = 0; r < NB; r++) nrm[r] = 0.0;
@@ -685,7 +689,7 @@ __global__ void __launch_bounds__(256, MINB) hop_kernel_pm(const HopParams P) {
                     A.re23[cc] = fma2(Af, A.re23[cc], mul2(X, xq.re23[cc]));
                     A.im23[cc] = fma2(Af, A.im23[cc], mul2(X, xq.im23[cc]));
                 }
-            } else if (P.a != 1.0) {
+            } else if (P.scaled) {
                 const float2 Af = bc2(a);
 #pragma unroll
                 for (int cc = 0; cc < 3; cc++) {
@@ -736,7 +740,7 @@ __device__ __forceinline__ void hop_dir_rl(PSpinor& acc, const HopParams& P, con
         SF::load_packed(in, g.stride, hn[2 * MU], q, sc);
         GF::decode(lsm + (2 * MU) * GF::nchunk * T, T, U);
         project_p<MU, SF_>(q, hh);
-        if (wrap >> (2 * MU) & 1u) apply_phase_p(hh, (float)g.ph[MU][0], (float)g.ph[MU][1]);
+        if (wrap >> (2 * MU) & 1u) apply_phase_p(hh, g.pf[MU][0], g.pf[MU][1]);
         su3_mul_p<false>(U, hh, w);
         expand_p<MU, SF_, FIRST>(acc, w, sc);
     }
@@ -748,7 +752,7 @@ __device__ __forceinline__ void hop_dir_rl(PSpinor& acc, const HopParams& P, con
         SF::load_packed(in, g.stride, hn[2 * MU + 1], q, sc);
         GF::decode(lsm + (2 * MU + 1) * GF::nchunk * T, T, U);
         project_p<MU, -SF_>(q, hh);
-        if (wrap >> (2 * MU + 1) & 1u) apply_phase_p(hh, (float)g.ph[MU][0], -(float)g.ph[MU][1]);
+        if (wrap >> (2 * MU + 1) & 1u) apply_phase_p(hh, g.pf[MU][0], -g.pf[MU][1]);
         su3_mul_p<true>(U, hh, w);
         expand_p<MU, -SF_, false>(acc, w, sc);
     }
@@ -778,7 +782,7 @@ __global__ void __launch_bounds__(256, MINB) hop_kernel_rl(const HopParams P) {
     const int p = P.full ? (int)blockIdx.y : P.out_parity;
     const int pin = 1 - p;
     const Geom& g = P.g;
-    const float a = (float)P.a;
+    const float a = P.af;
     for (int h = sb * T + t; h - t < g.Vh; h += nb * T) {
         if (h >= g.Vh) continue;
         int hn[8];
@@ -822,7 +826,7 @@ __global__ void __launch_bounds__(256, MINB) hop_kernel_rl(const HopParams P) {
                     A.re23[cc] = fma2(Af, A.re23[cc], mul2(X, xq.re23[cc]));
                     A.im23[cc] = fma2(Af, A.im23[cc], mul2(X, xq.im23[cc]));
                 }
-            } else if (P.a != 1.0) {
+            } else if (P.scaled) {
                 const float2 Af = bc2(a);
 #pragma unroll
                 for (int cc = 0; cc < 3; cc++) {
@@ -868,7 +872,7 @@ __device__ __forceinline__ void pipe_hop(PSpinor& acc, const uint4 (&d)[3], floa
         }
         project_p<MU, S>(q, hh);
     }
-    if (wrap >> J & 1u) apply_phase_p(hh, (float)g.ph[MU][0], FWD ? (float)g.ph[MU][1] : -(float)g.ph[MU][1]);
+    if (wrap >> J & 1u) apply_phase_p(hh, g.pf[MU][0], FWD ? g.pf[MU][1] : -g.pf[MU][1]);
     su3_mul_p<!FWD>(U, hh, w);
     expand_p<MU, S, J == 0>(acc, w, sc);
 }

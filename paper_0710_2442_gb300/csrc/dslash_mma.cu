@@ -240,7 +240,7 @@ __global__ void __launch_bounds__(256, MINB) hop_kernel_mma(const HopParams P) {
     const bool bvalid = g < 6 && t < 3;
     const int efwd = bvalid ? bi * 3 + t : 0, ebwd = bvalid ? t * 3 + bi : 0;
     const uint32_t bmask = bvalid ? 0xFFFFFFFFu : 0u;
-    const float a = (float)P.a;
+    const float a = P.af;
     const int ntiles = (geo.Vh + 31) >> 5;
 
     for (int tile = sb * nwarps + warp; tile < ntiles; tile += nb * nwarps) {
@@ -272,7 +272,7 @@ __global__ void __launch_bounds__(256, MINB) hop_kernel_mma(const HopParams P) {
                 cpx<float> U[3][3];
                 GF::load(P.gauge, stride, ((j & 1) ? pin : p) * 4 + mu, (j & 1) ? hnb[j] : h, U);
                 if (wrap >> j & 1u) {
-                    const cpx<float> eta = {(float)geo.ph[mu][0], (float)geo.ph[mu][1]};
+                    const cpx<float> eta = {geo.pf[mu][0], geo.pf[mu][1]};
 #pragma unroll
                     for (int e = 0; e < 9; e++) U[e / 3][e % 3] = cmul(eta, U[e / 3][e % 3]);
                 }

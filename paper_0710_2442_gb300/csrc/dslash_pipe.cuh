@@ -52,7 +52,7 @@ __global__ void __launch_bounds__(TB) __maxnreg__(NREG) hop_kernel_pipe(const Ho
     const char* in = P.in + (P.full ? pin * P.in_pstep : 0) + k * P.in_rstep;
     const char* x = P.x ? P.x + (P.full ? p * P.x_pstep : 0) + k * P.x_rstep : nullptr;
     const Geom& g = P.g;
-    const float a = (float)P.a;
+    const float a = P.af;
     double nrm = 0.0;
     for (int h0 = sb * T + t; h0 - t < g.Vh; h0 += nb * T) {
         const bool ok = h0 < g.Vh;
@@ -72,7 +72,7 @@ __global__ void __launch_bounds__(TB) __maxnreg__(NREG) hop_kernel_pipe(const Ho
                 acc.re23[cc] = fma2(Af, acc.re23[cc], mul2(X, xq.re23[cc]));
                 acc.im23[cc] = fma2(Af, acc.im23[cc], mul2(X, xq.im23[cc]));
             }
-        } else if (P.a != 1.0) {
+        } else if (P.scaled) {
             const float2 Af = bc2(a);
 #pragma unroll
             for (int cc = 0; cc < 3; cc++) {
@@ -218,7 +218,7 @@ __global__ void __launch_bounds__(TB) __maxnreg__(NREG) hop_kernel_pipe2(const H
     const char* in = P.in + (P.full ? pin * P.in_pstep : 0) + k0 * P.in_rstep;
     const char* x = P.x ? P.x + (P.full ? p * P.x_pstep : 0) + k0 * P.x_rstep : nullptr;
     const Geom& g = P.g;
-    const float a = (float)P.a;
+    const float a = P.af;
     double nrm[2] = {0.0, 0.0};
     for (int h0 = sb * T + t; h0 - t < g.Vh; h0 += nb * T) {
         const bool ok = h0 < g.Vh;
@@ -241,7 +241,7 @@ __global__ void __launch_bounds__(TB) __maxnreg__(NREG) hop_kernel_pipe2(const H
                     A.re23[cc] = fma2(Af, A.re23[cc], mul2(X, xq.re23[cc]));
                     A.im23[cc] = fma2(Af, A.im23[cc], mul2(X, xq.im23[cc]));
                 }
-            } else if (P.a != 1.0) {
+            } else if (P.scaled) {
                 const float2 Af = bc2(a);
 #pragma unroll
                 for (int cc = 0; cc < 3; cc++) {

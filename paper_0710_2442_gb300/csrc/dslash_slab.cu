@@ -127,7 +127,7 @@ __device__ __forceinline__ void hop_t_staged(PSpinor& acc, const HopParams& P, c
         GF::load(P.gauge, g.stride, p * 4 + 3, h, U);
         project_p<3, SF_>(q, hh);
         if (c[3] == Lt - 1) {
-            const float er = (float)g.ph[3][0], ei = (float)g.ph[3][1];
+            const float er = g.pf[3][0], ei = g.pf[3][1];
 #pragma unroll
             for (int k = 0; k < 3; k++) {
                 const float2 r = hh.re[k], m = hh.im[k];
@@ -149,7 +149,7 @@ __device__ __forceinline__ void hop_t_staged(PSpinor& acc, const HopParams& P, c
         GF::load(P.gauge, g.stride, (1 - p) * 4 + 3, hn, U);
         project_p<3, -SF_>(q, hh);
         if (wrap) {
-            const float er = (float)g.ph[3][0], ei = -(float)g.ph[3][1];
+            const float er = g.pf[3][0], ei = -g.pf[3][1];
 #pragma unroll
             for (int k = 0; k < 3; k++) {
                 const float2 r = hh.re[k], m = hh.im[k];
@@ -215,7 +215,7 @@ __global__ void __launch_bounds__(256, 2) hop_kernel_slab(const HopParams P, int
     if (t == 0)
         for (int ts = t0 - 1; ts <= t0 + 2 && ts <= t0 + tt; ts++) issue(ts);
     const char* x = P.x;
-    const float a = (float)P.a;
+    const float a = P.af;
     for (int tc = t0; tc < t0 + tt; tc++) {
         const int rdown = tc - t0, rup = tc - t0 + 2;  // slot-relative indices of slices tc -+ 1
         const unsigned char* down = slab_smem + (size_t)(rdown & (kSlots - 1)) * slot_bytes;
@@ -244,7 +244,7 @@ __global__ void __launch_bounds__(256, 2) hop_kernel_slab(const HopParams P, int
                     acc.re23[cc] = fma2(A, acc.re23[cc], mul2(X, xq.re23[cc]));
                     acc.im23[cc] = fma2(A, acc.im23[cc], mul2(X, xq.im23[cc]));
                 }
-            } else if (P.a != 1.0) {
+            } else if (P.scaled) {
                 const float2 A = bc2(a);
 #pragma unroll
                 for (int cc = 0; cc < 3; cc++) {

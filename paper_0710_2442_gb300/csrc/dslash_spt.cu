@@ -57,7 +57,7 @@ __device__ __forceinline__ void hop_dir_ph(PSpinor& acc, const HopParams& P, con
         PHalf hh, w;
         if (fwd) project_f16_packed<MU, SF_>(d, hh);
         else project_f16_packed<MU, -SF_>(d, hh);
-        if (wrap) apply_phase_p(hh, (float)g.ph[MU][0], fwd ? (float)g.ph[MU][1] : -(float)g.ph[MU][1]);
+        if (wrap) apply_phase_p(hh, g.pf[MU][0], fwd ? g.pf[MU][1] : -g.pf[MU][1]);
         if (fwd) {
             su3_mul_p<false>(U, hh, w);
             expand_p<MU, SF_, FIRST>(acc, w, sc);
@@ -90,7 +90,7 @@ __global__ void __launch_bounds__(256, MINB) hop_kernel_ps(const HopParams P) {
     const char* x = P.x ? P.x + (P.full ? p * P.x_pstep : 0) + k * P.x_rstep : nullptr;
     const Geom& g = P.g;
     const int T = blockDim.x;
-    const float a = (float)P.a;
+    const float a = P.af;
     double nrm = 0.0;
     // block-uniform trip count: the block iterates while its first site is inside
     for (int h0 = sb * T * SPT + threadIdx.x; h0 - (int)threadIdx.x < g.Vh; h0 += nb * T * SPT) {
@@ -129,7 +129,7 @@ __global__ void __launch_bounds__(256, MINB) hop_kernel_ps(const HopParams P) {
                     A.re23[cc] = fma2(Af, A.re23[cc], mul2(X, xq.re23[cc]));
                     A.im23[cc] = fma2(Af, A.im23[cc], mul2(X, xq.im23[cc]));
                 }
-            } else if (P.a != 1.0) {
+            } else if (P.scaled) {
                 const float2 Af = bc2(a);
 #pragma unroll
                 for (int cc = 0; cc < 3; cc++) {

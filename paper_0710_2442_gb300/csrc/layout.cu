@@ -20,8 +20,10 @@ Geom make_geom(const int dims[4], const double ph[4][2]) {
     for (int mu = 0; mu < 4; mu++) {
         g.L[mu] = dims[mu];
         V *= dims[mu];
-        g.ph[mu][0] = ph[mu][0];
-        g.ph[mu][1] = ph[mu][1];
+        for (int z = 0; z < 2; z++) {
+            g.ph[mu][z] = ph[mu][z];
+            g.pf[mu][z] = (float)ph[mu][z];
+        }
     }
     g.Vh = (int)(V / 2);
     g.stride = round_up(g.Vh, 64);
