@@ -417,6 +417,7 @@ int wilson_cg_solve(double* x, const double* gauge, const double* b, const wilso
         SolveStream& ss = solve_stream();
         WL_CUDA(cudaEventRecord(ss.e0, caller));
         WL_CUDA(cudaStreamWaitEvent(ss.s, ss.e0, 0));
+        WorkspaceScope ws(ss.s);
         stats = cg_solve(x, gauge, b, 1, g, kappa, prm, ss.s)[0];
         WL_CUDA(cudaEventRecord(ss.e1, ss.s));
         WL_CUDA(cudaStreamWaitEvent(caller, ss.e1, 0));
@@ -448,6 +449,7 @@ int wilson_cg_solve_multi(double* x, const double* gauge, const double* b, int n
         SolveStream& ss = solve_stream();
         WL_CUDA(cudaEventRecord(ss.e0, caller));
         WL_CUDA(cudaStreamWaitEvent(ss.s, ss.e0, 0));
+        WorkspaceScope ws(ss.s);
         stats = cg_solve(x, gauge, b, nrhs, g, kappa, prm, ss.s);
         WL_CUDA(cudaEventRecord(ss.e1, ss.s));
         WL_CUDA(cudaStreamWaitEvent(caller, ss.e1, 0));
@@ -493,6 +495,7 @@ int wilson_batch_solve(int n, const wilson_problem* probs, const wilson_solver_p
         SolveStream& ss = solve_stream();
         WL_CUDA(cudaEventRecord(ss.e0, caller));
         WL_CUDA(cudaStreamWaitEvent(ss.s, ss.e0, 0));
+        WorkspaceScope ws(ss.s);
         batch_solve(n, probs, prm, st_out, info, ss.s);
         WL_CUDA(cudaEventRecord(ss.e1, ss.s));
         WL_CUDA(cudaStreamWaitEvent(caller, ss.e1, 0));

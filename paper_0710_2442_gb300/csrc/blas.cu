@@ -74,8 +74,14 @@ __global__ void __launch_bounds__(256) cg_xs_kernel(Vec x, Vec p, Vec s, Vec q, 
 
 // p = r + beta p
 template <int PP>
-__global__ void __launch_bounds__(256) cg_p_kernel(Vec p, Vec rv, Geom g, int nrhs, const CGScalars* sc) {
+__global__ void __launch_bounds__(256) cg_p_kernel(Vec p, Vec rv, Geom g, int nrhs, const CGScalars* sc,
+                                                   LoopHandle loop) {
     const RhsIdx r = rhs_index(nrhs);
+    if (loop.on && blockIdx.x == 0 && threadIdx.x == 0) {
+        unsigned go = 0;
+        for (int k = 0; k < nrhs; k++) go |= __ldcg(&sc[k].done) == 0;
+        cudaGraphSetConditional(loop.handle, go);
+    }
     if (__ldcg(&sc[r.k].done)) return;
     using T = typename SpinorFmt<PP>::real;
     const T beta = (T)__ldcg(&sc[r.k].beta);
@@ -191,13 +197,14 @@ void cg_xs_update(Prec xp, Prec pp, Vec x, Vec p, Vec s, Vec q, Vec s_low, const
     WL_LAUNCH_CHECK();
 }
 
-void cg_p_update(Prec pp, Vec p, Vec r, const Geom& g, int nrhs, const CGScalars* sc, cudaStream_t st) {
+void cg_p_update(Prec pp, Vec p, Vec r, const Geom& g, int nrhs, const CGScalars* sc, cudaStream_t st,
+                 const LoopHandle& loop) {
     const int block = 256, grid = blas_grid(g.Vh, block, 64 * device_sm_count()) * nrhs;
     switch (pp) {
-        case P_F64: cg_p_kernel<P_F64><<<grid, block, 0, st>>>(p, r, g, nrhs, sc); break;
-        case P_F32: cg_p_kernel<P_F32><<<grid, block, 0, st>>>(p, r, g, nrhs, sc); break;
-        case P_F16: cg_p_kernel<P_F16><<<grid, block, 0, st>>>(p, r, g, nrhs, sc); break;
-        case P_BF16: cg_p_kernel<P_BF16><<<grid, block, 0, st>>>(p, r, g, nrhs, sc); break;
+        case P_F64: cg_p_kernel<P_F64><<<grid, block, 0, st>>>(p, r, g, nrhs, sc, loop); break;
+        case P_F32: cg_p_kernel<P_F32><<<grid, block, 0, st>>>(p, r, g, nrhs, sc, loop); break;
+        case P_F16: cg_p_kernel<P_F16><<<grid, block, 0, st>>>(p, r, g, nrhs, sc, loop); break;
+        case P_BF16: cg_p_kernel<P_BF16><<<grid, block, 0, st>>>(p, r, g, nrhs, sc, loop); break;
     }
     WL_LAUNCH_CHECK();
 }

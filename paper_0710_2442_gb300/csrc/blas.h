@@ -21,8 +21,15 @@ inline Vec vec(const SpinorField& f, int parity) { return Vec{f.block(parity), f
 void cg_xs_update(Prec xp, Prec pp, Vec x, Vec p, Vec s, Vec q, Vec s_low, const Geom& g, int nrhs,
                   const CGScalars* sc, const RedArgs& red, int grid_cap, cudaStream_t st);
 
-// p = r + beta p (beta read from sc[k]).
-void cg_p_update(Prec pp, Vec p, Vec r, const Geom& g, int nrhs, const CGScalars* sc, cudaStream_t st);
+// The condition of a device-side loop around the iterations (on = 0: none).
+struct LoopHandle {
+    cudaGraphConditionalHandle handle{};
+    int on = 0;
+};
+// p = r + beta p (beta read from sc[k]); sets the loop's condition: go on while
+// some right-hand side is not done.
+void cg_p_update(Prec pp, Vec p, Vec r, const Geom& g, int nrhs, const CGScalars* sc, cudaStream_t st,
+                 const LoopHandle& loop);
 
 // y += a x
 void axpy(Prec yp, Vec y, Prec xp, Vec x, double a, const Geom& g, int nrhs, cudaStream_t st);

@@ -115,11 +115,27 @@ void schur_tune(const GaugeField& gf, Prec sp, Vec out, Vec in, Vec tmp, int nrh
 
 namespace {
 
+// The thread's page-locked buffer for read-backs, grown as needed (64 right-hand
+// sides take 9 KB); one solve at a time uses it.
 struct Pinned {
     void* p = nullptr;
-    explicit Pinned(size_t n) { WL_CUDA(cudaMallocHost(&p, n)); }
+    size_t bytes = 0;
+    void* ensure(size_t n) {
+        if (n > bytes) {
+            if (p) cudaFreeHost(p);
+            p = nullptr;
+            bytes = 0;
+            WL_CUDA(cudaMallocHost(&p, n));
+            bytes = n;
+        }
+        return p;
+    }
     ~Pinned() { if (p) cudaFreeHost(p); }
 };
+Pinned& thread_pinned() {
+    static thread_local Pinned b;
+    return b;
+}
 
 struct Inner {
     Prec ip, xp;
@@ -161,8 +177,7 @@ std::vector<SolveStats> cg_solve_prepared(SpinorField& x, const SpinorField& b, 
     CGScalars* sc = scbuf.as<CGScalars>();
     DevBuf resbuf(sizeof(double) * 8 * nr);
     double* d_res = resbuf.as<double>();
-    Pinned hbuf(sizeof(CGScalars) * nr + sizeof(double) * 8 * nr);
-    CGScalars* h_sc = static_cast<CGScalars*>(hbuf.p);
+    CGScalars* h_sc = static_cast<CGScalars*>(thread_pinned().ensure((sizeof(CGScalars) + sizeof(double) * 8) * nr));
     double* h_res = reinterpret_cast<double*>(h_sc + nr);
     int hops = 0;
 
@@ -246,6 +261,7 @@ std::vector<SolveStats> cg_solve_prepared(SpinorField& x, const SpinorField& b, 
     }
     schur_tune(g64, P_F64, vec(q64, 0), vec(x, 0), vec(t64, 1), nr, 0, nullptr, 0, st);
 
+    LoopHandle loop;
     auto iteration = [&](cudaStream_t s) {
         const int* skip = &sc->done;
         RedArgs ra = red.args(slot(2), FIN_CG_ALPHA, nullptr, sc);
@@ -257,13 +273,49 @@ std::vector<SolveStats> cg_solve_prepared(SpinorField& x, const SpinorField& b, 
         RedArgs rb = red.args(slot(4), FIN_CG_BETA, nullptr, sc);
         schur_apply(glo, in.ip, vec(in.r, 0), in.s_in(), vec(in.t, 1), nr, kappa, 1, &rb, skip, kSkipStride,
                     grid_cap, s);
-        cg_p_update(in.ip, vec(in.p, 0), vec(in.r, 0), g, nr, sc, s);
+        cg_p_update(in.ip, vec(in.p, 0), vec(in.r, 0), g, nr, sc, s, loop);
     };
 
+    // The iterations of a correction as one device-side while loop (a
+    // conditional graph node, whose condition the p update sets): no iterations
+    // launched after convergence, no host round trip per chunk, and six nodes to
+    // instantiate instead of 96.  16^3 x 32 F16, seven corrections of 27
+    // iterations: see DESIGN's table.
     cudaGraphExec_t gexec = nullptr;
     cudaGraph_t graph = nullptr;
     const int chunk = prm.chunk > 0 ? prm.chunk : 16;
-    if (prm.use_graph) {
+    bool loops = false;
+    if (prm.use_graph && !blk) {
+        WL_CUDA(cudaGraphCreate(&graph, 0));
+        cudaGraphNodeParams cp = {cudaGraphNodeTypeConditional};
+        cp.conditional.type = cudaGraphCondTypeWhile;
+        cp.conditional.size = 1;
+        cudaGraphNode_t cnode;
+        if (cudaGraphConditionalHandleCreate(&loop.handle, graph, 1, cudaGraphCondAssignDefault) == cudaSuccess) {
+            cp.conditional.handle = loop.handle;
+            loops = cudaGraphAddNode(&cnode, graph, nullptr, nullptr, 0, &cp) == cudaSuccess;
+        }
+        if (loops) {
+            loop.on = 1;
+            cudaGraph_t out = nullptr;
+            try {
+                WL_CUDA(cudaStreamBeginCaptureToGraph(st, cp.conditional.phGraph_out[0], nullptr, nullptr, 0,
+                                                      cudaStreamCaptureModeThreadLocal));
+                iteration(st);
+            } catch (...) {
+                cudaStreamEndCapture(st, &out);
+                cudaGraphDestroy(graph);
+                throw;
+            }
+            WL_CUDA(cudaStreamEndCapture(st, &out));
+            WL_CUDA(cudaGraphInstantiate(&gexec, graph, 0));
+        } else {  // no conditional nodes here: chunks of captured iterations
+            (void)cudaGetLastError();
+            cudaGraphDestroy(graph);
+            graph = nullptr;
+        }
+    }
+    if (prm.use_graph && !loops) {
         WL_CUDA(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
         try {
             for (int k = 0; k < chunk; k++) iteration(st);
@@ -425,7 +477,7 @@ std::vector<SolveStats> cg_solve_prepared(SpinorField& x, const SpinorField& b, 
                         st);
             hops += 2;
             if (restart) convert(in.ip, vec(in.p, 0), in.ip, vec(in.r, 0), g, nr, st);
-            else cg_p_update(in.ip, vec(in.p, 0), vec(in.r, 0), g, nr, sc, st);
+            else cg_p_update(in.ip, vec(in.p, 0), vec(in.r, 0), g, nr, sc, st, LoopHandle{});
             first = false;
 
             while (true) {
