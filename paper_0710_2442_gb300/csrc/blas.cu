@@ -14,6 +14,13 @@ int blas_grid(int Vh, int block, int cap) {
     return b < 1 ? 1 : b;
 }
 
+// The grid of a kernel whose blocks each sum partials first: as few blocks as the
+// cap's number of turns needs, all with the same number of turns.
+int even_grid(int Vh, int block, int cap) {
+    const int tiles = (Vh + block - 1) / block, turns = (tiles + cap - 1) / cap;
+    return (tiles + turns - 1) / turns;
+}
+
 struct RhsIdx {
     int k, sb, nb;
 };
@@ -28,21 +35,49 @@ __device__ __forceinline__ T* at(const Vec& v, int k) {
 
 }  // namespace
 
-// x += alpha p,  s -= alpha q,  [s_low = s],  reduce |s|^2 (FIN_CG_RES)
+// One CG iteration's scalars without a reducer's last block: the kernels that need
+// a sum add up its partials themselves, every block the same way.  A last
+// block's fence, ticket, second pass and division took 4.5 us of each of the three reducing kernels of an
+// iteration (16^3 x 32 F16: 51 us an iteration with them).  A kernel's blocks read
+// fields of the scalars that only another kernel writes: the x, s update reads gam and
+// iter, and leaves copies (gam2, iter2) that the p update reads when it writes
+// the new ones; done is written to what every block finds for itself.
+
+// x += alpha p,  s -= alpha q,  [s_low = s],  partials of |s|^2; alpha = gam / |q|^2 from
+// the nq partials of q.
 template <int XP, int PP, bool SLOW>
 __global__ void __launch_bounds__(256) cg_xs_kernel(Vec x, Vec p, Vec s, Vec q, Vec s_low, Geom g, int nrhs,
-                                                    const CGScalars* sc, RedArgs red) {
+                                                    CGScalars* sc, RedArgs qred, int nq, RedArgs red) {
     const RhsIdx r = rhs_index(nrhs);
-    if (__ldcg(&sc[r.k].done)) return;
+    CGScalars& C = sc[r.k];
+    if (__ldcg(&C.done)) return;
     using TX = typename SpinorFmt<XP>::real;
     using TP = typename SpinorFmt<PP>::real;
-    const TX alpha = (TX)__ldcg(&sc[r.k].alpha);
     char* X = at<char>(x, r.k);
     char* S = at<char>(s, r.k);
     const char* Pp = at<const char>(p, r.k);
     const char* Q = at<const char>(q, r.k);
     char* SL = SLOW ? at<char>(s_low, r.k) : nullptr;
     double nrm = 0.0;
+    __shared__ double s_alpha;
+    __shared__ int s_stop;
+    const double qq = sum_partials(qred, r.k, nq);
+    if (threadIdx.x == 0) {
+        const double gam = __ldcg(&C.gam);
+        const bool fine = qq > 0.0 && isfinite(qq);
+        s_stop = fine ? 0 : isfinite(qq) ? 1 : 3;  // Mhat p = 0: nothing left to do; NaN or Inf
+        s_alpha = fine ? gam / qq : 0.0;
+        if (r.sb == 0) {
+            C.pq = qq;
+            C.alpha = s_alpha;
+            C.gam2 = gam;
+            C.iter2 = __ldcg(&C.iter);
+            if (!fine) C.done = s_stop;
+        }
+    }
+    __syncthreads();
+    if (s_stop) return;
+    const TX alpha = (TX)s_alpha;
     for (int h = r.sb * blockDim.x + threadIdx.x; h < g.Vh; h += r.nb * blockDim.x) {
         cpx<TX> xv[12], sv[12];
         cpx<TP> pv[12], qv[12];
@@ -72,21 +107,81 @@ __global__ void __launch_bounds__(256) cg_xs_kernel(Vec x, Vec p, Vec s, Vec q, 
     grid_reduce(nrm, red, r.k, r.nb, r.sb);
 }
 
-// p = r + beta p
+// p = r + beta p (beta read from sc[k])
 template <int PP>
-__global__ void __launch_bounds__(256) cg_p_kernel(Vec p, Vec rv, Geom g, int nrhs, const CGScalars* sc,
-                                                   LoopHandle loop) {
+__global__ void __launch_bounds__(256) cg_p_kernel(Vec p, Vec rv, Geom g, int nrhs, const CGScalars* sc) {
     const RhsIdx r = rhs_index(nrhs);
-    if (loop.on && blockIdx.x == 0 && threadIdx.x == 0) {
-        unsigned go = 0;
-        for (int k = 0; k < nrhs; k++) go |= __ldcg(&sc[k].done) == 0;
-        cudaGraphSetConditional(loop.handle, go);
-    }
     if (__ldcg(&sc[r.k].done)) return;
     using T = typename SpinorFmt<PP>::real;
     const T beta = (T)__ldcg(&sc[r.k].beta);
     char* P = at<char>(p, r.k);
     const char* R = at<const char>(rv, r.k);
+    for (int h = r.sb * blockDim.x + threadIdx.x; h < g.Vh; h += r.nb * blockDim.x) {
+        cpx<T> pv[12], rr[12];
+        SpinorFmt<PP>::load(P, g.stride, h, pv);
+        SpinorFmt<PP>::load(R, g.stride, h, rr);
+#pragma unroll
+        for (int c = 0; c < 12; c++) {
+            pv[c].re = fma(beta, pv[c].re, rr[c].re);
+            pv[c].im = fma(beta, pv[c].im, rr[c].im);
+        }
+        SpinorFmt<PP>::store(P, g.stride, h, pv);
+    }
+}
+
+// The end of an iteration: the convergence test on |s|^2 and beta = |r|^2 / gam from
+// their partials, then p = r + beta p; sets the loop's condition.
+template <int PP>
+__global__ void __launch_bounds__(256) cg_p_end_kernel(Vec p, Vec rv, Geom g, int nrhs, CGScalars* sc, RedArgs sred, int ns,
+                                                       RedArgs rred, int nr, LoopHandle loop) {
+    const RhsIdx r = rhs_index(nrhs);
+    CGScalars& C = sc[r.k];
+    const bool first = r.sb == 0 && threadIdx.x == 0;
+    // Right-hand side 0's first block sets the condition: its own outcome, and for
+    // the others whether they went into this iteration (one that ends in it
+    // costs an empty iteration).
+    auto condition = [&](bool mine) {
+        if (!loop.on || !first || r.k != 0) return;
+        unsigned go = mine;
+        for (int k = 1; k < nrhs; k++) go |= __ldcg(&sc[k].done) == 0;
+        cudaGraphSetConditional(loop.handle, go);
+    };
+    if (__ldcg(&C.done)) {
+        condition(false);
+        return;
+    }
+    using T = typename SpinorFmt<PP>::real;
+    char* P = at<char>(p, r.k);
+    const char* R = at<const char>(rv, r.k);
+    __shared__ double s_beta;
+    __shared__ int s_done;
+    const double ss = sum_partials(sred, r.k, ns);
+    const double r2 = sum_partials(rred, r.k, nr);
+    if (threadIdx.x == 0) {
+        const int iter = __ldcg(&C.iter2) + 1;
+        int done = !isfinite(ss) ? 3 : ss <= __ldcg(&C.stop2) ? 1 : iter >= __ldcg(&C.maxiter) ? 2 : 0;
+        double beta = 0.0;
+        if (!done) {
+            const double gam = __ldcg(&C.gam2);
+            if (!isfinite(r2)) done = 3;
+            else if (gam > 0.0) beta = r2 / gam;
+            if (first) {
+                C.beta = beta;
+                if (done == 0) C.gam = r2;
+            }
+        }
+        if (first) {
+            C.snorm2 = ss;
+            C.iter = iter;
+            if (done) C.done = done;
+            condition(done == 0);
+        }
+        s_beta = beta;
+        s_done = done;
+    }
+    __syncthreads();
+    if (s_done) return;
+    const T beta = (T)s_beta;
     for (int h = r.sb * blockDim.x + threadIdx.x; h < g.Vh; h += r.nb * blockDim.x) {
         cpx<T> pv[12], rr[12];
         SpinorFmt<PP>::load(P, g.stride, h, pv);
@@ -181,30 +276,43 @@ __global__ void __launch_bounds__(256) convert_kernel(Vec dst, Vec src, Geom g, 
 }
 
 // ---------------------------------------------------------------------------
-void cg_xs_update(Prec xp, Prec pp, Vec x, Vec p, Vec s, Vec q, Vec s_low, const Geom& g, int nrhs,
-                  const CGScalars* sc, const RedArgs& red, int grid_cap, cudaStream_t st) {
-    const int block = 256, grid = blas_grid(g.Vh, block, grid_cap) * nrhs;
-    WL_REQUIRE(grid / nrhs <= red.slot_cap, "reduction capacity below the grid size");
+int cg_xs_update(Prec xp, Prec pp, Vec x, Vec p, Vec s, Vec q, Vec s_low, const Geom& g, int nrhs, CGScalars* sc,
+                 const RedArgs& qred, int nq, const RedArgs& red, int grid_cap, cudaStream_t st) {
+    const int block = 256, blocks = even_grid(g.Vh, block, grid_cap), grid = blocks * nrhs;
+    WL_REQUIRE(nq <= kMaxPartials && blocks <= kMaxPartials && blocks <= red.slot_cap, "reduction capacity below the grid size");
     if (xp == P_F64 && pp == P_F64)
-        cg_xs_kernel<P_F64, P_F64, false><<<grid, block, 0, st>>>(x, p, s, q, s_low, g, nrhs, sc, red);
+        cg_xs_kernel<P_F64, P_F64, false><<<grid, block, 0, st>>>(x, p, s, q, s_low, g, nrhs, sc, qred, nq, red);
     else if (xp == P_F32 && pp == P_F32)
-        cg_xs_kernel<P_F32, P_F32, false><<<grid, block, 0, st>>>(x, p, s, q, s_low, g, nrhs, sc, red);
+        cg_xs_kernel<P_F32, P_F32, false><<<grid, block, 0, st>>>(x, p, s, q, s_low, g, nrhs, sc, qred, nq, red);
     else if (xp == P_F32 && pp == P_F16)
-        cg_xs_kernel<P_F32, P_F16, true><<<grid, block, 0, st>>>(x, p, s, q, s_low, g, nrhs, sc, red);
+        cg_xs_kernel<P_F32, P_F16, true><<<grid, block, 0, st>>>(x, p, s, q, s_low, g, nrhs, sc, qred, nq, red);
     else if (xp == P_F32 && pp == P_BF16)
-        cg_xs_kernel<P_F32, P_BF16, true><<<grid, block, 0, st>>>(x, p, s, q, s_low, g, nrhs, sc, red);
+        cg_xs_kernel<P_F32, P_BF16, true><<<grid, block, 0, st>>>(x, p, s, q, s_low, g, nrhs, sc, qred, nq, red);
     else throw Error(7, "cg_xs_update: unsupported precision pair");
+    WL_LAUNCH_CHECK();
+    return blocks;
+}
+
+void cg_p_update(Prec pp, Vec p, Vec r, const Geom& g, int nrhs, const CGScalars* sc, cudaStream_t st) {
+    const int block = 256, grid = blas_grid(g.Vh, block, 64 * device_sm_count()) * nrhs;
+    switch (pp) {
+        case P_F64: cg_p_kernel<P_F64><<<grid, block, 0, st>>>(p, r, g, nrhs, sc); break;
+        case P_F32: cg_p_kernel<P_F32><<<grid, block, 0, st>>>(p, r, g, nrhs, sc); break;
+        case P_F16: cg_p_kernel<P_F16><<<grid, block, 0, st>>>(p, r, g, nrhs, sc); break;
+        case P_BF16: cg_p_kernel<P_BF16><<<grid, block, 0, st>>>(p, r, g, nrhs, sc); break;
+    }
     WL_LAUNCH_CHECK();
 }
 
-void cg_p_update(Prec pp, Vec p, Vec r, const Geom& g, int nrhs, const CGScalars* sc, cudaStream_t st,
-                 const LoopHandle& loop) {
-    const int block = 256, grid = blas_grid(g.Vh, block, 64 * device_sm_count()) * nrhs;
+void cg_p_end(Prec pp, Vec p, Vec r, const Geom& g, int nrhs, CGScalars* sc, const RedArgs& sred, int ns,
+              const RedArgs& rred, int nr, const LoopHandle& loop, int grid_cap, cudaStream_t st) {
+    const int block = 256, grid = even_grid(g.Vh, block, grid_cap) * nrhs;
+    WL_REQUIRE(ns <= kMaxPartials && nr <= kMaxPartials, "too many partials");
     switch (pp) {
-        case P_F64: cg_p_kernel<P_F64><<<grid, block, 0, st>>>(p, r, g, nrhs, sc, loop); break;
-        case P_F32: cg_p_kernel<P_F32><<<grid, block, 0, st>>>(p, r, g, nrhs, sc, loop); break;
-        case P_F16: cg_p_kernel<P_F16><<<grid, block, 0, st>>>(p, r, g, nrhs, sc, loop); break;
-        case P_BF16: cg_p_kernel<P_BF16><<<grid, block, 0, st>>>(p, r, g, nrhs, sc, loop); break;
+        case P_F64: cg_p_end_kernel<P_F64><<<grid, block, 0, st>>>(p, r, g, nrhs, sc, sred, ns, rred, nr, loop); break;
+        case P_F32: cg_p_end_kernel<P_F32><<<grid, block, 0, st>>>(p, r, g, nrhs, sc, sred, ns, rred, nr, loop); break;
+        case P_F16: cg_p_end_kernel<P_F16><<<grid, block, 0, st>>>(p, r, g, nrhs, sc, sred, ns, rred, nr, loop); break;
+        case P_BF16: cg_p_end_kernel<P_BF16><<<grid, block, 0, st>>>(p, r, g, nrhs, sc, sred, ns, rred, nr, loop); break;
     }
     WL_LAUNCH_CHECK();
 }

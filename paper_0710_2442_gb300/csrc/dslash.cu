@@ -58,12 +58,9 @@ bool fx_hops(const GaugeField& gf) {
     return !(forced && *forced && gf.buf.p);
 }
 
-void launch_hop(const HopLaunch& L, cudaStream_t st) {
+int launch_hop(const HopLaunch& L, cudaStream_t st) {
     const GaugeField& gf = *L.gauge;
-    if (L.sprec == P_F64 && fx_hops(gf)) {
-        if (!L.tune_only) launch_hop_fx(L, st);
-        return;
-    }
+    if (L.sprec == P_F64 && fx_hops(gf)) return L.tune_only ? 0 : launch_hop_fx(L, st);
     HopParams P;
     P.out = static_cast<char*>(L.out);
     P.in = static_cast<const char*>(L.in);
@@ -163,7 +160,7 @@ void launch_hop(const HopLaunch& L, cudaStream_t st) {
     WL_REQUIRE(hop_variant_valid(cfg.variant, sp, R, P.nrhs), "hop variant does not fit this launch");
     // a pinned variant without a fused reduction: the paired kernel, same block
     if (L.red && !reduces(cfg.variant)) cfg.variant = 3;
-    if (L.tune_only) return;
+    if (L.tune_only) return 0;
     if (L.red) {
         P.reduce = 1;
         P.red = *L.red;
@@ -173,6 +170,7 @@ void launch_hop(const HopLaunch& L, cudaStream_t st) {
     WL_REQUIRE(!L.red || site_blocks <= L.red->slot_cap, "reduction capacity below the grid size");
     dispatch(P, sp, gp, R, cfg.block, site_blocks, ny, dag, cfg.variant, st);
     WL_LAUNCH_CHECK();
+    return site_blocks;
 }
 
 }  // namespace wl

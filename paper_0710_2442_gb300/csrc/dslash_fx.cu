@@ -45,7 +45,7 @@ bool fx_site_kernel(const Geom& g, int nrhs, int full) {
     return (long long)g.Vh * std::max(nrhs, 1) * (full ? 2 : 1) >= kFxSiteMin;
 }
 
-void launch_hop_fx(const HopLaunch& L, cudaStream_t st) {
+int launch_hop_fx(const HopLaunch& L, cudaStream_t st) {
     const GaugeField& gf = *L.gauge;
     const Geom& g = gf.g;
     const int nrhs = L.nrhs > 1 ? L.nrhs : 1, ny = L.full ? 2 : 1;
@@ -93,7 +93,7 @@ void launch_hop_fx(const HopLaunch& L, cudaStream_t st) {
         } else {
             launch_split<true, false>(P, blocks, ny, st);
         }
-        return;
+        return blocks;
     }
     if (L.fx_in) {
         P.in = soa(L.fx_in, L.full ? L.fx_pstep : 0, L.fx_rstep, g.stride);
@@ -110,6 +110,7 @@ void launch_hop_fx(const HopLaunch& L, cudaStream_t st) {
     } else {
         launch_site<false, false>(P, blocks, ny, st);
     }
+    return blocks;
 }
 
 }  // namespace wl

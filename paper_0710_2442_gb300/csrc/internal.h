@@ -261,13 +261,13 @@ struct HopLaunch {
     int canon;             // bits kCanonIn, kCanonX, kCanonOut: that field is canonical (one rhs)
 };
 constexpr int kCanonIn = 1, kCanonX = 2, kCanonOut = 4;
-void launch_hop(const HopLaunch& L, cudaStream_t st);
+int launch_hop(const HopLaunch& L, cudaStream_t st);  // returns a reducing launch's blocks per rhs
 
 // FP64 hops on the integer pipe (dslash_fx.cu).  They run wherever the links
 // have a fixed-point form, unless WILSON_HOP_VARIANT pins the FP64 stencil and the
 // links are there as doubles.
 bool fx_hops(const GaugeField& gf);
-void launch_hop_fx(const HopLaunch& L, cudaStream_t st);
+int launch_hop_fx(const HopLaunch& L, cudaStream_t st);
 long long fx_spinor_bytes(int stride);  // one parity, one rhs
 // Whether the kernel on fixed-point fields is taken, given room for them: below
 // kFxSiteMin output sites the conversion costs more than it saves (12^4: 14 against 12.3 + 4.2 us

@@ -20,7 +20,8 @@ enum FinOp {
     FIN_CG_RES = 2,    // |s|^2: convergence test, iteration count
     FIN_CG_BETA = 3,   // |r|^2: beta = |r|^2 / gam, gam = |r|^2
     FIN_ADD = 4,       // result[0] += sum
-    FIN_CG_GAM = 5     // |r|^2: gam = |r|^2 (start of a CG)
+    FIN_CG_GAM = 5,    // |r|^2: gam = |r|^2 (start of a CG)
+    FIN_PARTIAL = 6    // the blocks' partials stay where they are: the next kernel sums them
 };
 
 // Scalars of one CG solve, kept on the device so that iterations never wait
@@ -35,7 +36,8 @@ struct CGScalars {
     int done;        // 1: converged (snorm2 <= stop2), 2: maxiter, 3: NaN/Inf, 4: finished earlier
     int iter;        // iterations completed since the counter was last reset
     int maxiter;     // iteration cap for this inner solve
-    int pad;
+    int iter2;       // iter and gam as the x, s update left them for the p update (blas.cu)
+    double gam2;
 };
 
 // A reduction may have several independent slots (one per right-hand side):
@@ -55,8 +57,8 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
-// Sum over the block; the value is valid in thread 0.
-__device__ __forceinline__ double block_sum(double v) {
+// Sum over the block by FP64 additions; valid in thread 0.
+inline __device__ __noinline__ double block_sum_fp64(double v) {
     __shared__ double sm[32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int nwarps = (blockDim.x + 31) >> 5;
@@ -69,6 +71,68 @@ __device__ __forceinline__ double block_sum(double v) {
         v = warp_sum(v);
     }
     return v;
+}
+
+// Sum over the block of N values >= 0 a thread; valid in thread 0.  An FP64 addition
+// takes the FP64 pipe 64 cycles, and a shuffle tree is ten of them in a row.
+// Here the values become integers of 62 bits below the block's largest
+// exponent, in three limbs that are added per thread and then by a warp with one
+// instruction each (redux), so a term is off by less than 2^-62 of the largest one and the
+// sum is rounded to FP64 once.  Zeros, tiny values, Inf and NaN take the FP64 additions.
+// A limb's sum fits 32 bits: 21 bits, N blockDim <= 2048 values.
+template <int N>
+__device__ __forceinline__ double block_sum_of(const double (&v)[N]) {
+    __shared__ unsigned smx[32];
+    __shared__ unsigned sl[3][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int nwarps = (blockDim.x + 31) >> 5;
+    unsigned m = 0;
+#pragma unroll
+    for (int i = 0; i < N; i++) m = max(m, (unsigned)__double2hiint(v[i]));
+    m = __reduce_max_sync(0xffffffffu, m);  // a sign bit or a NaN comes out on top
+    __syncthreads();  // protects the arrays against a previous use
+    if (lane == 0) smx[warp] = m;
+    __syncthreads();
+    m = __reduce_max_sync(0xffffffffu, lane < nwarps ? smx[lane] : 0u);
+    const int e = (int)(m >> 20);
+    if (e < 128 || e >= 2047) {
+        double a = v[0];
+#pragma unroll
+        for (int i = 1; i < N; i++) a += v[i];
+        return block_sum_fp64(a);
+    }
+    unsigned l[3] = {0, 0, 0};
+#pragma unroll
+    for (int i = 0; i < N; i++) {
+        const unsigned hi = (unsigned)__double2hiint(v[i]), lo = (unsigned)__double2loint(v[i]);
+        const unsigned mh = (hi & 0xFFFFFu) | (hi >> 20 ? 0x100000u : 0u);
+        const int t = min(2 + e - (int)(hi >> 20), 63);
+        const unsigned long long n = ((unsigned long long)mh << 32 | lo) << 11 >> t;  // below 2^62
+        l[0] += (unsigned)n & 0x1FFFFFu;
+        l[1] += (unsigned)(n >> 21) & 0x1FFFFFu;
+        l[2] += (unsigned)(n >> 42);
+    }
+#pragma unroll
+    for (int k = 0; k < 3; k++) l[k] = __reduce_add_sync(0xffffffffu, l[k]);
+    if (lane == 0) {
+#pragma unroll
+        for (int k = 0; k < 3; k++) sl[k][warp] = l[k];
+    }
+    __syncthreads();
+    if (warp != 0) return 0.0;
+    unsigned long long s[3];
+#pragma unroll
+    for (int k = 0; k < 3; k++) s[k] = __reduce_add_sync(0xffffffffu, lane < nwarps ? sl[k][lane] : 0u);
+    // s2 2^42 + s1 2^21 + s0 in units of 2^(e - 1023 - 61)
+    const unsigned long long q = (s[2] << 31) + (s[1] << 10) + (s[0] >> 11);
+    // q 2^11 as a double with two FP64 additions: its words under the exponents of 2^84 and 2^52
+    const double a = __hiloint2double(0x45300000, (int)(unsigned)(q >> 32)), b = __hiloint2double(0x43300000, (int)(unsigned)q);
+    const double r = (a - __hiloint2double(0x45300000, 0x00100000)) + b;  // 2^84 + 2^52
+    return r * __hiloint2double((e - 61 + 11) << 20, 0);
+}
+__device__ inline double block_sum(double v) {
+    const double one[1] = {v};
+    return block_sum_of(one);
 }
 
 __device__ inline void run_finisher(const RedArgs& r, int slot, double sum) {
@@ -111,6 +175,10 @@ __device__ inline void grid_reduce(double v, const RedArgs& r, int slot, unsigne
     const double bs = block_sum(v);
     __shared__ int s_last;
     double* part = r.partials + (size_t)slot * r.slot_cap;
+    if (r.op == FIN_PARTIAL) {
+        if (threadIdx.x == 0) part[bid] = bs;
+        return;
+    }
     if (threadIdx.x == 0) {
         part[bid] = bs;
         __threadfence();
@@ -140,6 +208,24 @@ __device__ inline void grid_reduce(double v, const RedArgs& r, int slot, unsigne
         r.counter[slot] = 0u;
         __threadfence();
     }
+}
+
+// The sum of a slot's n partials (FIN_PARTIAL, an earlier kernel), the same in every block
+// that forms it (blocks of 256 threads, at most kMaxPartials of them); valid in thread 0.
+constexpr int kMaxPartials = 2048;
+__device__ inline double sum_partials(const RedArgs& r, int slot, int n) {
+    const double* part = r.partials + (size_t)slot * r.slot_cap;
+    if (n <= 512) {
+        double v[2];
+#pragma unroll
+        for (int i = 0; i < 2; i++) v[i] = i * 256 + (int)threadIdx.x < n ? __ldcg(part + i * 256 + threadIdx.x) : 0.0;
+        return block_sum_of(v);
+    }
+    double v[kMaxPartials / 256];
+#pragma unroll
+    for (int i = 0; i < kMaxPartials / 256; i++)
+        v[i] = i * 256 + (int)threadIdx.x < n ? __ldcg(part + i * 256 + threadIdx.x) : 0.0;
+    return block_sum_of(v);
 }
 
 // Single-slot form: every block of the grid contributes.

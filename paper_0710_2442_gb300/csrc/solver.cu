@@ -49,7 +49,7 @@ namespace wl {
 
 namespace {
 
-void schur_launch(const GaugeField& gf, Prec sp, Vec out, Vec in, Vec tmp, int nrhs, double kappa, int dag,
+int schur_launch(const GaugeField& gf, Prec sp, Vec out, Vec in, Vec tmp, int nrhs, double kappa, int dag,
                   const RedArgs* red, const int* skip, int skip_stride, int grid_cap, bool tune_only,
                   cudaStream_t st) {
     // F64 on fixed-point fields: the input is converted, the intermediate field
@@ -98,14 +98,14 @@ void schur_launch(const GaugeField& gf, Prec sp, Vec out, Vec in, Vec tmp, int n
     b.skip = skip;
     b.skip_stride = skip_stride;
     b.grid_cap = red ? grid_cap : 0;
-    launch_hop(b, st);
+    return launch_hop(b, st);
 }
 
 }  // namespace
 
-void schur_apply(const GaugeField& gf, Prec sp, Vec out, Vec in, Vec tmp, int nrhs, double kappa, int dag,
-                 const RedArgs* red, const int* skip, int skip_stride, int grid_cap, cudaStream_t st) {
-    schur_launch(gf, sp, out, in, tmp, nrhs, kappa, dag, red, skip, skip_stride, grid_cap, false, st);
+int schur_apply(const GaugeField& gf, Prec sp, Vec out, Vec in, Vec tmp, int nrhs, double kappa, int dag,
+                const RedArgs* red, const int* skip, int skip_stride, int grid_cap, cudaStream_t st) {
+    return schur_launch(gf, sp, out, in, tmp, nrhs, kappa, dag, red, skip, skip_stride, grid_cap, false, st);
 }
 
 void schur_tune(const GaugeField& gf, Prec sp, Vec out, Vec in, Vec tmp, int nrhs, int dag, const RedArgs* red,
@@ -264,23 +264,22 @@ std::vector<SolveStats> cg_solve_prepared(SpinorField& x, const SpinorField& b, 
     LoopHandle loop;
     auto iteration = [&](cudaStream_t s) {
         const int* skip = &sc->done;
-        RedArgs ra = red.args(slot(2), FIN_CG_ALPHA, nullptr, sc);
-        schur_apply(glo, in.ip, vec(in.q, 0), vec(in.p, 0), vec(in.t, 1), nr, kappa, 0, &ra, skip, kSkipStride,
-                    grid_cap, s);
-        RedArgs rs = red.args(slot(3), FIN_CG_RES, nullptr, sc);
-        cg_xs_update(in.xp, in.ip, vec(in.xin, 0), vec(in.p, 0), vec(in.s, 0), vec(in.q, 0),
-                     in.has_slow ? vec(in.slow, 0) : Vec{nullptr, 0}, g, nr, sc, rs, grid_cap, s);
-        RedArgs rb = red.args(slot(4), FIN_CG_BETA, nullptr, sc);
-        schur_apply(glo, in.ip, vec(in.r, 0), in.s_in(), vec(in.t, 1), nr, kappa, 1, &rb, skip, kSkipStride,
-                    grid_cap, s);
-        cg_p_update(in.ip, vec(in.p, 0), vec(in.r, 0), g, nr, sc, s, loop);
+        const RedArgs rq = red.args(slot(2), FIN_PARTIAL, nullptr, nullptr);
+        const int nq = schur_apply(glo, in.ip, vec(in.q, 0), vec(in.p, 0), vec(in.t, 1), nr, kappa, 0, &rq, skip,
+                                   kSkipStride, grid_cap, s);
+        const RedArgs rs = red.args(slot(3), FIN_PARTIAL, nullptr, nullptr);
+        const int ns = cg_xs_update(in.xp, in.ip, vec(in.xin, 0), vec(in.p, 0), vec(in.s, 0), vec(in.q, 0),
+                                    in.has_slow ? vec(in.slow, 0) : Vec{nullptr, 0}, g, nr, sc, rq, nq, rs, grid_cap, s);
+        const RedArgs rr = red.args(slot(4), FIN_PARTIAL, nullptr, nullptr);
+        const int nb = schur_apply(glo, in.ip, vec(in.r, 0), in.s_in(), vec(in.t, 1), nr, kappa, 1, &rr, skip, kSkipStride,
+                                   grid_cap, s);
+        cg_p_end(in.ip, vec(in.p, 0), vec(in.r, 0), g, nr, sc, rs, ns, rr, nb, loop, grid_cap, s);
     };
 
     // The iterations of a correction as one device-side while loop (a
     // conditional graph node, whose condition the p update sets): no iterations
     // launched after convergence, no host round trip per chunk, and six nodes to
-    // instantiate instead of 96.  16^3 x 32 F16, seven corrections of 27
-    // iterations: see DESIGN's table.
+    // instantiate instead of 96.
     cudaGraphExec_t gexec = nullptr;
     cudaGraph_t graph = nullptr;
     const int chunk = prm.chunk > 0 ? prm.chunk : 16;
@@ -477,7 +476,7 @@ std::vector<SolveStats> cg_solve_prepared(SpinorField& x, const SpinorField& b, 
                         st);
             hops += 2;
             if (restart) convert(in.ip, vec(in.p, 0), in.ip, vec(in.r, 0), g, nr, st);
-            else cg_p_update(in.ip, vec(in.p, 0), vec(in.r, 0), g, nr, sc, st, LoopHandle{});
+            else cg_p_update(in.ip, vec(in.p, 0), vec(in.r, 0), g, nr, sc, st);
             first = false;
 
             while (true) {

@@ -69,8 +69,9 @@ struct SolveStats {
 
 // Mhat (dag = 0) or Mhat^dag (dag = 1) on even blocks of nrhs right-hand
 // sides: out = in - kappa^2 D_eo D_oe in.  tmp: odd blocks of the same
-// precision.  Optional per-rhs |out|^2 reduction and per-rhs skip flags.
-void schur_apply(const GaugeField& gf, Prec sp, Vec out, Vec in, Vec tmp, int nrhs, double kappa, int dag,
+// precision.  Optional per-rhs |out|^2 reduction (the number of its partials is
+// returned) and per-rhs skip flags.
+int schur_apply(const GaugeField& gf, Prec sp, Vec out, Vec in, Vec tmp, int nrhs, double kappa, int dag,
                  const RedArgs* red, const int* skip, int skip_stride, int grid_cap, cudaStream_t st);
 // Tunes the launch configurations of schur_apply's two hops where they are
 // not known yet (the tuning launches write out and tmp); launches nothing else.
