@@ -320,7 +320,7 @@ struct BatchRun {
     DevBuf probs, state, tile_prob, global, partials, counters, ids;
     BatchArgs A{};
     int grid = 1;
-    LaunchConfig hop_lo{128, 1}, hop_64{128, 0}, hop_32{128, 3};
+    LaunchConfig hop_lo{128, 1}, hop_32{128, 3};
     cudaGraphConditionalHandle handle{};
     BatchGlobal* G() const { return global.as<BatchGlobal>(); }
 
@@ -349,7 +349,8 @@ struct BatchRun {
     }
     void hop(const BOp& o, int dag, cudaStream_t st) const {
         if (o.use64 == 1) {
-            hop_t<P_F64, P_F64>(o, dag, hop_64, st);
+            WL_REQUIRE(!dag, "the batched FP64 hop is never daggered");
+            launch_bhop_fx(A, o, grid, st);
         } else if (o.use64 == 2) {
             hop_t<P_F32, P_F32>(o, dag, hop_32, st);
         } else {
@@ -361,13 +362,16 @@ struct BatchRun {
 
 namespace {
 
-void build_problem(HostProb& P, const wilson_problem& in, Prec ip, const SolveParams& prm, cudaStream_t st) {
+void build_problem(HostProb& P, const wilson_problem& in, Prec ip, const SolveParams& prm, int small_vh,
+                   cudaStream_t st) {
     P.g = make_geom(in.L.dims, in.L.bc_phase);
     P.kappa = in.kappa;
     P.g64.prec = P_F64;
     P.g64.recon = 18;
     P.g64.g = P.g;
-    P.g64.buf.alloc(gauge_bytes(P_F64, 18, P.g.stride));
+    // on-chip solves read doubles, the loops' FP64 hop fixed point
+    P.g64.canon = in.gauge;
+    (P.g.Vh <= small_vh ? P.g64.buf : P.g64.fx).alloc(gauge_bytes(P_F64, 18, P.g.stride));
     pack_gauge(P.g64, in.gauge, st);
     P.glo.prec = ip;
     P.glo.recon = 12;
@@ -428,7 +432,8 @@ std::unique_ptr<BatchRun> make_run(const std::vector<HostProb>& hp, const std::v
             D.f[f] = static_cast<char*>(P.f[f].block(parity));
             D.fp[f] = P.f[f].subset == 2 ? P.f[f].pbytes : 0;
         }
-        D.g64 = P.g64.buf.as<const char>();
+        D.g64 = small ? P.g64.buf.as<const char>() : P.g64.fx.as<const char>();
+        D.canon = reinterpret_cast<const char*>(P.g64.canon);
         D.glo = P.glo.buf.as<const char>();
         D.g32 = !P.res32_ok ? nullptr : P.glo.prec == P_F32 ? D.glo : P.g32.buf.as<const char>();
         D.res32_ok = P.res32_ok && !small;
@@ -518,13 +523,13 @@ void batch_solve(int n, const wilson_problem* probs, const SolveParams& prm, wil
     NvtxRange nvtx_batch("wilson batch solve");
     auto t0 = std::chrono::steady_clock::now();
     const Prec ip = prm.inner;
-    std::vector<HostProb> hp(n);
-    for (int i = 0; i < n; i++) build_problem(hp[i], probs[i], ip, prm, st);
-
     // Problems with at most small_vh sites per parity get their own CTA; the
     // others run device loops, one per class of lattice sizes.
     int small_vh = prm.batch_small_vh;
     if (const char* e = std::getenv("WILSON_BATCH_SMALL_VH")) small_vh = std::atoi(e);
+    std::vector<HostProb> hp(n);
+    for (int i = 0; i < n; i++) build_problem(hp[i], probs[i], ip, prm, small_vh, st);
+
     int max_classes = 4;
     if (const char* e = std::getenv("WILSON_BATCH_CLASSES"))
         if (std::atoi(e) > 0) max_classes = std::atoi(e);
@@ -583,11 +588,7 @@ void batch_solve(int n, const wilson_problem* probs, const SolveParams& prm, wil
         if (std::atoll(e) > 0) budget_ns = std::min(budget_ns, (unsigned long long)std::atoll(e) * 1000000ULL);
 
     // tune the batched hop kernels of every loop class (non-reducing launches on scratch fields)
-    std::vector<LaunchConfig> cands, cands64;
-    for (const LaunchConfig& c : hop_candidates()) {
-        cands.push_back(c);
-        if (c.variant < 3) cands64.push_back(c);
-    }
+    const std::vector<LaunchConfig>& cands = hop_candidates();
     // F16 / BF16 inner hops: the pipelined stencil first, so that another candidate
     // replaces it only when more than the tuner's margin faster (inside the
     // graph the pipelined hop wins by more than it does alone: the 64-problem
@@ -615,10 +616,6 @@ void batch_solve(int n, const wilson_problem* probs, const SolveParams& prm, wil
             dispatch_low(ip, [&](auto I) { Rp->hop_t<decltype(I)::value, decltype(I)::value>(o, 0, c, st); });
         });
         if (hop_pin.variant >= 0) R->hop_lo = hop_pin;
-        snprintf(key, sizeof(key), "bhop:f64:n%d:t%d", R->nprob, R->ntiles);
-        const BOp o64 = R->op(BF_Q64, BF_T64, BF_X, 0, 1, 2, -1, 0, BF_NONE, 0);
-        R->hop_64 = tune_launch(key, cands64, LaunchConfig{128, 0}, st,
-                                [&](const LaunchConfig& c) { Rp->hop_t<P_F64, P_F64>(o64, 0, c, st); });
         bool any32 = false;
         for (int i : R->members) any32 = any32 || hp[i].res32_ok;
         if (any32) {

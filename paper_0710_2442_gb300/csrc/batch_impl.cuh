@@ -25,7 +25,8 @@ struct BatchProb {
     Geom g;
     char* f[BF_N];        // parity block (half fields) or parity-0 block (full fields)
     long long fp[BF_N];   // parity step of full fields, 0 for half fields
-    const char* g64;      // FP64 18-real links
+    const char* g64;      // FP64 18-real links (small problems), or their fixed-point form
+    const char* canon;    // the problem's canonical links
     const char* glo;      // inner links
     const char* g32;      // FP32 12-real links of the FP32 residuals (null: none)
     double kappa, tol, delta;
@@ -227,15 +228,13 @@ __global__ void __launch_bounds__(256, MINB) bhop_kernel(const BatchArgs A, cons
         const BatchProb& Pr = A.probs[pid];
         HopParams P;
         P.g = Pr.g;
-        P.gauge = op.use64 == 1 ? Pr.g64 : op.use64 == 2 ? Pr.g32 : Pr.glo;
+        P.gauge = op.use64 == 2 ? Pr.g32 : Pr.glo;
         const int p = op.out_parity;
         char* out = Pr.f[op.f_out] + p * Pr.fp[op.f_out];
         const char* in = Pr.f[op.f_in] + (1 - p) * Pr.fp[op.f_in];
         const char* x = op.f_x >= 0 ? Pr.f[op.f_x] + p * Pr.fp[op.f_x] : nullptr;
         const T a = (T)coef_of(op.coef, Pr.kappa);
         const Geom& g = P.g;
-        // outer is written only by the correction finisher, a later kernel
-        const bool zero = op.zero_first && __ldcg(&A.state[pid].outer) == 0;
         double nrm = 0.0;
         const int h0 = (t - Pr.tile0) * A.tile;
         for (int j = threadIdx.x; j < A.tile; j += blockDim.x) {
@@ -244,15 +243,10 @@ __global__ void __launch_bounds__(256, MINB) bhop_kernel(const BatchArgs A, cons
             int c[4], s;
             site_of_half(h, p, g, c, s);
             cpx<T> acc[12];
-            if (zero) {
-#pragma unroll
-                for (int k = 0; k < 12; k++) acc[k] = {T(0), T(0)};
-            } else {
-                hop_dir<SP, GP, R, DAG, 0, true>(acc, P, in, p, h, c, s);
-                hop_dir<SP, GP, R, DAG, 1, false>(acc, P, in, p, h, c, s);
-                hop_dir<SP, GP, R, DAG, 2, false>(acc, P, in, p, h, c, s);
-                hop_dir<SP, GP, R, DAG, 3, false>(acc, P, in, p, h, c, s);
-            }
+            hop_dir<SP, GP, R, DAG, 0, true>(acc, P, in, p, h, c, s);
+            hop_dir<SP, GP, R, DAG, 1, false>(acc, P, in, p, h, c, s);
+            hop_dir<SP, GP, R, DAG, 2, false>(acc, P, in, p, h, c, s);
+            hop_dir<SP, GP, R, DAG, 3, false>(acc, P, in, p, h, c, s);
             if (x) {
                 cpx<T> xv[12];
                 SF::load(x, g.stride, h, xv);
@@ -764,7 +758,8 @@ void launch_bhop(const BatchArgs& A, const BOp& o, int dag, int v, int block, in
 extern template void launch_bhop<P_F32, P_F32>(const BatchArgs&, const BOp&, int, int, int, int, cudaStream_t);
 extern template void launch_bhop<P_F16, P_F16>(const BatchArgs&, const BOp&, int, int, int, int, cudaStream_t);
 extern template void launch_bhop<P_BF16, P_BF16>(const BatchArgs&, const BOp&, int, int, int, int, cudaStream_t);
-extern template void launch_bhop<P_F64, P_F64>(const BatchArgs&, const BOp&, int, int, int, int, cudaStream_t);
+// The FP64 hop, dagger = 0 (batch_hop_64.cu).
+void launch_bhop_fx(const BatchArgs& A, const BOp& o, int blocks, cudaStream_t st);
 
 // The CTA-resident solves of nprob small problems (ids: their indices), inner
 // precision IP.  Instantiated one inner precision per translation unit

@@ -140,7 +140,7 @@ __device__ __forceinline__ longlong2 fx_row(const FxCplx u[3], const FxCplx h[3]
     return make_longlong2(fx_sum(re), fx_sum(im));
 }
 // h times the boundary phase (pr, pi).
-__device__ __noinline__ void fx_phase3(double pr, double pi, FxCplx* h) {
+inline __device__ __noinline__ void fx_phase3(double pr, double pi, FxCplx* h) {
     const FxCplx eta{fx_link((unsigned)__double2hiint(pr), (unsigned)__double2loint(pr)),
                      fx_link((unsigned)__double2hiint(pi), (unsigned)__double2loint(pi))};
 #pragma unroll
@@ -297,7 +297,7 @@ __device__ __forceinline__ void fx_spin_of(const FxTile& T, int spin, int c0, in
 }
 
 // A hop of the FP64 stencil (a link or field out of the fixed-point ranges).
-__device__ __noinline__ void fx_native_hop(const cpx<double> v[12], const double2* lk, int ws, int recon, int mu, bool fwd,
+inline __device__ __noinline__ void fx_native_hop(const cpx<double> v[12], const double2* lk, int ws, int recon, int mu, bool fwd,
                                            int dag, bool wrap, const Geom& g, cpx<double> acc[12]) {
     cpx<double> h[6], w[6], U[3][3];
 #pragma unroll
@@ -368,7 +368,7 @@ __device__ __forceinline__ double fx_norm(const double2 (&v)[N]) {
 }
 
 // The output of a site computed that way; returns its squared modulus.
-__device__ __noinline__ double fx_finish_native(const FxParams& P, int p, int k, int s, const cpx<double> acc[12]) {
+inline __device__ __noinline__ double fx_finish_native(const FxParams& P, int p, int k, int s, const cpx<double> acc[12]) {
     uint4* out = const_cast<uint4*>(fx_at(P.out, p, k, s));
     const uint4* x = P.xpay ? fx_at(P.x, p, k, s) : nullptr;
     double n2 = 0.0;
@@ -382,7 +382,7 @@ __device__ __noinline__ double fx_finish_native(const FxParams& P, int p, int k,
 }
 
 // One site of fields in doubles on the FP64 stencil, output included.
-__device__ __noinline__ double fx_redo_site(const FxParams& P, int p, int k, int h) {
+inline __device__ __noinline__ double fx_redo_site(const FxParams& P, int p, int k, int h) {
     cpx<double> acc[12];
 #pragma unroll 1
     for (int q = 0; q < 12; q++) acc[q] = cpx<double>{0.0, 0.0};
@@ -604,7 +604,7 @@ __device__ __forceinline__ bool fx_turn_hop(const FxParams& P, FxSlots<TB>& T, F
 
 // One site of fixed-point fields, if it is out of range, on the FP64 stencil, output
 // included; returns its squared modulus.
-__device__ __noinline__ double fx_redo_site1(const FxParams& P, int p, int k, int h, int outfx);
+inline __device__ __noinline__ double fx_redo_site1(const FxParams& P, int p, int k, int h, int outfx);
 
 // One site on two threads, lanes l and l + 16 of a warp, one per half-spin row: a
 // thread keeps 18 64-bit sums instead of the 24 of a thread with both rows, and half of
@@ -752,7 +752,7 @@ __global__ void __launch_bounds__(TB, MINB) hop_kernel_fx1(const __grid_constant
     if (RED) grid_reduce(nrm, P.red, k, nb * gridDim.y, sb + nb * blockIdx.y);
 }
 
-__device__ __noinline__ double fx_redo_site1(const FxParams& P, int p, int k, int h, int outfx) {
+inline __device__ __noinline__ double fx_redo_site1(const FxParams& P, int p, int k, int h, int outfx) {
     const Geom& g = P.g;
     const char* in = P.in.p + (P.full && p == 0 ? P.in.pstep : 0) + k * P.in.rstep;
     const int* ex = reinterpret_cast<const int*>(in + 192LL * g.stride);
@@ -796,12 +796,51 @@ __device__ __noinline__ double fx_redo_site1(const FxParams& P, int p, int k, in
     return fx_finish_native(P, p, k, s, acc);
 }
 
+// Up to 32 sites, h0 to end, of parity p and right-hand side k, by a block of W warps; returns
+// this thread's share of the output's squared modulus (RED).  Ends with a barrier.
+template <bool FXL, bool RED, int W>
+__device__ __forceinline__ double fx_tile(const FxParams& P, FxTile& T, int p, int k, int h0, int end) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int h = h0 + lane;
+    const bool ok = h < end;
+    double nrm = 0.0;
+    int c[4], s;
+    site_of_half(ok ? h : 0, p, P.g, c, s);
+    if (warp == 0) T.bad[lane] = 0;
+    __syncthreads();
+#pragma unroll 1
+    for (int j = warp; j < 8; j += W) fx_hop<FXL>(P, T, j, p, k, c, s, lane);
+    __syncthreads();
+    if (ok) {
+        uint4* out = const_cast<uint4*>(fx_at(P.out, p, k, s));
+        const uint4* x = P.xpay ? fx_at(P.x, p, k, s) : nullptr;
+        if (!T.bad[lane]) {
+            const int spin = warp & 3;
+            if (warp < 4) {
+                double2 v[W == 8 ? 2 : 3];
+                fx_spin_of(T, spin, 0, P.dag, lane, v);
+                fx_finish(P, out, x, spin * 3, v);
+                if (RED) nrm += fx_norm(v);
+            } else {
+                double2 v[1];
+                fx_spin_of(T, spin, 2, P.dag, lane, v);
+                fx_finish(P, out, x, spin * 3 + 2, v);
+                if (RED) nrm += fx_norm(v);
+            }
+        } else if (warp == 0) {
+            const double n2 = fx_redo_site(P, p, k, h);
+            if (RED) nrm += n2;
+        }
+    }
+    __syncthreads();  // the tile is reused
+    return nrm;
+}
+
 // Grid: blockIdx.x = tile * nrhs + rhs, tiles of 32 sites; blockIdx.y = output
 // parity of a full launch.  W warps, 4 or 8.
 template <bool FXL, bool RED, int W, int MINB>
 __global__ void __launch_bounds__(32 * W, MINB) hop_kernel_fx(const __grid_constant__ FxParams P) {
     __shared__ FxTile T;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int k = blockIdx.x % P.nrhs;
     const int sb = blockIdx.x / P.nrhs;
     const int nb = gridDim.x / P.nrhs;
@@ -810,37 +849,8 @@ __global__ void __launch_bounds__(32 * W, MINB) hop_kernel_fx(const __grid_const
     if (P.skip && __ldcg(P.skip + (size_t)k * P.skip_stride)) return;
     double nrm = 0.0;
     for (int h0 = sb * 32; h0 < P.g.Vh; h0 += nb * 32) {
-        const int h = h0 + lane;
-        const bool ok = h < P.g.Vh;
-        int c[4], s;
-        site_of_half(ok ? h : 0, p, P.g, c, s);
-        if (warp == 0) T.bad[lane] = 0;
-        __syncthreads();
-#pragma unroll 1
-        for (int j = warp; j < 8; j += W) fx_hop<FXL>(P, T, j, p, k, c, s, lane);
-        __syncthreads();
-        if (ok) {
-            uint4* out = const_cast<uint4*>(fx_at(P.out, p, k, s));
-            const uint4* x = P.xpay ? fx_at(P.x, p, k, s) : nullptr;
-            if (!T.bad[lane]) {
-                const int spin = warp & 3;
-                if (warp < 4) {
-                    double2 v[W == 8 ? 2 : 3];
-                    fx_spin_of(T, spin, 0, P.dag, lane, v);
-                    fx_finish(P, out, x, spin * 3, v);
-                    if (RED) nrm += fx_norm(v);
-                } else {
-                    double2 v[1];
-                    fx_spin_of(T, spin, 2, P.dag, lane, v);
-                    fx_finish(P, out, x, spin * 3 + 2, v);
-                    if (RED) nrm += fx_norm(v);
-                }
-            } else if (warp == 0) {
-                const double n2 = fx_redo_site(P, p, k, h);
-                if (RED) nrm += n2;
-            }
-        }
-        __syncthreads();  // the tile is reused
+        const double n2 = fx_tile<FXL, RED, W>(P, T, p, k, h0, P.g.Vh);
+        if (RED) nrm += n2;
     }
     pdl_trigger();
     if (RED) grid_reduce(nrm, P.red, k, nb * gridDim.y, sb + nb * blockIdx.y);

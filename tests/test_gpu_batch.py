@@ -255,3 +255,22 @@ def test_batch_fp32_outer_residuals(w, oracle_mod, monkeypatch, inner):
     assert rc == 0 and all(s["outer_f32"] == 0 for s in st)
     for q, (dims, U, b, kappa), s in zip(probs, hf, st):
         assert true_resid(oracle_mod, U, host(q["x"]), b, dims, kappa) <= 1.1e-6
+
+
+# The device loops' FP64 hop is in fixed point and takes its sites 32 at a time: ragged last
+# groups, tiles longer and shorter than the lattice, and links without a fixed-point form
+# (zero ones), whose sites are done over in FP64.
+@pytest.mark.parametrize("tile,zero_links", [("128", True), ("256", False), ("512", True)])
+def test_batch_fixed_point_hop(w, oracle_mod, monkeypatch, tile, zero_links):
+    monkeypatch.setenv("WILSON_BATCH_SMALL_VH", "0")
+    monkeypatch.setenv("WILSON_BATCH_TILE", tile)
+    dims, kappa = (6, 2, 10, 6), 0.13
+    U = inputs.gauge_field(dims, "weak", eps=0.3, seed=77)
+    if zero_links:
+        U.reshape(-1, 4, 3, 3)[::37, 2] = 0.0
+    b = inputs.gaussian_spinor(dims, seed=78)
+    L = w.lattice(dims, inputs.DEFAULT_PHASES)
+    q = dict(L=L, kappa=kappa, gauge=dev(U), b=dev(b), x=dev(np.zeros_like(b)))
+    rc, st, info = w.wilson_batch_solve([q], w.solver_defaults(w.PREC["f32"]))
+    assert rc == 0 and info["tiles"] > 0 and st[0]["status"] == 0
+    assert true_resid(oracle_mod, U, host(q["x"]), b, dims, kappa) <= 1.1e-10
