@@ -128,6 +128,20 @@ __device__ __forceinline__ double fx_double(long long v, const FxBias& b) {
     const int h = (int)((unsigned)(v >> 32) ^ 0x80000000u), l = (int)(unsigned)v;
     return (__hiloint2double(b.a, h) - b.c) + __hiloint2double(b.b, l);
 }
+// The same, bit for bit, in integer instructions, for results that are normal or zero (kFxEmin): where
+// several warps of a sub-partition convert at a time, the two additions of each wait for
+// the FP64 pipe (64 cycles an instruction).
+__device__ __forceinline__ double fx_double_int(long long v, int k) {
+    const unsigned sg = (unsigned)(v >> 32) & 0x80000000u;
+    unsigned long long m = (unsigned long long)(v < 0 ? -v : v);
+    const int n = __clzll((long long)m);
+    m <<= n & 63;
+    const unsigned long long q = m >> 11;  // 53 bits; the others round, to nearest even
+    const unsigned up = ((unsigned)m & 0x7FFu) + ((unsigned)q & 1) > 0x400u;
+    // the leading bit of q adds 1 to the exponent field, a carry of the rounding another
+    const unsigned long long w = q + up + ((unsigned long long)(unsigned)(1023 + 63 - 1 + k - n) << 52);
+    return m ? __hiloint2double((int)((unsigned)(w >> 32) | sg), (int)(unsigned)w) : 0.0;
+}
 #endif
 
 // A sum of products of link-like numbers back to limbs at 2^58, l in [0, 2^30).

@@ -115,3 +115,18 @@ def test_output_over_an_input(w, dims):
         out = both[1200:].view_as(src)
         w.wilson_dslash_eo(out, U, both[: src.numel()].view_as(src), L, 0, 0.13, op)
         assert torch.equal(out, want)
+
+
+@pytest.mark.parametrize("scale", [1.0, 2.0**-400, 2.0**450])
+def test_conversions_agree(w, scale):
+    """The split kernel rounds its sums to FP64 with FP64 additions at up to one tile per SM
+    (53 tiles, one right-hand side) and with integers beyond (three): the same bits."""
+    dims = (6, 10, 4, 14)
+    U = inputs.gauge_field(dims, "random", seed=409)
+    src = inputs.gaussian_spinor(inputs.volume(dims) // 2, seed=410) * scale
+    src[::3] = 0.0  # exact zeros and sums of few terms, of either sign
+    src[1::3] = np.where(np.abs(src[1::3].real) > scale, src[1::3], -scale * 2.0**-30)
+    args = (dims, PHASES, w.WILSON_F64, 18, 1, 0, w.WILSON_OP_HOP)
+    three = handle_hop(w, U, np.stack([src, -src, src]), *args, nrhs=3)
+    for k, sign in enumerate((1.0, -1.0, 1.0)):
+        assert np.array_equal(three[k], handle_hop(w, U, sign * src, *args))
