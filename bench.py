@@ -47,7 +47,7 @@ SOLUTIONS = []
 # DRAM bytes (read + write) per launch of the tuned 32^3 x 64 even-odd kernel, read from one
 # ncu capture of that kernel (keyed by storage precision and link reals); a fixed figure, not
 # measured by this run.
-NCU_TRAFFIC = {("f32", 12): 581.6e6, ("f16", 12): 298.5e6, ("f64", 18): 1621.5e6}
+NCU_TRAFFIC = {("f32", 12): 581.6e6, ("f16", 12): 298.5e6}
 TRAFFIC_SOURCE = "ncu capture of the tuned kernel (dram__bytes_read.sum + dram__bytes_write.sum), fixed figure"
 WORKLOAD = "dslash_eo_f32_32^3x64"
 L2_NOTE = ("inputs larger than L2: each application streams 403 MB of links plus 2 x 101 MB of spinors "
@@ -310,18 +310,6 @@ def run_ours(args, ws, rank, local, fields):
                      "traffic_source": TRAFFIC_SOURCE, "peak_kind": peak_kind,
                      "algorithmic_bytes_per_launch": comp_bytes, "launch_us": round(t_launch * 1e6, 2)},
     }
-    if args.prec == "f64":
-        # FP64 is bound by GB300's FP64 rate (FP64 pipe 91 % busy at 12 % DRAM
-        # throughput): roofline against the FP64 FMA peak measured above.
-        gf_launch = flops / t_launch / 1e9
-        f64_peak = alu["f64_gflops"]
-        line["roofline"] = {"bound": "alu", "achieved": round(gf_launch, 1), "peak": f64_peak,
-                            "unit": "GFLOP/s", "frac": round(gf_launch / f64_peak, 4),
-                            "traffic": NCU_TRAFFIC.get((args.prec, args.recon)), "traffic_source": TRAFFIC_SOURCE,
-                            "peak_kind": "measured (wilson_probe_fma_peak, FP64 FMA)",
-                            "launch_us": round(t_launch * 1e6, 2),
-                            "hbm": {"achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
-                                    "frac": round(achieved / peak, 4)}}
     line.update({"clocks": clocks, "e2e": e2e, "gpu_launches": launches, "alu_peaks": alu,
                  "access_pattern": access})
     if rank == 0 and not args.no_solver:
@@ -383,7 +371,7 @@ def run_solver_block(w, torch, dev, stream, precs, hbm_peak):
             byts = model.cg_inner_bytes_per_site(name, recon) * Vh
             t_it = st["inner_seconds"] / st["inner_iters"]
             rec["roofline_inner_iteration"] = {
-                "bound": "alu" if name == "f64" else "hbm", "bytes_per_site": model.cg_inner_bytes_per_site(name, recon),
+                "bound": "hbm", "bytes_per_site": model.cg_inner_bytes_per_site(name, recon),
                 "algorithmic_bytes": byts, "us_per_iteration": round(t_it * 1e6, 2),
                 "achieved_GBs": round(byts / t_it / 1e9, 1), "peak_GBs": hbm_peak,
                 "frac": round(byts / t_it / 1e9 / hbm_peak, 4),

@@ -93,8 +93,8 @@ int launch_hop(const HopLaunch& L, cudaStream_t st) {
     auto slab_ok = [&](int block) { return P.nrhs == 1 && !L.full && hop_slab_fits(P.g, block); };
 
     // The grid of a launch.  A reducing launch walks the lattice with a capped
-    // grid (one partial per block, summed by the last block in a fixed
-    // order): one resident wave of the block size, the blocks that the
+    // grid (one partial per block, summed in a fixed order by the last
+    // block or by the kernels that use the sum): one resident wave of the block size, the blocks that the
     // variant's register budget guarantees on every SM, so no tail wave.
     auto grid_of = [&](const LaunchConfig& c) {
         int cap = 0;
@@ -150,12 +150,9 @@ int launch_hop(const HopLaunch& L, cudaStream_t st) {
         if (L.red) cands.erase(std::remove_if(cands.begin(), cands.end(),
                                               [&](const LaunchConfig& c) { return !reduces(c.variant); }),
                                cands.end());
-        if (L.no_tune)
-            cfg = tune_lookup(key, cands, LaunchConfig{});
-        else
-            cfg = tune_launch(key, cands, LaunchConfig{}, st, [&](const LaunchConfig& c) {
-                dispatch(Pt, sp, gp, R, c.block, grid_of(c), ny, dag, c.variant, st);
-            });
+        cfg = tune_launch(key, cands, LaunchConfig{}, st, [&](const LaunchConfig& c) {
+            dispatch(Pt, sp, gp, R, c.block, grid_of(c), ny, dag, c.variant, st);
+        });
     }
     WL_REQUIRE(hop_variant_valid(cfg.variant, sp, R, P.nrhs), "hop variant does not fit this launch");
     // a pinned variant without a fused reduction: the paired kernel, same block

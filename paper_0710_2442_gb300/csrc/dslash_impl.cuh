@@ -26,7 +26,7 @@
 //
 // Kernel families (the variant numbers the autotuner and WILSON_HOP_VARIANT
 // use):
-//   hop_kernel     0..2  scalar stencil (and every FP64 launch)
+//   hop_kernel     0..2  scalar stencil (FP64: pinned launches; others take dslash_fx.cuh)
 //   hop_kernel_p   3..5  the same stencil on paired FP32 instructions
 //   hop_kernel_pm  6..9  several right-hand sides per thread (register-blocked)
 //   hop_kernel_rl  10    links staged in shared memory, loop over right-hand sides

@@ -251,7 +251,6 @@ struct HopLaunch {
     int variant;           // kernel register-budget variant when block > 0
     int grid_cap;          // max blocks of a reducing launch (0 = no cap)
     int tune_only;         // 1: tune the launch configuration if it is not known yet, launch nothing else
-    int no_tune;           // 1: take a cached decision or the default configuration, never time candidates
     // F64 on the fixed-point hops (fx_hops(*gauge)); fields of fx_spinor_bytes per parity
     const void* fx_in;     // the input as a fixed-point field, or null
     void* fx_tmp;          // else room to convert it (null: the kernel that takes doubles)

@@ -16,8 +16,6 @@ namespace wl {
 
 enum FinOp {
     FIN_STORE = 0,     // result[0] = sum
-    FIN_CG_ALPHA = 1,  // |q|^2: alpha = gam / |q|^2
-    FIN_CG_RES = 2,    // |s|^2: convergence test, iteration count
     FIN_CG_BETA = 3,   // |r|^2: beta = |r|^2 / gam, gam = |r|^2
     FIN_ADD = 4,       // result[0] += sum
     FIN_CG_GAM = 5,    // |r|^2: gam = |r|^2 (start of a CG)
@@ -140,23 +138,6 @@ __device__ inline void run_finisher(const RedArgs& r, int slot, double sum) {
     switch (r.op) {
         case FIN_STORE: r.result[slot] = sum; break;
         case FIN_ADD: r.result[slot] += sum; break;
-        case FIN_CG_ALPHA:
-            sc->pq = sum;
-            if (!(sum > 0.0) || !isfinite(sum)) {
-                sc->alpha = 0.0;
-                if (!isfinite(sum)) sc->done = 3;
-                else if (sc->done == 0) sc->done = 1;  // Mhat p = 0: nothing left to do
-            } else {
-                sc->alpha = sc->gam / sum;
-            }
-            break;
-        case FIN_CG_RES:
-            sc->snorm2 = sum;
-            sc->iter += 1;
-            if (!isfinite(sum)) sc->done = 3;
-            else if (sum <= sc->stop2) sc->done = 1;
-            else if (sc->iter >= sc->maxiter) sc->done = 2;
-            break;
         case FIN_CG_GAM:
             sc->gam = sum;
             if (!isfinite(sum)) sc->done = 3;

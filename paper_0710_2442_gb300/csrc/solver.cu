@@ -29,12 +29,13 @@
 //
 // One inner iteration is six launches, all reading their scalars from device
 // memory and exiting at once when their right-hand side is done:
-//   t = D_oe p;  q = p - k^2 D_eo t, |q|^2 -> alpha
-//   x += alpha p, s -= alpha q, |s|^2 -> convergence test
-//   t = D'_oe s;  r = s - k^2 D'_eo t, |r|^2 -> beta      (D' = g5 D g5)
-//   p = r + beta p
-// A chunk of iterations is captured once into a CUDA graph and replayed; the
-// host reads the scalars once per chunk.
+//   t = D_oe p;  q = p - k^2 D_eo t, partials of |q|^2
+//   alpha from them; x += alpha p, s -= alpha q, partials of |s|^2
+//   t = D'_oe s;  r = s - k^2 D'_eo t, partials of |r|^2      (D' = g5 D g5)
+//   convergence test, beta; p = r + beta p
+// The iteration is the body of a device-side loop (a conditional graph node, whose
+// condition the last launch sets); the host reads the scalars when the loop has
+// ended.  Without conditional nodes a chunk of iterations is captured and replayed.
 #include <algorithm>
 #include <chrono>
 #include <cmath>
@@ -253,7 +254,7 @@ std::vector<SolveStats> cg_solve_prepared(SpinorField& x, const SpinorField& b, 
     {
         // the inner operators as the iterations launch them (second hop
         // reducing: its own launch kind) and without reductions
-        const RedArgs rt = red.args(slot(2), FIN_CG_ALPHA, nullptr, sc);
+        const RedArgs rt = red.args(slot(2), FIN_PARTIAL, nullptr, nullptr);
         for (int dag = 0; dag < 2; dag++) {
             schur_tune(glo, in.ip, vec(in.q, 0), vec(in.p, 0), vec(in.t, 1), nr, dag, &rt, grid_cap, st);
             schur_tune(glo, in.ip, vec(in.q, 0), vec(in.p, 0), vec(in.t, 1), nr, dag, nullptr, 0, st);
