@@ -76,9 +76,10 @@ __device__ __forceinline__ int site_parity(int s, const Geom& g) {
 // Canonical <-> SoA over all right-hand sides in one launch: blockIdx.y is the
 // right-hand side.  Both are bound by their bytes; one launch of 21 us per
 // right-hand side reached 4.5 TB/s on 24^3 x 48 F32 and, on 16^3 x 32 BF16, spent 12 x 7.4 us on
-// what the bytes allow in 37.  They are launched like the hops (launch_dep).
+// what the bytes allow in 37.  They are launched like the hops (launch_dep).  A launch bound of 256
+// threads on the import made it 4 us slower on 32^3 x 64 F32 (50 to 54 us).
 template <int SP>
-__global__ void __launch_bounds__(256) pack_spinor_kernel(const double2* __restrict__ canon, char* base,
+__global__ void pack_spinor_kernel(const double2* __restrict__ canon, char* base,
                                                           long long pbytes, long long rstep, int subset, Geom g) {
     using SF = SpinorFmt<SP>;
     using T = typename SF::real;
