@@ -372,12 +372,13 @@ __device__ __forceinline__ double fx_norm(const double2 (&v)[N]) {
 }
 
 // The output of a site computed that way; returns its squared modulus.
-inline __device__ __noinline__ double fx_finish_native(const FxParams& P, int p, int k, int s, const cpx<double> acc[12]) {
+inline __device__ __noinline__ double fx_finish_native(const FxParams& P, int p, int k, int s, const cpx<double> acc[12], int q0,
+                                                        int q1) {
     uint4* out = const_cast<uint4*>(fx_at(P.out, p, k, s));
     const uint4* x = P.xpay ? fx_at(P.x, p, k, s) : nullptr;
     double n2 = 0.0;
 #pragma unroll 1
-    for (int q = 0; q < 12; q++) {
+    for (int q = q0; q < q1; q++) {
         double2 v[1] = {make_double2(acc[q].re, acc[q].im)};
         fx_finish(P, out, x, q, v);
         n2 += fx_norm(v);
@@ -407,7 +408,7 @@ inline __device__ __noinline__ double fx_redo_site(const FxParams& P, int p, int
         }
         fx_native_hop(v, lk, P.un.word_step, P.un_recon, j >> 1, (j & 1) == 0, P.dag, wrap, P.g, acc);
     }
-    return fx_finish_native(P, p, k, s, acc);
+    return fx_finish_native(P, p, k, s, acc, 0, 12);
 }
 
 // ---------------------------------------------------------------------------
@@ -606,9 +607,11 @@ __device__ __forceinline__ bool fx_turn_hop(const FxParams& P, FxSlots<TB>& T, F
     return bad;
 }
 
-// One site of fixed-point fields, if it is out of range, on the FP64 stencil, output
-// included; returns its squared modulus.
-inline __device__ __noinline__ double fx_redo_site1(const FxParams& P, int p, int k, int h, int outfx);
+// One site of fixed-point fields, if it is out of range, on the FP64 stencil by its two threads
+// (r = 0 the x and y directions, 1 z and t), output included where mine; returns this thread's share of its
+// squared modulus.  All lanes of a warp call it.  A lattice that is out of range throughout takes 1.1 ms a hop
+// this way (24^3 x 48), 2.0 ms on one of the two threads.
+inline __device__ __noinline__ double fx_redo_site1(const FxParams& P, int p, int k, int h, int r, bool mine, int outfx);
 
 // One site on two threads, lanes l and l + 16 of a warp, one per half-spin row: a
 // thread keeps 18 64-bit sums instead of the 24 of a thread with both rows, and half of
@@ -743,20 +746,21 @@ __global__ void __launch_bounds__(TB, MINB) hop_kernel_fx1(const __grid_constant
             if (RED) nrm += fx_norm(v);
         }
     }
-    if (redo && t.r == 0) {
+    if (__any_sync(0xffffffffu, redo != 0)) {
         it = 0;
 #pragma unroll 1
-        for (int h = sb * SITES + t.sl; h < g.Vh; h += nb * SITES, it = (it + 1) & 63)
-            if (redo >> it & 1) {
-                const double n2 = fx_redo_site1(P, p, k, h, OUTFX);
-                if (RED) nrm += n2;
-            }
+        for (int h0 = sb * SITES; h0 < g.Vh; h0 += nb * SITES, it = (it + 1) & 63) {
+            const bool mine = h0 + t.sl < g.Vh && (redo >> it & 1);
+            if (!__any_sync(0xffffffffu, mine)) continue;
+            const double n2 = fx_redo_site1(P, p, k, mine ? h0 + t.sl : 0, t.r, mine, OUTFX);
+            if (RED) nrm += n2;
+        }
     }
     pdl_trigger();
     if (RED) grid_reduce(nrm, P.red, k, nb * gridDim.y, sb + nb * blockIdx.y);
 }
 
-inline __device__ __noinline__ double fx_redo_site1(const FxParams& P, int p, int k, int h, int outfx) {
+inline __device__ __noinline__ double fx_redo_site1(const FxParams& P, int p, int k, int h, int r, bool mine, int outfx) {
     const Geom& g = P.g;
     const char* in = P.in.p + (P.full && p == 0 ? P.in.pstep : 0) + k * P.in.rstep;
     const int* ex = reinterpret_cast<const int*>(in + 192LL * g.stride);
@@ -767,7 +771,7 @@ inline __device__ __noinline__ double fx_redo_site1(const FxParams& P, int p, in
     site_of_half(h, p, g, c, s);
     bool bad = false;
 #pragma unroll 1
-    for (int j = 0; j < 8; j++) {
+    for (int j = 4 * r; j < 4 * r + 4; j++) {
         bool wrap;
         const int sn = fx_neighbour(g, c, s, j, wrap), hn = sn >> 1, e = ex[hn];
         const uint4* fl = (j & 1) == 0 ? fx_link_at(P.u, p, j >> 1, s) : fx_link_at(P.u, 1 - p, j >> 1, sn);
@@ -788,16 +792,22 @@ inline __device__ __noinline__ double fx_redo_site1(const FxParams& P, int p, in
                                                                           : fx_link_at(P.un, 1 - p, j >> 1, sn));
         fx_native_hop(v, lk, P.un.word_step, P.un_recon, j >> 1, (j & 1) == 0, P.dag, wrap, g, acc);
     }
-    if (!bad && !outfx) return 0.0;
+#pragma unroll 1
+    for (int q = 0; q < 12; q++) {  // the other thread's hops
+        acc[q].re += __shfl_xor_sync(0xffffffffu, acc[q].re, 16);
+        acc[q].im += __shfl_xor_sync(0xffffffffu, acc[q].im, 16);
+    }
+    bad = __shfl_xor_sync(0xffffffffu, (int)bad, 16) || bad;
+    if (!mine || (!bad && !outfx)) return 0.0;
     if (outfx) {
         char* out = P.out.p + (P.full ? p * P.out.pstep : 0) + k * P.out.rstep;
 #pragma unroll 1
-        for (int q = 0; q < 12; q++)
+        for (int q = 6 * r; q < 6 * r + 6; q++)
             reinterpret_cast<double2*>(out)[h + (long long)q * g.stride] = make_double2(acc[q].re, acc[q].im);
-        fx_exponents(out, g.stride)[h] = 0;
+        if (r == 0) fx_exponents(out, g.stride)[h] = 0;
         return 0.0;
     }
-    return fx_finish_native(P, p, k, s, acc);
+    return fx_finish_native(P, p, k, s, acc, 6 * r, 6 * r + 6);
 }
 
 // Up to 32 sites, h0 to end, of parity p and right-hand side k, by a block of W warps; returns

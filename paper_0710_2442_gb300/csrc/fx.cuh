@@ -17,10 +17,12 @@
 // (mostly its final rounding).
 //
 // Ranges, with the unit of a term at 2^56 = scale: |v.h| <= 2^28, v.l < 2^30 for
-// a component, twice that after the projection's one addition; link entries
-// |u.h| <= 2^28, |u.l| < 2^30.  Six terms: |hh| <= 6 2^57 < 2^60,
-// |mid| <= 12 2^59 < 2^63; eight hops of at most 12 2^56: below 2^63.
-// Fields outside the ranges (a link entry above 1 or a link with no entry above
+// a component, twice that after the projection's one addition and sqrt(2) times more after a
+// boundary phase; link entries |u.h| <= 1.25 2^28, |u.l| < 2^30 (SU(3), and SU(3) over a mean link of 0.8 or
+// more).  Six terms: |hh| < 2^61, |mid| <= 6 2^58 (1.25 + 2.83) < 2^63; a row of a hop
+// sums three products of moduli 1.25 sqrt(2) and 2 sqrt(2) at most, so eight hops give at
+// most 120 2^56 < 2^63.
+// Fields outside the ranges (a link entry above 1.25 or a link with no entry above
 // 1/4, exponents below 2^-423 or above 2^477, Inf, NaN) are reported to the caller, who
 // takes the FP64 stencil for that site.
 #pragma once
@@ -31,8 +33,9 @@ namespace wl {
 
 // exponents (biased) of half spinors that the fixed-point path takes
 constexpr int kFxEmin = 600, kFxEmax = 1500;
-// |hi word| << 1 of a link's largest entry: 0.25 <= max |U_ij| < 1 + 2^-20
-constexpr unsigned kFxLinkLo = 0x3FD00000u << 1, kFxLinkHi = 0x3FF00000u << 1 | 1u;
+// |hi word| << 1 of a link's largest entry: 0.25 <= max |U_ij| < 1.25 + 2^-20
+constexpr unsigned kFxLinkLo = 0x3FD00000u << 1, kFxLinkHi = 0x3FF40000u << 1;
+constexpr int kFxLinkLimb = 5 << 26;  // 1.25 at 2^28
 
 // Right shifts that give 0 for counts of the word length and more.
 __host__ __device__ __forceinline__ unsigned fx_shr32(unsigned v, unsigned s) {

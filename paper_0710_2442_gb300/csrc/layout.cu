@@ -252,8 +252,13 @@ __global__ void pack_gauge_fx_kernel(const double2* __restrict__ canon, char* ba
                 f[k / 3][k % 3] = FxCplx{fx_link(rh, (unsigned)__double2loint(u[k].x)),
                                          fx_link(ih, (unsigned)__double2loint(u[k].y))};
             }
-            if (R == 12) fx_recon_row2(f);
-            if (mx < kFxLinkLo || mx > kFxLinkHi) f[0][0].re.h = (int)kFxBadLink;
+            bool fits = mx >= kFxLinkLo && mx <= kFxLinkHi;
+            if (R == 12) {
+                fx_recon_row2(f);  // a third row of rows that are no SU(3) ones can be larger
+#pragma unroll
+                for (int k = 0; k < 3; k++) fits = fits && abs(f[2][k].re.h) <= kFxLinkLimb && abs(f[2][k].im.h) <= kFxLinkLimb;
+            }
+            if (!fits) f[0][0].re.h = (int)kFxBadLink;
             uint4* b = fx + (size_t)(p * 4 + mu) * 9 * g.stride + h;
 #pragma unroll
             for (int k = 0; k < 9; k++) {

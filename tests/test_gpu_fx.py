@@ -130,3 +130,28 @@ def test_conversions_agree(w, scale):
     three = handle_hop(w, U, np.stack([src, -src, src]), *args, nrhs=3)
     for k, sign in enumerate((1.0, -1.0, 1.0)):
         assert np.array_equal(three[k], handle_hop(w, U, sign * src, *args))
+
+
+@pytest.mark.parametrize("dims", [(4, 2, 4, 6), (12, 14, 16, 16)])
+@pytest.mark.parametrize("case", ["mean link", "all entries", "third row"])
+def test_links_at_the_edge_of_the_range(w, monkeypatch, dims, case):
+    """Entries up to 1.25 stay in fixed point: SU(3) over a mean link of 0.8, and links whose every entry is as large
+    as it may be, with a field that adds all products up; 12-real links whose third row leaves the range do not.
+    Against the FP64 stencil, whose own error is at most 16 roundings of a sum of moduli."""
+    V = inputs.volume(dims)
+    U = inputs.gauge_field(dims, "random", seed=411)
+    src = inputs.gaussian_spinor(V // 2, seed=412)
+    recon = 18
+    if case == "mean link":
+        U = U / 0.8
+    elif case == "all entries":
+        U = np.full_like(U, 1.25 - 1.25j)
+        src = np.full_like(src, 1.0 + 1.0j)
+    else:
+        recon = 12
+        U[..., 0, :] = 0.95 + 0.95j
+        U[..., 1, :] = (0.95 - 0.95j) * np.array([1.0, -1.0, 1.0])
+    args = (w, U, src, dims, PHASES, w.WILSON_F64, recon, 1, 0, w.WILSON_OP_HOP)
+    got = handle_hop(*args)
+    monkeypatch.setenv("WILSON_HOP_VARIANT", "0")
+    assert_parity(got, handle_hop(*args), TOL)
