@@ -41,7 +41,14 @@ __device__ __forceinline__ T* at(const Vec& v, int k) {
 // iteration (16^3 x 32 F16: 51 us an iteration with them).  A kernel's blocks read
 // fields of the scalars that only another kernel writes: the x, s update reads gam and
 // iter, and leaves copies (gam2, iter2) that the p update reads when it writes
-// the new ones; done is written to what every block finds for itself.
+// the new ones.  done is the exception: the first block writes it, to what every block finds
+// for itself, while blocks that start later test it.  Such a block may see either value, so
+// its threads leave on one decision (finished).
+
+// Whether the right-hand side was done, the same for the whole block: a thread that tested
+// the flag by itself could leave while others of its block, which read it a moment
+// before, stay for the sums and the barriers.
+__device__ __forceinline__ bool finished(const CGScalars& C) { return __syncthreads_or(__ldcg(&C.done)) != 0; }
 
 // x += alpha p,  s -= alpha q,  [s_low = s],  partials of |s|^2; alpha = gam / |q|^2 from
 // the nq partials of q.
@@ -50,7 +57,7 @@ __global__ void __launch_bounds__(256) cg_xs_kernel(Vec x, Vec p, Vec s, Vec q, 
                                                     CGScalars* sc, RedArgs qred, int nq, RedArgs red) {
     const RhsIdx r = rhs_index(nrhs);
     CGScalars& C = sc[r.k];
-    if (__ldcg(&C.done)) return;
+    if (finished(C)) return;
     using TX = typename SpinorFmt<XP>::real;
     using TP = typename SpinorFmt<PP>::real;
     char* X = at<char>(x, r.k);
@@ -146,7 +153,7 @@ __global__ void __launch_bounds__(256) cg_p_end_kernel(Vec p, Vec rv, Geom g, in
         for (int k = 1; k < nrhs; k++) go |= __ldcg(&sc[k].done) == 0;
         cudaGraphSetConditional(loop.handle, go);
     };
-    if (__ldcg(&C.done)) {
+    if (finished(C)) {
         condition(false);
         return;
     }

@@ -259,3 +259,26 @@ def test_fp32_outer_residuals(w, oracle_mod, inner):
     xh = host(xs)
     for k in range(3):
         assert true_resid(oracle_mod, U, xh[k], bs[k], dims, kappa) <= 1.1e-10
+
+
+@pytest.mark.parametrize("inner", ["f16", "f32"])
+def test_lockstep_solve_repeats_itself(w, inner):
+    """Kernels of a 12-right-hand-side iteration run in several waves (12 x 144 blocks of 256
+    threads), with blocks of a right-hand side starting while its first block
+    records that it has finished: every run takes the same iterations and gives the same bits.
+    The sources span scales and shapes, so that they finish at different times."""
+    dims, kappa = (24, 16, 12, 16), 0.13
+    U = dev(inputs.gauge_field(dims, "weak", eps=0.3, seed=250))
+    b = inputs.gaussian_spinor(dims, seed=251, nrhs=12)
+    b[3] = 0
+    b[5:9] = inputs.point_sources(dims, site=9)[:4]
+    db = dev(b)
+    runs = []
+    for _ in range(4):
+        x = dev(np.zeros_like(b))
+        rc, st = w.wilson_cg_solve_multi(x, U, db, 12, w.lattice(dims), kappa, w.solver_defaults(w.PREC[inner]))
+        assert rc == 0
+        runs.append((host(x), [s["inner_iters"] for s in st], st[0]["outer_iters"]))
+    for x, it, outer in runs[1:]:
+        assert it == runs[0][1] and outer == runs[0][2]
+        assert np.array_equal(x, runs[0][0])
