@@ -633,7 +633,7 @@ void with_nbm(int nbm, F&& f) {
 
 }  // namespace
 
-BlockInner::BlockInner(Prec ip, Prec xp, const Geom& g, int nrhs) : ip_(ip), xp_(xp), g_(g), nr_(nrhs) {
+BlockInner::BlockInner(Prec ip, Prec xp, const Geom& g, int nrhs, cudaStream_t st) : ip_(ip), xp_(xp), g_(g), nr_(nrhs) {
     WL_REQUIRE(nrhs >= 1 && nrhs <= kBlockMax, "block CG takes at most 16 right-hand sides");
     nbm_ = nrhs <= 4 ? 4 : nrhs <= 8 ? 8 : nrhs <= 12 ? 12 : 16;
     const int spb = kBThreads / nbm_;
@@ -643,8 +643,9 @@ BlockInner::BlockInner(Prec ip, Prec xp, const Geom& g, int nrhs) : ip_(ip), xp_
     partials_.alloc(sizeof(double) * 2 * (size_t)kBlockMax * kBlockMax * grid_);
     counter_.alloc(sizeof(unsigned int));
     skip_.alloc(sizeof(int) * nrhs);
-    WL_CUDA(cudaMemset(counter_.p, 0, sizeof(unsigned int)));
-    WL_CUDA(cudaMemset(state_.p, 0, sizeof(BCGState)));
+    // on st: the buffers may come from its pool, where they are this solve's only in its order
+    WL_CUDA(cudaMemsetAsync(counter_.p, 0, sizeof(unsigned int), st));
+    WL_CUDA(cudaMemsetAsync(state_.p, 0, sizeof(BCGState), st));
 }
 
 BlockInner::~BlockInner() {

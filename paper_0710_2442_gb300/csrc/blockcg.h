@@ -26,7 +26,7 @@ struct BCGState;
 // its search directions (the block form of a reliable update).
 class BlockInner {
 public:
-    BlockInner(Prec ip, Prec xp, const Geom& g, int nrhs);
+    BlockInner(Prec ip, Prec xp, const Geom& g, int nrhs, cudaStream_t st);
     ~BlockInner();
     BlockInner(const BlockInner&) = delete;
     BlockInner& operator=(const BlockInner&) = delete;

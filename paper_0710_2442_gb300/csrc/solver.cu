@@ -238,7 +238,7 @@ std::vector<SolveStats> cg_solve_prepared(SpinorField& x, const SpinorField& b, 
     Inner in;
     in.alloc(prm.inner, g, nr);
     std::unique_ptr<BlockInner> blk;
-    if (prm.block_cg && nr > 1) blk = std::make_unique<BlockInner>(in.ip, in.xp, g, nr);
+    if (prm.block_cg && nr > 1) blk = std::make_unique<BlockInner>(in.ip, in.xp, g, nr, st);
     // The block's own reduction per correction: the caller's delta, else a
     // conservative default (longer block runs in reduced precision lose the
     // orthogonality of their residual basis).

@@ -282,3 +282,29 @@ def test_lockstep_solve_repeats_itself(w, inner):
     for x, it, outer in runs[1:]:
         assert it == runs[0][1] and outer == runs[0][2]
         assert np.array_equal(x, runs[0][0])
+
+
+def test_block_cg_beside_a_busy_default_stream(w):
+    """A solve's set-up is ordered on its own stream alone: work queued on the legacy default
+    stream, which the solve does not wait for, changes nothing."""
+    import torch
+    dims, kappa = (4, 4, 4, 8), 0.1350
+    U = dev(inputs.gauge_field(dims, "weak", eps=0.3, seed=252))
+    b = dev(inputs.gaussian_spinor(dims, seed=253, nrhs=4))
+    L = w.lattice(dims)
+    p = w.solver_defaults(w.WILSON_F32)
+    p.block_cg = 1
+    side = torch.cuda.Stream()
+    load = torch.ones(2048, 2048, device="cuda")
+    runs = []
+    for busy in (False, True, True):
+        x = torch.zeros_like(b)
+        torch.cuda.synchronize()
+        if busy:
+            for _ in range(200):
+                load @ load
+        rc, st = w.wilson_cg_solve_multi(x, U, b, 4, L, kappa, p, stream=side)
+        assert rc == 0
+        runs.append((host(x), [s["inner_iters"] for s in st]))
+    for x, it in runs[1:]:
+        assert it == runs[0][1] and np.array_equal(x, runs[0][0])
