@@ -1,13 +1,14 @@
 // reduce.cuh -- deterministic FP64 global reductions fused into kernels.
 //
-// Every block reduces its threads' FP64 values by warp shuffles and a
-// shared-memory pass, writes one partial per block, and takes a ticket from a
-// global counter.  The block that draws the last ticket sums all partials in
-// a fixed order (thread t adds partials t, t+B, ...; then the same shuffle
-// tree), so the result does not depend on block scheduling, and then runs
-// the finisher that turns the sum into solver scalars.  It also resets the
-// counter, so the same reducer can be reused by the next launch on the
-// stream.  No block ever waits for another one.
+// Every block sums its threads' FP64 values (block_sum: integers of a common
+// scale, rounded once) and writes one partial.  Who adds the partials up:
+//  - FIN_PARTIAL: the blocks of the kernel that uses the sum, all the same way
+//    (sum_partials; the CG iterations, blas.cu);
+//  - else a ticket from a global counter decides: the block that draws the last
+//    one sums all partials in a fixed order (thread t adds partials t, t+B, ...;
+//    then block_sum), runs the finisher that turns the sum into solver scalars,
+//    and resets the counter for the next launch on the stream.
+// No result depends on block scheduling, and no block ever waits for another one.
 #pragma once
 
 #include "common.cuh"
@@ -71,12 +72,43 @@ inline __device__ __noinline__ double block_sum_fp64(double v) {
     return v;
 }
 
+// A term of block_sum_of: the value >= 0 with words hi, lo in units of 2^(e - 1023 - 61), to nearest;
+// e: the largest term's exponent field, 128 or more.  At most 2^62.
+__host__ __device__ __forceinline__ unsigned long long sum_term(unsigned hi, unsigned lo, int e) {
+    const unsigned mh = (hi & 0xFFFFFu) | (hi >> 20 ? 0x100000u : 0u);
+    int t = 2 + e - (int)(hi >> 20);  // from the top of 64 bits
+    t = t < 65 ? t : 65;
+    const unsigned long long y = ((unsigned long long)mh << 32 | lo) << 10;  // half of that
+    return ((y >> (t - 2)) + 1) >> 1;
+}
+// The bits of the double nearest to (s2 2^42 + s1 2^21 + s0) 2^(e - 1023 - 61), a sum of at
+// most 2048 terms (s2 <= 2^31, s1 and s0 < 2^32) of which one is 2^61 or more.
+__host__ __device__ __forceinline__ unsigned long long sum_bits(unsigned s2, unsigned s1, unsigned s0, int e) {
+    const unsigned long long a = ((unsigned long long)s2 << 21) + s1 + (s0 >> 21);  // 2^40 .. 2^52
+    const unsigned r = s0 & 0x1FFFFFu;                                             // the sum is a 2^21 + r
+#ifdef __CUDA_ARCH__
+    const int n = __clzll((long long)a);
+#else
+    const int n = __builtin_clzll(a);
+#endif
+    const bool more = n < 21 && (r & ((1u << (21 - n)) - 1));
+    const unsigned long long m = a << n | ((unsigned long long)r << 43) >> (64 - n) | (more ? 1u : 0u);
+    const unsigned long long q = m >> 11;  // 53 bits; the others round, to nearest even
+    const unsigned up = ((unsigned)m & 0x7FFu) + ((unsigned)q & 1) > 0x400u;
+    const int field = e + 23 - n;  // of the result, before the rounding
+    if (field >= 2047) return 0x7FFULL << 52;
+    return q + up + ((unsigned long long)(field - 1) << 52);  // q's leading bit adds 1 to the field
+}
+
 // Sum over the block of N values >= 0 a thread; valid in thread 0.  An FP64 addition
 // takes the FP64 pipe 64 cycles, and a shuffle tree is ten of them in a row.
 // Here the values become integers of 62 bits below the block's largest
 // exponent, in three limbs that are added per thread and then by a warp with one
-// instruction each (redux), so a term is off by less than 2^-62 of the largest one and the
-// sum is rounded to FP64 once.  Zeros, tiny values, Inf and NaN take the FP64 additions.
+// instruction each (redux); the sum is rounded to FP64 once.  A term within 2^-9 of the
+// largest one is exact, a smaller one is rounded to 2^-62 of the scale: a single value comes
+// back as it is, and a sum of n terms is off by at most half a unit in its last place and
+// n 2^-62 of its largest term (a tree of FP64 additions: half a unit at each of its levels).
+// Zeros, tiny values, Inf and NaN take the FP64 additions.
 // A limb's sum fits 32 bits: 21 bits, N blockDim <= 2048 values.
 template <int N>
 __device__ __forceinline__ double block_sum_of(const double (&v)[N]) {
@@ -102,10 +134,7 @@ __device__ __forceinline__ double block_sum_of(const double (&v)[N]) {
     unsigned l[3] = {0, 0, 0};
 #pragma unroll
     for (int i = 0; i < N; i++) {
-        const unsigned hi = (unsigned)__double2hiint(v[i]), lo = (unsigned)__double2loint(v[i]);
-        const unsigned mh = (hi & 0xFFFFFu) | (hi >> 20 ? 0x100000u : 0u);
-        const int t = min(2 + e - (int)(hi >> 20), 63);
-        const unsigned long long n = ((unsigned long long)mh << 32 | lo) << 11 >> t;  // below 2^62
+        const unsigned long long n = sum_term((unsigned)__double2hiint(v[i]), (unsigned)__double2loint(v[i]), e);
         l[0] += (unsigned)n & 0x1FFFFFu;
         l[1] += (unsigned)(n >> 21) & 0x1FFFFFu;
         l[2] += (unsigned)(n >> 42);
@@ -118,15 +147,9 @@ __device__ __forceinline__ double block_sum_of(const double (&v)[N]) {
     }
     __syncthreads();
     if (warp != 0) return 0.0;
-    unsigned long long s[3];
 #pragma unroll
-    for (int k = 0; k < 3; k++) s[k] = __reduce_add_sync(0xffffffffu, lane < nwarps ? sl[k][lane] : 0u);
-    // s2 2^42 + s1 2^21 + s0 in units of 2^(e - 1023 - 61)
-    const unsigned long long q = (s[2] << 31) + (s[1] << 10) + (s[0] >> 11);
-    // q 2^11 as a double with two FP64 additions: its words under the exponents of 2^84 and 2^52
-    const double a = __hiloint2double(0x45300000, (int)(unsigned)(q >> 32)), b = __hiloint2double(0x43300000, (int)(unsigned)q);
-    const double r = (a - __hiloint2double(0x45300000, 0x00100000)) + b;  // 2^84 + 2^52
-    return r * __hiloint2double((e - 61 + 11) << 20, 0);
+    for (int k = 0; k < 3; k++) l[k] = __reduce_add_sync(0xffffffffu, lane < nwarps ? sl[k][lane] : 0u);
+    return __longlong_as_double((long long)sum_bits(l[2], l[1], l[0], e));
 }
 __device__ inline double block_sum(double v) {
     const double one[1] = {v};
