@@ -10,6 +10,21 @@ namespace bt {
 // kernel's work).  The FP64 stencil it replaces took 128 us for a 16^3 x 32
 // problem's hop on its FP64 arithmetic, and a correction waits for two of them; F16 batch of
 // 8 x 8^4, 4 x 12^4 and 2 x 16^3 x 32 problems 23.4 -> 19.6 ms.
+// Not inline: a call to fx_redo inside a loop costs the loop spills.
+__device__ __noinline__ void bhop_fx_tile(const FxParams& P, FxTile& T, int p, int h0, int h1) {
+    __shared__ unsigned redo[16];  // of the tile's groups (at most 512 sites)
+    unsigned any = 0;
+    double none = 0.0;
+    for (int h = h0; h < h1; h += 32) {
+        const unsigned m = fx_tile<true, false, 4>(P, T, p, 0, h, h1, none);
+        if (threadIdx.x == 0) redo[(h - h0) >> 5] = m;
+        any |= m;
+        __syncthreads();
+    }
+    if (!any) return;
+    for (int h = h0; h < h1; h += 32) fx_tile_redo<4>(P, T, p, 0, h, redo[(h - h0) >> 5]);
+}
+
 __global__ void __launch_bounds__(128, 4) bhop_fx_kernel(const BatchArgs A, const BOp op) {
     __shared__ FxTile T;
     __shared__ FxParams P;
@@ -35,6 +50,7 @@ __global__ void __launch_bounds__(128, 4) bhop_fx_kernel(const BatchArgs A, cons
             const long long s = stride;
             P.out = FxField{out, 0, 0, 1, stride, 0};
             P.in = FxField{Pr.f[op.f_in] + (1 - p) * Pr.fp[op.f_in], 0, 0, 1, stride, 0};
+            P.nat = P.in;
             P.x = FxField{const_cast<char*>(x), 0, 0, 1, stride, 0};
             P.u = FxLinks{Pr.g64, 36 * s, 9 * s, 1, stride, 0};
             P.un = FxLinks{Pr.canon, 0, 9, 36, 1, 1};
@@ -48,7 +64,7 @@ __global__ void __launch_bounds__(128, 4) bhop_fx_kernel(const BatchArgs A, cons
             P.scaled = !x && op.coef != 0;
         }
         __syncthreads();
-        for (int h = h0; h < h1; h += 32) fx_tile<true, false, 4>(P, T, p, 0, h, h1);
+        bhop_fx_tile(P, T, p, h0, h1);
     }
 }
 

@@ -56,6 +56,7 @@ int launch_hop_fx(const HopLaunch& L, cudaStream_t st) {
     WL_REQUIRE(!L.canon || nrhs == 1, "canonical fields: one right-hand side");
     P.out = L.canon & kCanonOut ? canonical(L.out, L.full) : soa(L.out, L.full ? L.out_pstep : 0, L.out_rstep, g.stride);
     P.in = L.canon & kCanonIn ? canonical(L.in, L.full) : soa(L.in, L.full ? L.in_pstep : 0, L.in_rstep, g.stride);
+    P.nat = P.in;
     P.x = L.canon & kCanonX ? canonical(L.x, L.full) : soa(L.x, L.full ? L.x_pstep : 0, L.x_rstep, g.stride);
     P.u = FxLinks{gf.fx.as<const char>(), 36 * s, 9 * s, 1, g.stride, 0};
     P.un_recon = gf.recon;
@@ -97,6 +98,7 @@ int launch_hop_fx(const HopLaunch& L, cudaStream_t st) {
     }
     if (L.fx_in) {
         P.in = soa(L.fx_in, L.full ? L.fx_pstep : 0, L.fx_rstep, g.stride);
+        P.nat.p = nullptr;  // the hop that wrote it left the sites out of range as doubles
     } else {
         launch_dep(fx_pack_kernel, dim3((g.Vh + 127) / 128 * nrhs, ny), dim3(128), st, P.in,
                    static_cast<char*>(L.fx_tmp), L.fx_pstep, L.fx_rstep, nrhs, 0, ny, g, L.skip, L.skip_stride);

@@ -51,8 +51,9 @@ struct FxLinks {
 
 struct FxParams {
     FxField out, in, x;
-    FxLinks u;   // the links the kernel reads: doubles, or fixed point (FXL)
-    FxLinks un;  // the same links as doubles, for sites out of the fixed-point ranges
+    FxField nat;  // the input as doubles, for sites done over in FP64 (p null: in, fixed point with some doubles)
+    FxLinks u;    // the links the kernel reads: doubles, or fixed point (FXL)
+    FxLinks un;   // the same links as doubles, for those sites
     int un_recon;  // of 12 or 18 reals
     Geom g;
     int nrhs, skip_stride, out_parity, full, xpay, dag;
@@ -89,11 +90,11 @@ __device__ __forceinline__ unsigned fx_max2(unsigned m, const uint4& d) { return
 __device__ __forceinline__ unsigned fx_nonzero(const uint4& d) { return d.x | d.y << 1 | d.z | d.w << 1; }
 
 // Half-spin row r of the projected neighbour, in units of its own largest
-// exponent, which is returned (0: out of range).  The projector's partner spin
-// comes in with factor sigma, times i for IMAG; cj = -1 gives the complex
-// conjugate of the row.
+// exponent, which is returned (0: out of range; kFxZero: both spins are zero).  The projector's partner spin
+// comes in with factor sigma, times i for IMAG; the row comes times sg = +-1.
+constexpr int kFxZero = kFxEmin - 1;
 template <bool IMAG>
-__device__ __forceinline__ int fx_project(const uint4* psi, int ws, int r, int partner, int sigma, int cj,
+__device__ __forceinline__ int fx_project(const uint4* psi, int ws, int r, int partner, int sigma, int sg,
                                           FxCplx h[3]) {
     uint4 p[3], q[3];
 #pragma unroll
@@ -109,10 +110,10 @@ __device__ __forceinline__ int fx_project(const uint4* psi, int ws, int r, int p
         unsigned nz = 0;
 #pragma unroll
         for (int c = 0; c < 3; c++) nz |= fx_nonzero(p[c]) | fx_nonzero(q[c]);
-        e = nz ? 0 : kFxEmin;
+        e = nz ? 0 : kFxZero;
     }
     const unsigned ew = fx_scale_word(e + kFxOffSpinor);
-    const int sre = IMAG ? -sigma : sigma, sim = cj * sigma;  // i q = (-q.im, q.re)
+    const int sre = sg * (IMAG ? -sigma : sigma), sim = sg * sigma;  // i q = (-q.im, q.re)
 #pragma unroll
     for (int c = 0; c < 3; c++) {
         const unsigned ah = IMAG ? q[c].w : q[c].y, al = IMAG ? q[c].z : q[c].x;
@@ -120,22 +121,22 @@ __device__ __forceinline__ int fx_project(const uint4* psi, int ws, int r, int p
         const FxMag pr = fx_mag(p[c].y, p[c].x, fx_shift(ew, p[c].y << 1));
         const FxMag pi = fx_mag(p[c].w, p[c].z, fx_shift(ew, p[c].w << 1));
         const FxMag a = fx_mag(ah, al, fx_shift(ew, ah << 1)), b = fx_mag(bh, bl, fx_shift(ew, bh << 1));
-        const int spr = fx_sign(p[c].y, 1), spi = fx_sign(p[c].w, cj), sa = fx_sign(ah, sre), sb = fx_sign(bh, sim);
+        const int spr = fx_sign(p[c].y, sg), spi = fx_sign(p[c].w, sg), sa = fx_sign(ah, sre), sb = fx_sign(bh, sim);
         h[c].re = FxReal{a.h * sa + pr.h * spr, a.l * sa + pr.l * spr};
         h[c].im = FxReal{b.h * sb + pi.h * spi, b.l * sb + pi.l * spi};
     }
     return e;
 }
 
-// w_i = sum_k u_k h_k; nim: the negated imaginary parts of h
-__device__ __forceinline__ longlong2 fx_row(const FxCplx u[3], const FxCplx h[3], const FxReal nim[3]) {
+// w_i = sum_k u_k h_k, or with x, y in place of -Im h and Re h
+__device__ __forceinline__ longlong2 fx_row(const FxCplx u[3], const FxCplx h[3], const FxReal x[3], const FxReal y[3]) {
     FxAcc re = fx_zero(), im = fx_zero();
 #pragma unroll
     for (int k = 0; k < 3; k++) {
         fx_mac(re, u[k].re, h[k].re);
-        fx_mac(re, u[k].im, nim[k]);
+        fx_mac(re, u[k].im, x[k]);
         fx_mac(im, u[k].re, h[k].im);
-        fx_mac(im, u[k].im, h[k].re);
+        fx_mac(im, u[k].im, y[k]);
     }
     return make_longlong2(fx_sum(re), fx_sum(im));
 }
@@ -163,16 +164,18 @@ __device__ __forceinline__ void fx_wrap(double pr, double pi, FxCplx (&h)[3]) {
 }
 
 // Shared memory of a tile: the hops' half spinors [hop][row][colour][lane],
-// their exponents [hop][row][lane] and the lanes to be redone in FP64.
+// their exponents [hop][row][lane] and the lanes to be done over in FP64, whose
+// products take the place of w.
 struct FxTile {
     longlong2 w[8][2][3][32];
     int e[8][2][32];
     int bad[32];
 };
 
-// Hop j of one site.  A backward hop needs U^dag h = conj(U^T conj(h)): it
-// conjugates the half spinor in the projection and reads the link transposed;
-// the outer conjugation is left to fx_spin.
+// Hop j of one site; a backward hop reads the link transposed and conjugated.  What is
+// stored is w in x and y, -w in z and t: fx_spin cuts the contributions off at 2^-56 where it
+// aligns them, and with these signs each output component adds four and subtracts four of
+// the eight, so that what is cut off has no mean (rounding them instead: 12^4 Schur 24.3 -> 25.9 us).
 template <bool FXL>
 __device__ __forceinline__ void fx_hop(const FxParams& P, FxTile& T, int j, int p, int k, const int c[4], int s,
                                        int lane) {
@@ -182,17 +185,15 @@ __device__ __forceinline__ void fx_hop(const FxParams& P, FxTile& T, int j, int 
     const int sn = fx_neighbour(P.g, c, s, j, wrap);
     const uint4* psi = fx_at(P.in, 1 - p, k, sn);
     const uint4* lk = fwd ? fx_link_at(P.u, p, mu, s) : fx_link_at(P.u, 1 - p, mu, sn);
-    const int S = fwd != (P.dag != 0) ? 1 : -1, cj = fwd ? 1 : -1;
+    const int S = fwd != (P.dag != 0) ? 1 : -1, sg = mu < 2 ? 1 : -1, f = fwd ? 1 : -1;
     // (1 - S g_mu) psi, row r (project() in dslash_impl.cuh)
-    auto project = [&](int r, FxCplx (&h)[3], FxReal (&nim)[3]) {
+    auto project = [&](int r, FxCplx (&h)[3]) {
         const int e = mu == 0 || mu == 2
                           ? fx_project<true>(psi, P.in.word_step, r, (mu == 0) == (r == 0) ? 3 : 2,
-                                             mu == 2 && r == 1 ? S : -S, cj, h)
+                                             mu == 2 && r == 1 ? S : -S, sg, h)
                           : fx_project<false>(psi, P.in.word_step, r, (mu == 1) == (r == 0) ? 3 : 2,
-                                              mu == 1 && r == 0 ? S : -S, cj, h);
-        if (wrap) fx_wrap(P.g.ph[mu][0], P.g.ph[mu][1], h);  // conj(eta) on h is eta on conj(h)
-#pragma unroll
-        for (int q = 0; q < 3; q++) nim[q] = fx_neg(h[q].im);
+                                              mu == 1 && r == 0 ? S : -S, sg, h);
+        if (wrap) fx_wrap(P.g.ph[mu][0], f * P.g.ph[mu][1], h);
         T.e[j][r][lane] = e;
         return e == 0;
     };
@@ -204,8 +205,13 @@ __device__ __forceinline__ void fx_hop(const FxParams& P, FxTile& T, int j, int 
 #pragma unroll 1
         for (int r = 0; r < 2; r++) {
             FxCplx h[3];
-            FxReal nim[3];
-            bad |= project(r, h, nim);
+            FxReal x[3], y[3];
+            bad |= project(r, h);
+#pragma unroll
+            for (int q = 0; q < 3; q++) {
+                x[q] = FxReal{h[q].im.h * -f, h[q].im.l * -f};
+                y[q] = FxReal{h[q].re.h * f, h[q].re.l * f};
+            }
 #pragma unroll
             for (int i = 0; i < 3; i++) {
                 FxCplx u[3];
@@ -215,14 +221,21 @@ __device__ __forceinline__ void fx_hop(const FxParams& P, FxTile& T, int j, int 
                     u[q] = FxCplx{FxReal{(int)d.x, (int)d.y}, FxReal{(int)d.z, (int)d.w}};
                 }
                 if (i == 0) bad |= (unsigned)u[0].re.h == kFxBadLink;
-                T.w[j][r][i][lane] = fx_row(u, h, nim);
+                T.w[j][r][i][lane] = fx_row(u, h, x, y);
             }
         }
     } else {
         FxCplx h[2][3];
-        FxReal nim[2][3];
+        FxReal x[2][3], y[2][3];
 #pragma unroll
-        for (int r = 0; r < 2; r++) bad |= project(r, h[r], nim[r]);
+        for (int r = 0; r < 2; r++) {
+            bad |= project(r, h[r]);
+#pragma unroll
+            for (int q = 0; q < 3; q++) {
+                x[r][q] = fx_neg(h[r][q].im);
+                y[r][q] = h[r][q].re;
+            }
+        }
         unsigned mx = 0;
         const int wi = fwd ? 3 : 1, wk = fwd ? 1 : 3;
 #pragma unroll
@@ -232,22 +245,23 @@ __device__ __forceinline__ void fx_hop(const FxParams& P, FxTile& T, int j, int 
             for (int q = 0; q < 3; q++) {
                 const uint4 d = __ldg(lk + (long long)(i * wi + q * wk) * ws);
                 mx = fx_max2(mx, d);
-                u[q] = FxCplx{fx_link(d.y, d.x), fx_link(d.w, d.z)};
+                u[q] = FxCplx{fx_link(d.y, d.x, 1), fx_link(d.w, d.z, f)};
             }
 #pragma unroll
-            for (int r = 0; r < 2; r++) T.w[j][r][i][lane] = fx_row(u, h[r], nim[r]);
+            for (int r = 0; r < 2; r++) T.w[j][r][i][lane] = fx_row(u, h[r], x[r], y[r]);
         }
-        bad |= mx < kFxLinkLo || mx > kFxLinkHi;
+        bad |= mx > kFxLinkHi;
     }
     if (bad) T.bad[lane] = 1;
 }
 
 // N colours from C0 on of output spin SPIN: the eight hops' contributions (expand()
-// in dslash_impl.cuh) aligned to their largest exponent.  The sums become doubles with integer instructions
+// in dslash_impl.cuh) aligned to their largest exponent; returns whether a component is below
+// the guard (fx.cuh).  The sums become doubles with integer instructions
 // (INT) where a block is one of several on an SM: 12^4 F64 Schur 24.7 -> 24.0 us; one block of
 // eight warps on an SM is as fast or faster with the FP64 additions (8^4 hop 6.42 against 6.49 us).
 template <int SPIN, bool INT, int N>
-__device__ __forceinline__ void fx_spin(const FxTile& T, int c0, int dag, int lane, double2 (&v)[N]) {
+__device__ __forceinline__ bool fx_spin(const FxTile& T, int c0, int dag, int lane, double2 (&v)[N]) {
     constexpr bool lower = SPIN >= 2;
     // half-spin row of hop direction mu: SPIN itself, or for spin 2 rows 1, 1, 0, 0 and for spin 3 rows 0, 0, 1, 1
     auto row = [](int j) { return lower ? ((SPIN == 2) == (j < 4) ? 1 : 0) : SPIN; };
@@ -258,29 +272,36 @@ __device__ __forceinline__ void fx_spin(const FxTile& T, int c0, int dag, int la
         top = max(top, e[j]);
     }
 #pragma unroll
-    for (int j = 0; j < 8; j++) e[j] = min(top - e[j], 63);
+    for (int j = 0; j < 8; j++) e[j] = min(top - e[j], kFxMaxShift);
     const int k2 = top + 1 - 1023 - 56;
     const FxBias bias = fx_bias(k2);
+    bool below = false;
 #pragma unroll
     for (int c = 0; c < N; c++) {
         long long re = 0, im = 0;
+        unsigned nr = 0, ni = 0;
 #pragma unroll
         for (int j = 0; j < 8; j++) {
             const longlong2 w = T.w[j][row(j)][c0 + c][lane];
-            const long long x = fx_sar(w.x, e[j]), y = fx_sar(w.y, e[j]);  // backward: conj(w)
+            const long long x = fx_align(w.x, e[j]), y = fx_align(w.y, e[j]);
             // upper: w.  Lower, with S = +1 forward and -1 backward: S i w (x), spin 2: -S w (y),
-            // S i w (z), -S w (t); spin 3: S i w, S w, -S i w, -S w
+            // S i w (z), -S w (t); spin 3: S i w, S w, -S i w, -S w.  In z and t the stored one is -w.
             const int mu = j >> 1;
             const bool bwd = (j & 1) != 0, times_i = lower && (mu == 0 || mu == 2);
-            const bool flip = lower && (bwd != (mu == 3 || (mu == 1 && SPIN == 2) || (mu == 2 && SPIN == 3)));
+            const bool flip = (mu >= 2) != (lower && (bwd != (mu == 3 || (mu == 1 && SPIN == 2) || (mu == 2 && SPIN == 3))));
             if (times_i) {  // i (x + i y)
-                re = (flip == bwd) ? re - y : re + y;
+                re = flip ? re + y : re - y;
                 im = flip ? im - x : im + x;
+                nr = fx_modulus(y, nr);
+                ni = fx_modulus(x, ni);
             } else {
                 re = flip ? re - x : re + x;
-                im = (flip != bwd) ? im - y : im + y;
+                im = flip ? im - y : im + y;
+                nr = fx_modulus(x, nr);
+                ni = fx_modulus(y, ni);
             }
         }
+        below = below || min(nr, ni) < kFxGuard << 16;
         if (lower && dag) {
             re = -re;
             im = -im;
@@ -288,58 +309,19 @@ __device__ __forceinline__ void fx_spin(const FxTile& T, int c0, int dag, int la
         v[c] = INT ? make_double2(fx_double_int(re, k2), fx_double_int(im, k2))
                    : make_double2(fx_double(re, bias), fx_double(im, bias));
     }
+    return below && top != kFxZero;
 }
 
 template <bool INT, int N>
-__device__ __forceinline__ void fx_spin_of(const FxTile& T, int spin, int c0, int dag, int lane, double2 (&v)[N]) {
+__device__ __forceinline__ bool fx_spin_of(const FxTile& T, int spin, int c0, int dag, int lane, double2 (&v)[N]) {
     switch (spin) {
-        case 0: fx_spin<0, INT>(T, c0, dag, lane, v); break;
-        case 1: fx_spin<1, INT>(T, c0, dag, lane, v); break;
-        case 2: fx_spin<2, INT>(T, c0, dag, lane, v); break;
-        default: fx_spin<3, INT>(T, c0, dag, lane, v); break;
+        case 0: return fx_spin<0, INT>(T, c0, dag, lane, v);
+        case 1: return fx_spin<1, INT>(T, c0, dag, lane, v);
+        case 2: return fx_spin<2, INT>(T, c0, dag, lane, v);
+        default: return fx_spin<3, INT>(T, c0, dag, lane, v);
     }
 }
 
-// A hop of the FP64 stencil (a link or field out of the fixed-point ranges).
-inline __device__ __noinline__ void fx_native_hop(const cpx<double> v[12], const double2* lk, int ws, int recon, int mu, bool fwd,
-                                           int dag, bool wrap, const Geom& g, cpx<double> acc[12]) {
-    cpx<double> h[6], w[6], U[3][3];
-#pragma unroll
-    for (int q = 0; q < 9; q++)
-        if (q < recon / 2) {
-            const double2 d = __ldg(lk + (long long)q * ws);
-            U[q / 3][q % 3] = {d.x, d.y};
-        }
-    if (recon == 12) recon_row2(U);
-    const bool plus = fwd != (dag != 0);
-    switch (mu * 2 + (plus ? 0 : 1)) {
-        case 0: project<0, 1>(v, h); break;
-        case 1: project<0, -1>(v, h); break;
-        case 2: project<1, 1>(v, h); break;
-        case 3: project<1, -1>(v, h); break;
-        case 4: project<2, 1>(v, h); break;
-        case 5: project<2, -1>(v, h); break;
-        case 6: project<3, 1>(v, h); break;
-        default: project<3, -1>(v, h); break;
-    }
-    if (wrap) {
-        const cpx<double> eta = {g.ph[mu][0], fwd ? g.ph[mu][1] : -g.ph[mu][1]};
-#pragma unroll
-        for (int q = 0; q < 6; q++) h[q] = cmul(eta, h[q]);
-    }
-    if (fwd) su3_mul<false>(U, h, w);
-    else su3_mul<true>(U, h, w);
-    switch (mu * 2 + (plus ? 0 : 1)) {
-        case 0: expand<0, 1, false>(acc, w, 1.0); break;
-        case 1: expand<0, -1, false>(acc, w, 1.0); break;
-        case 2: expand<1, 1, false>(acc, w, 1.0); break;
-        case 3: expand<1, -1, false>(acc, w, 1.0); break;
-        case 4: expand<2, 1, false>(acc, w, 1.0); break;
-        case 5: expand<2, -1, false>(acc, w, 1.0); break;
-        case 6: expand<3, 1, false>(acc, w, 1.0); break;
-        default: expand<3, -1, false>(acc, w, 1.0); break;
-    }
-}
 // v = a v, or x + a v, of N words from word0 on, and out = v.  Branches, not
 // predicated instructions: the FP64 pipe takes 64 cycles for either.
 template <int N>
@@ -371,57 +353,131 @@ __device__ __forceinline__ double fx_norm(const double2 (&v)[N]) {
     return n;
 }
 
-// The output of a site computed that way; returns its squared modulus.
-inline __device__ __noinline__ double fx_finish_native(const FxParams& P, int p, int k, int s, const cpx<double> acc[12], int q0,
-                                                        int q1) {
-    uint4* out = const_cast<uint4*>(fx_at(P.out, p, k, s));
-    const uint4* x = P.xpay ? fx_at(P.x, p, k, s) : nullptr;
-    double n2 = 0.0;
-#pragma unroll 1
-    for (int q = q0; q < q1; q++) {
-        double2 v[1] = {make_double2(acc[q].re, acc[q].im)};
-        fx_finish(P, out, x, q, v);
-        n2 += fx_norm(v);
-    }
-    return n2;
+__device__ __forceinline__ const int* fx_exponents(const char* f, long long stride) {
+    return reinterpret_cast<const int*>(f + 192 * stride);
+}
+__device__ __forceinline__ int* fx_exponents(char* f, long long stride) { return reinterpret_cast<int*>(f + 192 * stride); }
+constexpr int kFxExpMask = 0xFFF;  // of a word of them; bits 12 to 15: the spins with a nonzero component
+
+__device__ __forceinline__ double fx_flip(double v, int neg) {
+    return __hiloint2double(__double2hiint(v) ^ neg << 31, __double2loint(v));
 }
 
-// One site of fields in doubles on the FP64 stencil, output included.
-inline __device__ __noinline__ double fx_redo_site(const FxParams& P, int p, int k, int h) {
-    cpx<double> acc[12];
-#pragma unroll 1
-    for (int q = 0; q < 12; q++) acc[q] = cpx<double>{0.0, 0.0};
+// Two sites, h of lanes 0 to 15 and h of lanes 16 to 31, in FP64, output included where mine;
+// returns this thread's share of its squared modulus.  All lanes of a warp call it; w: three rows of 32 words
+// of the warp's own, ws apart.  Sixteen lanes a site, one per hop and half-spin row, and then one per output
+// component for the sum, with the FP64 stencil's operations in its order.  A lone
+// site takes 54 FP64 instructions of 64 cycles in a row this way, one on a thread of its own 850.
+inline __device__ __noinline__ double fx_redo(const FxParams& P, double2* w, int ws, int p, int k, int h, bool mine, int outfx) {
+    const int lane = threadIdx.x & 31, l = lane & 15, j = l >> 1, r = l & 1, mu = j >> 1;
+    const bool fwd = (j & 1) == 0;
     int c[4], s;
     site_of_half(h, p, P.g, c, s);
-#pragma unroll 1
-    for (int j = 0; j < 8; j++) {
+    {
         bool wrap;
         const int sn = fx_neighbour(P.g, c, s, j, wrap);
-        const double2* psi = reinterpret_cast<const double2*>(fx_at(P.in, 1 - p, k, sn));
-        const double2* lk = reinterpret_cast<const double2*>((j & 1) == 0 ? fx_link_at(P.un, p, j >> 1, s)
-                                                                          : fx_link_at(P.un, 1 - p, j >> 1, sn));
-        cpx<double> v[12];
-#pragma unroll 1
-        for (int q = 0; q < 12; q++) {
-            const double2 d = __ldg(psi + (long long)q * P.in.word_step);
-            v[q] = {d.x, d.y};
+        const int partner = mu < 2 ? 3 - r : 2 + r;
+        const int S = fwd != (P.dag != 0) ? 1 : -1, imag = mu == 0 || mu == 2;
+        const int neg = ((mu == 2 && r == 1) || (mu == 1 && r == 0) ? S : -S) < 0;
+        cpx<double> u[3][3], a[3];
+        const FxField& f = P.nat.p ? P.nat : P.in;
+        const uint4* psi = fx_at(f, 1 - p, k, sn);
+        const int e = P.nat.p ? 0 : fx_exponents(reinterpret_cast<const char*>(fx_at(f, 1 - p, k, 0)), P.g.stride)[sn >> 1] & kFxExpMask;
+        const double scale = __hiloint2double((e - 57) << 20, 0);  // 2^(e + 1 - 1023 - 58), if e != 0
+        auto load = [&](int q) {
+            const uint4 d = __ldg(psi + (long long)q * f.word_step);
+            if (e == 0) return cpx<double>{__hiloint2double((int)d.y, (int)d.x), __hiloint2double((int)d.w, (int)d.z)};
+            return cpx<double>{__ll2double_rn((long long)(int)d.x * (kFxLow + 1LL) + (int)d.y) * scale,
+                               __ll2double_rn((long long)(int)d.z * (kFxLow + 1LL) + (int)d.w) * scale};
+        };
+        const double2* lk = reinterpret_cast<const double2*>(fwd ? fx_link_at(P.un, p, mu, s) : fx_link_at(P.un, 1 - p, mu, sn));
+#pragma unroll
+        for (int q = 0; q < 9; q++)
+            if (q < P.un_recon / 2) {
+                const double2 d = __ldg(lk + (long long)q * P.un.word_step);
+                u[q / 3][q % 3] = {d.x, d.y};
+            }
+        if (P.un_recon == 12) recon_row2(u);
+#pragma unroll
+        for (int q = 0; q < 3; q++) {  // (1 - S g_mu) psi, row r (project() in dslash_impl.cuh)
+            const cpx<double> x = load(3 * r + q), y = load(3 * partner + q);
+            a[q] = {x.re + fx_flip(imag ? y.im : y.re, imag ? 1 - neg : neg), x.im + fx_flip(imag ? y.re : y.im, neg)};
         }
-        fx_native_hop(v, lk, P.un.word_step, P.un_recon, j >> 1, (j & 1) == 0, P.dag, wrap, P.g, acc);
+        if (wrap) {
+            const cpx<double> eta = {P.g.ph[mu][0], fwd ? P.g.ph[mu][1] : -P.g.ph[mu][1]};
+#pragma unroll
+            for (int q = 0; q < 3; q++) a[q] = cmul(eta, a[q]);
+        }
+        if (!fwd) {  // U^dag
+#pragma unroll
+            for (int i = 0; i < 3; i++)
+#pragma unroll
+                for (int q = 0; q <= i; q++) {
+                    const cpx<double> t = cconj(u[i][q]);
+                    u[i][q] = cconj(u[q][i]);
+                    u[q][i] = t;
+                }
+        }
+#pragma unroll
+        for (int i = 0; i < 3; i++) {
+            cpx<double> t = cmul(u[i][0], a[0]);
+            t = cfma(u[i][1], a[1], t);
+            t = cfma(u[i][2], a[2], t);
+            w[ws * i + lane] = make_double2(t.re, t.im);
+        }
     }
-    return fx_finish_native(P, p, k, s, acc, 0, 12);
+    __syncwarp();
+    double n2 = 0.0;
+    if (mine && l < 12) {
+        const int spin = l / 3, lower = spin >= 2;
+        double2 v[1];
+#pragma unroll
+        for (int q = 0; q < 8; q++) {  // expand() in dslash_impl.cuh
+            const int m = q >> 1, row = lower ? (spin == 2) == (m < 2) : spin;
+            const double2 t = w[ws * (l - 3 * spin) + (lane & 16) + 2 * q + row];
+            const int i = lower && (m == 0 || m == 2);
+            const int neg = lower && (((q & 1) != 0) != (P.dag != 0)) != (m == 3 || (m == 1 && spin == 2) || (m == 2 && spin == 3));
+            const double2 x = make_double2(fx_flip(i ? t.y : t.x, i ? 1 - neg : neg), fx_flip(i ? t.x : t.y, neg));
+            v[0] = q ? make_double2(v[0].x + x.x, v[0].y + x.y) : x;
+        }
+        if (outfx) {
+            char* out = P.out.p + (P.full ? p * P.out.pstep : 0) + k * P.out.rstep;
+            reinterpret_cast<double2*>(out)[h + (long long)l * P.g.stride] = v[0];
+            if (l == 0) fx_exponents(out, P.g.stride)[h] = 0;
+        } else {
+            fx_finish(P, const_cast<uint4*>(fx_at(P.out, p, k, s)), P.xpay ? fx_at(P.x, p, k, s) : nullptr, l, v);
+            n2 = fx_norm(v);
+        }
+    }
+    __syncwarp();
+    return n2;
+}
+// The sites h0 + i of the bits i of m (the same for all lanes), of every `step` pairs the one numbered `turn`.
+__device__ __forceinline__ double fx_redo_sites(const FxParams& P, double2* w, int ws, int p, int k, int h0, unsigned m,
+                                                int turn, int step, int outfx) {
+    double n2 = 0.0;
+    for (; m; turn--) {
+        const int a = __ffs(m) - 1;
+        m &= m - 1;
+        const int b = m ? __ffs(m) - 1 : -1;
+        m &= m - 1;
+        if (turn) continue;
+        turn = step;
+        const bool second = threadIdx.x & 16;
+        n2 += fx_redo(P, w, ws, p, k, h0 + (second && b >= 0 ? b : a), !second || b >= 0, outfx);
+    }
+    return n2;
 }
 
 // ---------------------------------------------------------------------------
 // Fields and links in fixed point, for the kernel below: each is converted once
 // instead of in each of the eight hops that read it.  A spinor field has 12 rows
-// of 16-byte words (re.h, re.l, im.h, im.l; v = h 2^30 + l) and a row of exponents, one per site; a
-// site that does not fit has exponent 0 and holds its doubles.  Links: nine rows
+// of 16-byte words (re.h, re.l, im.h, im.l; v = h 2^29 + l) and a row of exponents, one per site, with its
+// nonzero spins; a site that does not fit has exponent 0 and holds its doubles.  Links: nine rows
 // per (parity, mu) as for doubles; a link that does not fit is marked in its first
 // word (kFxBadLink) and read from the doubles.
 // ---------------------------------------------------------------------------
 __host__ __device__ __forceinline__ long long fx_field_bytes(long long stride) { return 196 * stride; }
-
-__device__ __forceinline__ int* fx_exponents(char* f, long long stride) { return reinterpret_cast<int*>(f + 192 * stride); }
 
 // Converts doubles (src; half-site index i, parity par) to a fixed-point field.
 static __global__ void __launch_bounds__(128) fx_pack_kernel(FxField src, char* dst, long long pstep, long long rstep,
@@ -441,15 +497,15 @@ static __global__ void __launch_bounds__(128) fx_pack_kernel(FxField src, char* 
                       (long long)(src.by_site ? s : i) * src.site_step;
     char* f = dst + (npar == 2 ? par * pstep : 0) + k * rstep;
     uint4 d[12];
-    unsigned m = 0, nz = 0;
+    unsigned m = 0, spins = 0;
 #pragma unroll
     for (int q = 0; q < 12; q++) {
         d[q] = __ldg(in + (long long)q * src.word_step);
-        m = max(m, max(d[q].y << 1, d[q].w << 1));
-        nz |= d[q].x | d[q].y << 1 | d[q].z | d[q].w << 1;
+        m = fx_max2(m, d[q]);
+        if (fx_nonzero(d[q])) spins |= 1u << (q / 3);
     }
     int e = (int)(m >> 21);
-    if (e < kFxEmin || e > kFxEmax) e = nz ? 0 : kFxEmin;
+    if (e < kFxEmin || e > kFxEmax) e = spins ? 0 : kFxEmin;
     if (e) {
         const unsigned ew = fx_scale_word(e + kFxOffSpinor);
 #pragma unroll
@@ -463,7 +519,7 @@ static __global__ void __launch_bounds__(128) fx_pack_kernel(FxField src, char* 
     uint4* o = reinterpret_cast<uint4*>(f) + i;
 #pragma unroll
     for (int q = 0; q < 12; q++) o[(long long)q * g.stride] = d[q];
-    fx_exponents(f, g.stride)[i] = e;
+    fx_exponents(f, g.stride)[i] = e ? e | (int)(spins << 12) : 0;
     pdl_trigger();
 }
 
@@ -546,6 +602,7 @@ __device__ __forceinline__ void fx_take_row(const FxSlots<TB>& T, int sigma, FxC
 // directions, for spin 3 - r, and lo[1] from z and t, for spin 2 + r.
 struct FxSums {
     long long up[3][2], lo[2][3][2];
+    unsigned n[3][2], k[4][3];  // the guard's moduli of the current direction, and each direction's counts (re, im)
 };
 
 // The order of the hops: y, x, z, t, backward before forward (see hop_kernel_fx1).
@@ -579,14 +636,15 @@ __device__ __forceinline__ bool fx_turn_hop(const FxParams& P, FxSlots<TB>& T, F
     fx_take_row<MU>(T, bwd ? -sigma : sigma, h);
     if constexpr (N < 7) fx_issue_spinor<NX>(T, in, nhn, t.r, P.g.stride);
     if (nb.x < 0) fx_wrap(P.g.ph[MU][0], bwd ? -P.g.ph[MU][1] : P.g.ph[MU][1], h);
-    const int d = min(t.top - nb.y, 63);
+    const int d = min(t.top - nb.y, kFxMaxShift);
+    const long long half = fx_half(d);
     FxReal neg[3];  // forward U h: Ur hr - Ui hi, Ur hi + Ui hr; backward U^dag h: Ur hr + Ui hi, Ur hi - Ui hr
 #pragma unroll
     for (int k = 0; k < 3; k++) neg[k] = fx_neg(bwd ? h[k].re : h[k].im);
     bool bad = false;
 #pragma unroll
     for (int i = 0; i < 3; i++) {
-        FxAcc re = fx_zero(), im = fx_zero();
+        FxAcc re = fx_zero(half), im = fx_zero(half);
 #pragma unroll
         for (int k = 0; k < 3; k++) {
             const uint4 w = T.l[N & 1][bwd ? k * 3 + i : i * 3 + k][t.sl];
@@ -597,21 +655,18 @@ __device__ __forceinline__ bool fx_turn_hop(const FxParams& P, FxSlots<TB>& T, F
             fx_mac(re, ui, bwd ? h[k].im : neg[k]);
             fx_mac(im, ui, bwd ? neg[k] : h[k].re);
         }
-        const long long wr = fx_sar(fx_sum(re), d), wi = fx_sar(fx_sum(im), d);
+        const long long wr = fx_align(fx_sum(re), d), wi = fx_align(fx_sum(im), d);
         A.up[i][0] += wr;
         A.up[i][1] += wi;
         // lower spins: x: i w1, i w0; y: -w1, w0 (spin 2, spin 3); z: i w0, -i w1; t: -w0, -w1;
         // the minus of row 1 in y and z is put in by fx_negate_if
         fx_add<imag ? 1 : 0, bwd == (MU == 3) ? 1 : -1>(A.lo[MU >> 1][i], wr, wi);
+        A.n[i][0] = fx_modulus(wr, bwd ? 0 : A.n[i][0]);
+        A.n[i][1] = fx_modulus(wi, bwd ? 0 : A.n[i][1]);
+        if (!bwd) A.k[MU][i] = fx_count(A.n[i][0], A.n[i][1]);
     }
     return bad;
 }
-
-// One site of fixed-point fields, if it is out of range, on the FP64 stencil by its two threads
-// (r = 0 the x and y directions, 1 z and t), output included where mine; returns this thread's share of its
-// squared modulus.  All lanes of a warp call it.  A lattice out of range throughout takes 1.1 ms a hop
-// this way on 24^3 x 48 (on one thread a site, 6.1 ms on 32^3 x 64, 3.2 times the volume).
-inline __device__ __noinline__ double fx_redo_site1(const FxParams& P, int p, int k, int h, int r, bool mine, int outfx);
 
 // One site on two threads, lanes l and l + 16 of a warp, one per half-spin row: a
 // thread keeps 18 64-bit sums instead of the 24 of a thread with both rows, and half of
@@ -636,19 +691,20 @@ __global__ void __launch_bounds__(TB, MINB) hop_kernel_fx1(const __grid_constant
     const Geom& g = P.g;
     const char* in = P.in.p + (P.full && p == 0 ? P.in.pstep : 0) + k * P.in.rstep;
     double nrm = 0.0;
-    unsigned long long redo = 0;  // a bit per 64th of the sites' turns: has one to be redone
-    int it = 0;
-    // block-uniform turns; a thread past the end runs site 0 and stores nothing
-    for (int h0 = sb * SITES; h0 < g.Vh; h0 += nb * SITES, it = (it + 1) & 63) {
+    // Block-uniform turns (RED; else the grid covers the sites and there is one: a call in the
+    // loop costs 25 registers' spills); a thread past the end runs site 0 and stores nothing.
+    for (int h0 = sb * SITES; h0 < g.Vh; h0 += nb * SITES) {
         const bool ok = h0 + t.sl < g.Vh;
         const int h = ok ? h0 + t.sl : 0, r = t.r;
         t.h = h;
         bool bad;
+        int spins;  // nonzero ones of the neighbours: bits 0 to 3 in x and y, 4 to 7 in z and t
         __syncwarp();
         {
             // thread r: the forward (0) or backward (1) neighbours
-            const int* ex = reinterpret_cast<const int*>(in + 192LL * g.stride);
+            const int* ex = fx_exponents(in, g.stride);
             int c[4], s, top = 0, low = 1 << 30;
+            spins = 0;
             site_of_half(h, p, g, c, s);
 #pragma unroll
             for (int mu = 0; mu < 4; mu++) {
@@ -656,13 +712,15 @@ __global__ void __launch_bounds__(TB, MINB) hop_kernel_fx1(const __grid_constant
                 const bool w = c[mu] == (r ? 0 : g.L[mu] - 1);
                 const int step = r ? -smu : smu;
                 const int hn = (w ? s - step * (g.L[mu] - 1) : s + step) >> 1;
-                const int e = __ldg(ex + hn);
+                const int ew = __ldg(ex + hn), e = ew & kFxExpMask;
+                spins |= ew >> 12 << (mu < 2 ? 0 : 4);
                 top = max(top, e);
                 low = min(low, e);
                 T.nb[2 * mu + r][t.sl] = make_int2(hn | (w ? (int)0x80000000 : 0), e);
             }
             t.top = max(top, __shfl_xor_sync(0xffffffffu, top, 16));
             bad = min(low, __shfl_xor_sync(0xffffffffu, low, 16)) == 0;
+            spins |= __shfl_xor_sync(0xffffffffu, spins, 16);
         }
         __syncwarp();
         {
@@ -692,44 +750,56 @@ __global__ void __launch_bounds__(TB, MINB) hop_kernel_fx1(const __grid_constant
 #pragma unroll
             for (int z = 0; z < 2; z++) A.lo[0][i][z] += __shfl_xor_sync(0xffffffffu, A.lo[1][i][z], 16);
         if (P.dag) fx_negate_if(A.lo[0], 1);
+        {
+            // the guard, but for a spin to which only zeros contribute (row q: spin q, and 3 - q in x and y, 2 + q in z and t)
+            bool up = false, lo = false;
+#pragma unroll
+            for (int i = 0; i < 3; i++) {
+                const unsigned zt = fx_swap(A.k[2][i]) + A.k[3][i], zt1 = __shfl_xor_sync(0xffffffffu, zt, 16);
+                up = up || fx_below(A.k[0][i] + A.k[1][i] + A.k[2][i] + A.k[3][i]);
+                lo = lo || fx_below(fx_swap(A.k[0][i]) + A.k[1][i] + zt1);
+            }
+            const int xy = (1 << r | 8 >> r) & spins, zt = (1 << r | 4 << r) & spins >> 4, zt1 = (2 >> r | 8 >> r) & spins >> 4;
+            bad = bad || (up && (xy | zt)) || (lo && (xy | zt1));
+            const int bad2 = __shfl_xor_sync(0xffffffffu, (int)bad, 16);
+            bad = bad || bad2;
+        }
         if constexpr (OUTFX) {
             // to 58 bits below the largest component: shift right by sr, left if negative
-            unsigned long long m = 0;
+            unsigned long long mu = 0, ml = 0;
 #pragma unroll
             for (int i = 0; i < 3; i++)
 #pragma unroll
-                for (int z = 0; z < 2; z++)
-                    m |= (unsigned long long)((A.up[i][z] ^ (A.up[i][z] >> 63)) | (A.lo[0][i][z] ^ (A.lo[0][i][z] >> 63)));
+                for (int z = 0; z < 2; z++) {
+                    mu |= (unsigned long long)(A.up[i][z] ^ (A.up[i][z] >> 63));
+                    ml |= (unsigned long long)(A.lo[0][i][z] ^ (A.lo[0][i][z] >> 63));
+                }
+            unsigned long long m = mu | ml;
             m |= __shfl_xor_sync(0xffffffffu, m, 16);
+            int nz = (mu ? 1 << r : 0) | (ml ? 8 >> r : 0);
+            nz |= __shfl_xor_sync(0xffffffffu, nz, 16);
             const int sr = m ? 6 - __clzll((long long)m) : 0;
             const int eo = m ? top + 2 + sr : kFxEmin;
-            if (!ok) continue;
-            if (bad || eo < kFxEmin || eo > kFxEmax) {
-                redo |= 1ULL << it;
-                continue;
-            }
-            const long long half = sr > 0 ? 1LL << (sr - 1) : 0;
-            char* out = P.out.p + (P.full ? p * P.out.pstep : 0) + k * P.out.rstep;
-            uint4* ob = reinterpret_cast<uint4*>(out) + h;
+            bad = bad || eo < kFxEmin || eo > kFxEmax;
+            if (ok && !bad) {
+                const long long half = sr > 0 ? 1LL << (sr - 1) : 0;
+                char* out = P.out.p + (P.full ? p * P.out.pstep : 0) + k * P.out.rstep;
+                uint4* ob = reinterpret_cast<uint4*>(out) + h;
 #pragma unroll
-            for (int q = 0; q < 6; q++) {
-                long long v[2];
+                for (int q = 0; q < 6; q++) {
+                    long long v[2];
 #pragma unroll
-                for (int z = 0; z < 2; z++) {
-                    v[z] = q < 3 ? A.up[q][z] : A.lo[0][q - 3][z];
-                    v[z] = sr > 0 ? (v[z] + half) >> sr : v[z] << -sr;
+                    for (int z = 0; z < 2; z++) {
+                        v[z] = q < 3 ? A.up[q][z] : A.lo[0][q - 3][z];
+                        v[z] = sr > 0 ? (v[z] + half) >> sr : v[z] << -sr;
+                    }
+                    ob[(long long)(q < 3 ? 3 * r + q : 6 - 3 * r + q) * g.stride] =
+                        make_uint4((unsigned)(v[0] >> kFxLimb), (unsigned)v[0] & kFxLow, (unsigned)(v[1] >> kFxLimb),
+                                   (unsigned)v[1] & kFxLow);
                 }
-                ob[(long long)(q < 3 ? 3 * r + q : 6 - 3 * r + q) * g.stride] =
-                    make_uint4((unsigned)(v[0] >> 30), (unsigned)v[0] & 0x3FFFFFFFu, (unsigned)(v[1] >> 30),
-                               (unsigned)v[1] & 0x3FFFFFFFu);
+                if (r == 0) fx_exponents(out, g.stride)[h] = eo | nz << 12;
             }
-            if (r == 0) fx_exponents(out, g.stride)[h] = eo;
-        } else {
-            if (!ok) continue;
-            if (bad) {
-                redo |= 1ULL << it;
-                continue;
-            }
+        } else if (ok && !bad) {
             const FxBias b = fx_bias(top + 1 - 1023 - 56);
             int c[4], s;
             site_of_half(h, p, g, c, s);
@@ -745,79 +815,26 @@ __global__ void __launch_bounds__(TB, MINB) hop_kernel_fx1(const __grid_constant
             fx_finish(P, out, x, 9 - 3 * r, v);
             if (RED) nrm += fx_norm(v);
         }
-    }
-    if (__any_sync(0xffffffffu, redo != 0)) {
-        it = 0;
-#pragma unroll 1
-        for (int h0 = sb * SITES; h0 < g.Vh; h0 += nb * SITES, it = (it + 1) & 63) {
-            const bool mine = h0 + t.sl < g.Vh && (redo >> it & 1);
-            if (!__any_sync(0xffffffffu, mine)) continue;
-            const double n2 = fx_redo_site1(P, p, k, mine ? h0 + t.sl : 0, t.r, mine, OUTFX);
+        const unsigned redo = __ballot_sync(0xffffffffu, ok && bad) & 0xFFFFu;
+        if (redo) {
+            const int warp = threadIdx.x >> 5;  // the warp's columns of T.s, all of whose copies have arrived
+            const double n2 = fx_redo_sites(P, reinterpret_cast<double2*>(&T.s[0][32 * warp]), TB, p, k, h0 + 16 * warp, redo, 0, 1, OUTFX);
             if (RED) nrm += n2;
         }
+        if (!RED) break;
     }
     pdl_trigger();
     if (RED) grid_reduce(nrm, P.red, k, nb * gridDim.y, sb + nb * blockIdx.y);
 }
 
-inline __device__ __noinline__ double fx_redo_site1(const FxParams& P, int p, int k, int h, int r, bool mine, int outfx) {
-    const Geom& g = P.g;
-    const char* in = P.in.p + (P.full && p == 0 ? P.in.pstep : 0) + k * P.in.rstep;
-    const int* ex = reinterpret_cast<const int*>(in + 192LL * g.stride);
-    cpx<double> acc[12];
-#pragma unroll 1
-    for (int q = 0; q < 12; q++) acc[q] = cpx<double>{0.0, 0.0};
-    int c[4], s;
-    site_of_half(h, p, g, c, s);
-    bool bad = false;
-#pragma unroll 1
-    for (int j = 4 * r; j < 4 * r + 4; j++) {
-        bool wrap;
-        const int sn = fx_neighbour(g, c, s, j, wrap), hn = sn >> 1, e = ex[hn];
-        const uint4* fl = (j & 1) == 0 ? fx_link_at(P.u, p, j >> 1, s) : fx_link_at(P.u, 1 - p, j >> 1, sn);
-        bad = bad || e == 0 || fl->x == kFxBadLink;
-        cpx<double> v[12];
-#pragma unroll 1
-        for (int q = 0; q < 12; q++) {
-            const uint4 d = __ldg(reinterpret_cast<const uint4*>(in) + hn + (long long)q * g.stride);
-            if (e == 0) {
-                v[q] = {__hiloint2double((int)d.y, (int)d.x), __hiloint2double((int)d.w, (int)d.z)};
-            } else {
-                const double scale = __hiloint2double((e - 57) << 20, 0);  // 2^(e + 1 - 1023 - 58)
-                v[q] = {__ll2double_rn((long long)(int)d.x * (1LL << 30) + (int)d.y) * scale,
-                        __ll2double_rn((long long)(int)d.z * (1LL << 30) + (int)d.w) * scale};
-            }
-        }
-        const double2* lk = reinterpret_cast<const double2*>((j & 1) == 0 ? fx_link_at(P.un, p, j >> 1, s)
-                                                                          : fx_link_at(P.un, 1 - p, j >> 1, sn));
-        fx_native_hop(v, lk, P.un.word_step, P.un_recon, j >> 1, (j & 1) == 0, P.dag, wrap, g, acc);
-    }
-#pragma unroll 1
-    for (int q = 0; q < 12; q++) {  // the other thread's hops
-        acc[q].re += __shfl_xor_sync(0xffffffffu, acc[q].re, 16);
-        acc[q].im += __shfl_xor_sync(0xffffffffu, acc[q].im, 16);
-    }
-    bad = __shfl_xor_sync(0xffffffffu, (int)bad, 16) || bad;
-    if (!mine || (!bad && !outfx)) return 0.0;
-    if (outfx) {
-        char* out = P.out.p + (P.full ? p * P.out.pstep : 0) + k * P.out.rstep;
-#pragma unroll 1
-        for (int q = 6 * r; q < 6 * r + 6; q++)
-            reinterpret_cast<double2*>(out)[h + (long long)q * g.stride] = make_double2(acc[q].re, acc[q].im);
-        if (r == 0) fx_exponents(out, g.stride)[h] = 0;
-        return 0.0;
-    }
-    return fx_finish_native(P, p, k, s, acc, 6 * r, 6 * r + 6);
-}
-
-// Up to 32 sites, h0 to end, of parity p and right-hand side k, by a block of W warps; returns
-// this thread's share of the output's squared modulus (RED).  Ends with a barrier.
+// Up to 32 sites, h0 to end, of parity p and right-hand side k, by a block of W warps; adds
+// this thread's share of the output's squared modulus to nrm (RED) and returns the sites that are to be
+// done over (fx_tile_redo), the same to all threads.  A barrier has to come before the tile is used again.
 template <bool FXL, bool RED, int W>
-__device__ __forceinline__ double fx_tile(const FxParams& P, FxTile& T, int p, int k, int h0, int end) {
+__device__ __forceinline__ unsigned fx_tile(const FxParams& P, FxTile& T, int p, int k, int h0, int end, double& nrm) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int h = h0 + lane;
     const bool ok = h < end;
-    double nrm = 0.0;
     int c[4], s;
     site_of_half(ok ? h : 0, p, P.g, c, s);
     if (warp == 0) T.bad[lane] = 0;
@@ -825,29 +842,29 @@ __device__ __forceinline__ double fx_tile(const FxParams& P, FxTile& T, int p, i
 #pragma unroll 1
     for (int j = warp; j < 8; j += W) fx_hop<FXL>(P, T, j, p, k, c, s, lane);
     __syncthreads();
-    if (ok) {
+    const int spin = warp & 3;
+    double2 va[W == 8 ? 2 : 3], vb[1];  // warps 4 to 7: the third colour
+    const bool below = warp < 4 ? fx_spin_of<W == 4>(T, spin, 0, P.dag, lane, va) : fx_spin_of<W == 4>(T, spin, 2, P.dag, lane, vb);
+    if (below) T.bad[lane] = 1;
+    __syncthreads();
+    const bool bad = T.bad[lane];
+    if (ok && !bad) {
         uint4* out = const_cast<uint4*>(fx_at(P.out, p, k, s));
         const uint4* x = P.xpay ? fx_at(P.x, p, k, s) : nullptr;
-        if (!T.bad[lane]) {
-            const int spin = warp & 3;
-            if (warp < 4) {
-                double2 v[W == 8 ? 2 : 3];
-                fx_spin_of<W == 4>(T, spin, 0, P.dag, lane, v);
-                fx_finish(P, out, x, spin * 3, v);
-                if (RED) nrm += fx_norm(v);
-            } else {
-                double2 v[1];
-                fx_spin_of<W == 4>(T, spin, 2, P.dag, lane, v);
-                fx_finish(P, out, x, spin * 3 + 2, v);
-                if (RED) nrm += fx_norm(v);
-            }
-        } else if (warp == 0) {
-            const double n2 = fx_redo_site(P, p, k, h);
-            if (RED) nrm += n2;
+        if (warp < 4) {
+            fx_finish(P, out, x, spin * 3, va);
+            if (RED) nrm += fx_norm(va);
+        } else {
+            fx_finish(P, out, x, spin * 3 + 2, vb);
+            if (RED) nrm += fx_norm(vb);
         }
     }
-    __syncthreads();  // the tile is reused
-    return nrm;
+    return __ballot_sync(0xffffffffu, ok && bad);
+}
+template <int W>
+__device__ __forceinline__ double fx_tile_redo(const FxParams& P, FxTile& T, int p, int k, int h0, unsigned redo) {
+    const int warp = threadIdx.x >> 5;
+    return fx_redo_sites(P, reinterpret_cast<double2*>(T.w) + 96 * warp, 32, p, k, h0, redo, warp, W, 0);
 }
 
 // Grid: blockIdx.x = tile * nrhs + rhs, tiles of 32 sites; blockIdx.y = output
@@ -863,8 +880,13 @@ __global__ void __launch_bounds__(32 * W, MINB) hop_kernel_fx(const __grid_const
     if (P.skip && __ldcg(P.skip + (size_t)k * P.skip_stride)) return;
     double nrm = 0.0;
     for (int h0 = sb * 32; h0 < P.g.Vh; h0 += nb * 32) {
-        const double n2 = fx_tile<FXL, RED, W>(P, T, p, k, h0, P.g.Vh);
-        if (RED) nrm += n2;
+        const unsigned redo = fx_tile<FXL, RED, W>(P, T, p, k, h0, P.g.Vh, nrm);
+        if (redo) {
+            const double n2 = fx_tile_redo<W>(P, T, p, k, h0, redo);
+            if (RED) nrm += n2;
+        }
+        if (!RED) break;  // the grid covers the sites
+        __syncthreads();
     }
     pdl_trigger();
     if (RED) grid_reduce(nrm, P.red, k, nb * gridDim.y, sb + nb * blockIdx.y);

@@ -252,7 +252,7 @@ __global__ void pack_gauge_fx_kernel(const double2* __restrict__ canon, char* ba
                 f[k / 3][k % 3] = FxCplx{fx_link(rh, (unsigned)__double2loint(u[k].x)),
                                          fx_link(ih, (unsigned)__double2loint(u[k].y))};
             }
-            bool fits = mx >= kFxLinkLo && mx <= kFxLinkHi;
+            bool fits = mx <= kFxLinkHi;
             if (R == 12) {
                 fx_recon_row2(f);  // a third row of rows that are no SU(3) ones can be larger
 #pragma unroll

@@ -10,8 +10,8 @@ about 8 rms of the output.  1e-14 relative L2 holds all of it, oracle rounding i
 import numpy as np
 import pytest
 
-from conftest import assert_parity
-from gpu_helpers import handle_hop
+from conftest import assert_parity, parity_merge, parity_split
+from gpu_helpers import dev, empty_like_dev, handle_hop, host
 from paper_0710_2442_gb300 import inputs
 
 pytestmark = pytest.mark.gpu
@@ -155,3 +155,98 @@ def test_links_at_the_edge_of_the_range(w, monkeypatch, dims, case):
     got = handle_hop(*args)
     monkeypatch.setenv("WILSON_HOP_VARIANT", "0")
     assert_parity(got, handle_hop(*args), TOL)
+
+
+def hop_moduli(U, a, dims):
+    """Each component's sum of the moduli of its terms: a = (|re|, |im|) of a full field [V, 4, 3],
+    as [2, V, 4, 3]; boundary phases +-1.  Partner spins: 3 - s in x and y, s ^ 2 in z and t, with a factor i in x and z."""
+    L = tuple(reversed(dims))
+    u = np.stack([np.abs(U.real), np.abs(U.imag)]).reshape(2, *L, 4, 3, 3)
+    a = a.reshape(2, *L, 4, 3)
+    s = np.zeros_like(a)
+    for mu in range(4):
+        axis = 3 - mu  # of the lattice: t, z, y, x
+        h = a + (a[:, ..., [3, 2, 1, 0], :] if mu < 2 else a[:, ..., [2, 3, 0, 1], :])[::-1 if mu in (0, 2) else 1]
+        f = np.roll(h, -1, axis=axis + 1)
+        m = u[..., mu, :, :]
+        for re, im, links in ((f[0], f[1], m), (h[0], h[1], np.swapaxes(m, -1, -2))):
+            x = np.stack([np.einsum("...ik,...sk->...si", links[0], re) + np.einsum("...ik,...sk->...si", links[1], im),
+                          np.einsum("...ik,...sk->...si", links[0], im) + np.einsum("...ik,...sk->...si", links[1], re)])
+            s += x if links is m else np.roll(x, 1, axis=axis + 1)
+    return s.reshape(2, -1, 4, 3)
+
+
+def graded_field(kind, V, seed):
+    rng = np.random.default_rng(seed)
+    psi = inputs.gaussian_spinor(V, seed=seed)
+    if kind == "colour":
+        return psi * np.array([1.0, 1e-4, 1e-8])
+    if kind == "spin":
+        return psi * np.array([1e-10, 1.0, 1e-2, 1e-6])[:, None]
+    if kind == "imaginary":
+        return psi.real + 1e-9j * psi.imag
+    if kind == "component":
+        return psi.real * 2.0 ** -rng.integers(0, 40, psi.shape) + 1j * psi.imag * 2.0 ** -rng.integers(0, 40, psi.shape)
+    if kind == "one spin":
+        psi[:, [0, 1, 3]] = 0
+        return psi
+    if kind == "site":
+        return psi * 2.0 ** -rng.integers(0, 40, V)[:, None, None]
+    return psi
+
+
+def links_of(kind, dims):
+    if kind == "abelian":
+        U = inputs.gauge_field(dims, "unit")
+        a = np.random.default_rng(421).standard_normal(U.shape[:-1])
+        a[..., 2] = -a[..., 0] - a[..., 1]
+        return U * np.exp(1j * a)[..., None]
+    if kind == "slice of zeros":
+        U = inputs.gauge_field(dims, "random", seed=422).reshape(-1, 4, 3, 3)
+        U[: V3(dims), 3] = 0
+        return U
+    return inputs.gauge_field(dims, "weak", eps=1e-6, seed=423) if kind == "near unit" else inputs.gauge_field(dims, kind, seed=424)
+
+
+def V3(dims):
+    return dims[0] * dims[1] * dims[2]
+
+
+@pytest.mark.parametrize("dims", [(4, 4, 4, 6), (14, 14, 12, 18)])
+@pytest.mark.parametrize("links", ["unit", "abelian", "near unit", "random", "slice of zeros"])
+@pytest.mark.parametrize("field", ["gaussian", "colour", "spin", "imaginary", "component", "one spin", "site"])
+def test_component_accuracy(w, oracle_mod, dims, links, field):
+    """Every component as accurate as FP64 arithmetic leaves it, whatever the others of its site are: a component of the
+    hop is 13 roundings (1 projection, 6 products, 7 sums) of a sum of terms, so two FP64 evaluations
+    differ by at most 28 units 2^-53 of its terms' moduli; M adds 2 more; a Schur operator applies it twice.  Stateless and on
+    handles; one lattice on each of the two kernels."""
+    V, kappa = inputs.volume(dims), 0.13
+    U = links_of(links, dims)
+    psi = graded_field(field, V, 425)
+    mod = np.stack([np.abs(psi.real), np.abs(psi.imag)])
+    s1 = hop_moduli(U, mod, dims)
+    unit = 2.0 ** -53
+    L = w.lattice(dims)
+
+    def check(got, want, bound, what):
+        err = np.stack([np.abs((got - want).real), np.abs((got - want).imag)])
+        assert np.all(err <= bound), (what, float(np.max(err / np.maximum(bound, 1e-300))))
+
+    out = empty_like_dev(psi)
+    w.wilson_dslash(out, dev(U), dev(psi), L, kappa, w.WILSON_OP_M)
+    want = oracle_mod.wilson_m(U, psi, dims, kappa)
+    check(host(out), want, 32 * unit * (kappa * s1 + mod), "m")
+    got = handle_hop(w, U, psi, dims, inputs.DEFAULT_PHASES, w.WILSON_F64, 18, w.WILSON_FULL, w.WILSON_FULL, w.WILSON_OP_M, kappa)
+    check(got, want, 32 * unit * (kappa * s1 + mod), "m on handles")
+
+    even, odd = parity_split(psi, dims)
+    s2 = hop_moduli(U, hop_moduli(U, np.stack([np.abs(parity_merge(even, 0 * odd, dims).real),
+                                               np.abs(parity_merge(even, 0 * odd, dims).imag)]), dims), dims)
+    bound = np.stack([parity_split(s2[z], dims)[0] for z in (0, 1)]) * kappa ** 2 * 64 * unit
+    bound += 4 * unit * np.stack([np.abs(even.real), np.abs(even.imag)])
+    want = oracle_mod.schur(U, even, dims, kappa, 0)
+    out = empty_like_dev(even)
+    w.wilson_dslash_eo(out, dev(U), dev(even), L, 0, kappa, w.WILSON_OP_SCHUR)
+    check(host(out), want, bound, "schur")
+    got = handle_hop(w, U, even, dims, inputs.DEFAULT_PHASES, w.WILSON_F64, 18, 0, 0, w.WILSON_OP_SCHUR, kappa)
+    check(got, want, bound, "schur on handles")
