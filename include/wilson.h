@@ -118,7 +118,8 @@ typedef struct {
 /* and fields as they are; larger ones convert them into workspace taken    */
 /* from a per-device memory pool of the library with stream-ordered         */
 /* allocation on the caller's stream (the pool keeps its memory, so only    */
-/* the first call of a size grows it).  The calls do not synchronise.       */
+/* the first call of a size grows it; wilson_release_workspace gives it     */
+/* back).  The calls do not synchronise.                                    */
 /* ---------------------------------------------------------------------- */
 
 /* out = D_h in (op = HOP) or M in (op = M), full lattice.
@@ -146,6 +147,8 @@ int wilson_dslash_eo(double* out, const double* gauge, const double* in, const w
 /* 1e-4 |bhat| (and tol < 1e-7) computes it with FP32 fields and links      */
 /* (error about 1e-7 |Mhat| |x|); every other residual, and every          */
 /* convergence decision, is FP64.                                          */
+/* A solve's fields come from a memory pool of the library, which keeps at  */
+/* most 1/32 of the device's memory between solves.                         */
 /* ---------------------------------------------------------------------- */
 typedef struct {
     int inner;              /* wilson_prec of the inner CG (F64 = plain FP64 CG)            */
@@ -253,8 +256,10 @@ typedef struct wilson_spinor_s wilson_spinor;
  * the 12-real form stores 12).  canon: 4V links, canonical complex128, host
  * or device memory; prec: wilson_prec; recon: 12 or 18.  The handle owns
  * its device copy; canon may be freed on return (the call synchronises the
- * stream).  WILSON_ERR_ARG for invalid arguments, WILSON_ERR_OOM when the
- * device copy cannot be allocated. */
+ * stream).  An F64 handle holds the links twice, as doubles (12 or 18 reals) and in
+ * block fixed point (18 words of 8 bytes); where the second does not fit in memory, its
+ * operators run on the FP64 stencil instead.  WILSON_ERR_ARG for invalid arguments,
+ * WILSON_ERR_OOM when the device copy cannot be allocated. */
 int wilson_gauge_create(wilson_gauge** g, const double* canon, const wilson_lattice* L, int prec,
                         int recon, void* stream);
 /* Frees the handle's device memory; NULL is accepted. */
@@ -420,6 +425,14 @@ int wilson_probe_hop_access(wilson_spinor* out, const wilson_gauge* g, const wil
  * sweep and returns, so a solver reports WILSON_ERR_NUMERIC).  A healthy run
  * reads 0.  Synchronises the stream. */
 int wilson_stage_timeouts(unsigned long long* count, void* stream);
+
+/* ---------------------------------------------------------------------- */
+/* Memory that the library keeps on the current device between calls, for   */
+/* the workspace of operators and solves, goes back to the device as far as */
+/* no call in flight uses it (synchronise first to give back all of it).    */
+/* Allocations of the library itself do this before they fail.              */
+/* ---------------------------------------------------------------------- */
+int wilson_release_workspace(void);
 
 /* ---------------------------------------------------------------------- */
 /* Errors and version                                                      */

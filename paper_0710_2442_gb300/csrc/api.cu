@@ -123,46 +123,10 @@ SolveStream& solve_stream() {
     return ss;
 }
 
-
-// Workspace of the stateless operator calls: one memory pool per device that
-// keeps its memory after release (release threshold: unlimited).  A call
-// takes its packed fields from the pool with cudaMallocFromPoolAsync and
-// returns them with cudaFreeAsync, both ordered on the caller's stream, so
-// the call never synchronises: the pool reuses the memory once the stream
-// has passed the release (a later call on another stream gets other memory
-// or an ordering dependency the pool inserts).  Only the first call of a new
-// size grows the pool.
-cudaMemPool_t device_pool(std::mutex& m, cudaMemPool_t (&pools)[64]) {
-    int dev = 0;
-    WL_CUDA(cudaGetDevice(&dev));
-    WL_REQUIRE(dev >= 0 && dev < 64, "device ordinal out of range");
-    std::lock_guard<std::mutex> lk(m);
-    if (!pools[dev]) {
-        cudaMemPoolProps props = {};
-        props.allocType = cudaMemAllocationTypePinned;
-        props.handleTypes = cudaMemHandleTypeNone;
-        props.location.type = cudaMemLocationTypeDevice;
-        props.location.id = dev;
-        cudaMemPool_t pool = nullptr;
-        WL_CUDA(cudaMemPoolCreate(&pool, &props));
-        unsigned long long keep = ~0ULL;
-        WL_CUDA(cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep));
-        pools[dev] = pool;
-    }
-    return pools[dev];
-}
-cudaMemPool_t stateless_pool() {
-    static std::mutex m;
-    static cudaMemPool_t pools[64] = {};
-    return device_pool(m, pools);
-}
-// The same for the fixed-point inputs of F64 handle hops; what is unused goes
-// back to the device when an F64 gauge handle is destroyed.
-cudaMemPool_t hop_pool() {
-    static std::mutex m;
-    static cudaMemPool_t pools[64] = {};
-    return device_pool(m, pools);
-}
+// Workspace of the operator calls, from the library's memory pools (workspace.cu) with
+// stream-ordered allocation on the caller's stream, so that a call never synchronises: a pool
+// reuses the memory once the stream has passed the release (a later call on
+// another stream gets other memory or an ordering dependency the pool inserts).
 
 // Stream-ordered allocations of one call, released on the stream when the
 // call's scope ends (also when it throws).
@@ -173,16 +137,16 @@ struct StreamAllocs {
     explicit StreamAllocs(cudaStream_t s) : st(s) {}
     void* get(size_t bytes) {
         void* q = nullptr;
-        WL_CUDA(cudaMallocFromPoolAsync(&q, bytes, stateless_pool(), st));
+        WL_CUDA(pool_alloc(&q, bytes, POOL_STATELESS, st));
         p[n++] = q;
         return q;
     }
     // Null where there is no memory, or the stream is being captured.
-    void* try_get(cudaMemPool_t pool, size_t bytes) {
+    void* try_get(Pool pool, size_t bytes) {
         cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
         void* q = nullptr;
         if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone ||
-            cudaMallocFromPoolAsync(&q, bytes, pool, st) != cudaSuccess) {
+            pool_alloc(&q, bytes, pool, st) != cudaSuccess) {
             (void)cudaGetLastError();
             return nullptr;
         }
@@ -315,6 +279,13 @@ void wl::stateless_op(double* out, const double* gauge, const double* in, const 
 
 // ---------------------------------------------------------------------------
 extern "C" {
+
+int wilson_release_workspace(void) {
+    return guarded([] {
+        check_device();
+        trim_pools();
+    });
+}
 
 const char* wilson_last_error(void) { return g_last_error.c_str(); }
 
@@ -526,7 +497,14 @@ int wilson_gauge_create(wilson_gauge** out, const double* canon, const wilson_la
         h->f.recon = recon;
         h->f.g = g;
         h->f.buf.alloc(gauge_bytes(p, recon, g.stride));
-        if (p == P_F64) h->f.fx.alloc(gauge_bytes(P_F64, 18, g.stride));
+        if (p == P_F64) {
+            try {
+                h->f.fx.alloc(gauge_bytes(P_F64, 18, g.stride));
+            } catch (const Error& e) {  // no room for both forms: the FP64 stencil runs on the doubles
+                if (e.code != WILSON_ERR_OOM) throw;
+                (void)cudaGetLastError();
+            }
+        }
         DevBuf tmp;
         const double* d = device_view(canon, sizeof(double) * 72 * 2 * (size_t)g.Vh, tmp, st);
         pack_gauge(h->f, d, st);
@@ -536,11 +514,7 @@ int wilson_gauge_create(wilson_gauge** out, const double* canon, const wilson_la
 }
 
 int wilson_gauge_destroy(wilson_gauge* g) {
-    return guarded([&] {
-        const bool trim = g && g->f.fx.p;
-        delete g;
-        if (trim) WL_CUDA(cudaMemPoolTrimTo(hop_pool(), 0));
-    });
+    return guarded([&] { delete g; });
 }
 
 int wilson_spinor_create(wilson_spinor** out, const wilson_lattice* L, int subset, int nrhs, int prec) {
@@ -673,7 +647,7 @@ int wilson_dslash_h(wilson_spinor* out, const wilson_gauge* gh, const wilson_spi
         if (fx) {
             h.fx_pstep = fx_spinor_bytes(a.g.stride);
             h.fx_rstep = h.fx_pstep * a.nparity();
-            h.fx_tmp = mem.try_get(hop_pool(), (size_t)h.fx_rstep * a.nrhs);
+            h.fx_tmp = mem.try_get(POOL_HOP, (size_t)h.fx_rstep * a.nrhs);
             fx = h.fx_tmp != nullptr;
         }
         if (op == WILSON_OP_HOP || op == WILSON_OP_M) {

@@ -71,11 +71,20 @@ void launch_dep(void (*kernel)(KArgs...), dim3 grid, dim3 block, cudaStream_t st
 // ---------------------------------------------------------------------------
 // device memory owned by the library
 // ---------------------------------------------------------------------------
+// The memory pools, one per device and use: the stateless calls' workspace (keeps all it
+// ever took, so that only the first call of a size grows it), the fixed-point inputs of F64
+// handle hops, and the solves' workspace (these two keep at most a thirty-second of the device's
+// memory while unused).  An allocation that finds no memory first gives back what all of them hold
+// unused; so does wilson_release_workspace.
+enum Pool { POOL_STATELESS, POOL_HOP, POOL_SOLVE, kPools };
+cudaError_t pool_alloc(void** p, size_t n, Pool which, cudaStream_t st);
+cudaError_t device_alloc(void** p, size_t n);  // cudaMalloc, with that
+void trim_pools();                             // on the current device
+
 // While one is alive, the DevBufs that this thread allocates come from a pool
 // with stream-ordered allocation on st, and go back to it on st (workspace.cu): a solve's
 // 25 to 30 buffers a problem then cost a microsecond each instead of a cudaMalloc
-// and a cudaFree, which waits for the device.  The pool keeps at most a
-// thirty-second of the device's memory between solves.
+// and a cudaFree, which waits for the device.
 struct WorkspaceScope {
     explicit WorkspaceScope(cudaStream_t st);
     ~WorkspaceScope();
@@ -109,7 +118,7 @@ struct DevBuf {
         if (n) {
             p = workspace_alloc(n, &st);
             pooled = p != nullptr;
-            if (!pooled) WL_CUDA(cudaMalloc(&p, n));
+            if (!pooled) WL_CUDA(device_alloc(&p, n));
         }
         bytes = n;
     }

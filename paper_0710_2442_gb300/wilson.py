@@ -92,6 +92,7 @@ def _declare(lib):
         "wilson_dd_halo_bytes": (ctypes.c_longlong, [P(wilson_lattice), I]),
         "wilson_dd_pack": (I, [VP, VP, VP, VP, I, VP]),
         "wilson_dd_hop": (I, [VP, VP, VP, VP, VP, I, I, I, I, VP]),
+        "wilson_release_workspace": (I, []),
         "wilson_last_error": (ctypes.c_char_p, []),
         "wilson_version": (I, []),
     }
@@ -348,3 +349,8 @@ def wilson_stage_timeouts(stream=None) -> int:
 def wilson_dslash_h(out: Spinor, gauge: Gauge, inp: Spinor, kappa: float = 0.0, op: int = WILSON_OP_HOP,
                     stream=None):
     _check(lib().wilson_dslash_h(out.h, gauge.h, inp.h, float(kappa), int(op), _stream(stream)))
+
+
+def wilson_release_workspace():
+    """Gives the memory that the library keeps between calls back to the current device."""
+    _check(lib().wilson_release_workspace())
