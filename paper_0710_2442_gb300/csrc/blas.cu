@@ -1,7 +1,7 @@
 // blas.cu -- BLAS-1 kernels of the CG solves (the paper's caxpy class of
 // kernels, Sec. 4: memory-bound, one pass over each vector), with the FP64
 // reductions fused in.  Each kernel checks its right-hand side's "done" flag
-// first, so iterations captured after convergence cost one empty launch.
+// first: an iteration costs one that has finished an empty launch.
 #include "blas.h"
 
 namespace wl {
@@ -140,7 +140,7 @@ __global__ void __launch_bounds__(256) cg_p_kernel(Vec p, Vec rv, Geom g, int nr
 // their partials, then p = r + beta p; sets the loop's condition.
 template <int PP>
 __global__ void __launch_bounds__(256) cg_p_end_kernel(Vec p, Vec rv, Geom g, int nrhs, CGScalars* sc, RedArgs sred, int ns,
-                                                       RedArgs rred, int nr, LoopHandle loop) {
+                                                       RedArgs rred, int nr, cudaGraphConditionalHandle loop) {
     const RhsIdx r = rhs_index(nrhs);
     CGScalars& C = sc[r.k];
     const bool first = r.sb == 0 && threadIdx.x == 0;
@@ -148,10 +148,10 @@ __global__ void __launch_bounds__(256) cg_p_end_kernel(Vec p, Vec rv, Geom g, in
     // the others whether they went into this iteration (one that ends in it
     // costs an empty iteration).
     auto condition = [&](bool mine) {
-        if (!loop.on || !first || r.k != 0) return;
+        if (!first || r.k != 0) return;
         unsigned go = mine;
         for (int k = 1; k < nrhs; k++) go |= __ldcg(&sc[k].done) == 0;
-        cudaGraphSetConditional(loop.handle, go);
+        cudaGraphSetConditional(loop, go);
     };
     if (finished(C)) {
         condition(false);
@@ -312,7 +312,7 @@ void cg_p_update(Prec pp, Vec p, Vec r, const Geom& g, int nrhs, const CGScalars
 }
 
 void cg_p_end(Prec pp, Vec p, Vec r, const Geom& g, int nrhs, CGScalars* sc, const RedArgs& sred, int ns,
-              const RedArgs& rred, int nr, const LoopHandle& loop, int grid_cap, cudaStream_t st) {
+              const RedArgs& rred, int nr, cudaGraphConditionalHandle loop, int grid_cap, cudaStream_t st) {
     const int block = 256, grid = even_grid(g.Vh, block, grid_cap) * nrhs;
     WL_REQUIRE(ns <= kMaxPartials && nr <= kMaxPartials, "too many partials");
     switch (pp) {

@@ -22,18 +22,13 @@ inline Vec vec(const SpinorField& f, int parity) { return Vec{f.block(parity), f
 int cg_xs_update(Prec xp, Prec pp, Vec x, Vec p, Vec s, Vec q, Vec s_low, const Geom& g, int nrhs, CGScalars* sc,
                  const RedArgs& qred, int nq, const RedArgs& red, int grid_cap, cudaStream_t st);
 
-// The condition of a device-side loop around the iterations (on = 0: none).
-struct LoopHandle {
-    cudaGraphConditionalHandle handle{};
-    int on = 0;
-};
 // p = r + beta p (beta read from sc[k]).
 void cg_p_update(Prec pp, Vec p, Vec r, const Geom& g, int nrhs, const CGScalars* sc, cudaStream_t st);
 // The end of an iteration: iter and done from the ns partials of |s|^2, beta and gam
 // from the nr partials of |r|^2, p = r + beta p for a right-hand side that goes on, and
-// the loop's condition.
+// the condition of the device-side loop around the iterations.
 void cg_p_end(Prec pp, Vec p, Vec r, const Geom& g, int nrhs, CGScalars* sc, const RedArgs& sred, int ns,
-              const RedArgs& rred, int nr, const LoopHandle& loop, int grid_cap, cudaStream_t st);
+              const RedArgs& rred, int nr, cudaGraphConditionalHandle loop, int grid_cap, cudaStream_t st);
 
 // y += a x
 void axpy(Prec yp, Vec y, Prec xp, Vec x, double a, const Geom& g, int nrhs, cudaStream_t st);

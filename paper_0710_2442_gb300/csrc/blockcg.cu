@@ -706,7 +706,7 @@ void BlockInner::iteration(const GaugeField& glo, double kappa, Vec S, Vec W, Ve
 
 BlockInner::Result BlockInner::run(const GaugeField& glo, double kappa, Vec s_in, Vec S, Vec W, Vec Z, Vec T, Vec X,
                                    const std::vector<int>& finished, const std::vector<double>& delta,
-                                   int maxiter, int chunk, bool use_graph, bool reliable, cudaStream_t st) {
+                                   int maxiter, bool reliable, cudaStream_t st) {
     NvtxRange nvtx("block cg");
     // host-side state: the active columns
     BCGState h;
@@ -752,10 +752,10 @@ BlockInner::Result BlockInner::run(const GaugeField& glo, double kappa, Vec s_in
         update(UP_REL, S, X, st);
     }
 
-    if (use_graph && !exec_) {
+    if (!exec_) {
         WL_CUDA(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
         try {
-            for (int k = 0; k < chunk; k++) iteration(glo, kappa, S, W, Z, T, X, st);
+            for (int k = 0; k < kBlockChunk; k++) iteration(glo, kappa, S, W, Z, T, X, st);
         } catch (...) {
             cudaGraph_t junk = nullptr;
             cudaStreamEndCapture(st, &junk);
@@ -767,8 +767,7 @@ BlockInner::Result BlockInner::run(const GaugeField& glo, double kappa, Vec s_in
     }
     int flags[2] = {0, 0};
     while (true) {
-        if (exec_) WL_CUDA(cudaGraphLaunch(exec_, st));
-        else for (int k = 0; k < chunk; k++) iteration(glo, kappa, S, W, Z, T, X, st);
+        WL_CUDA(cudaGraphLaunch(exec_, st));
         WL_CUDA(cudaMemcpyAsync(flags, &d->iter, 2 * sizeof(int), cudaMemcpyDeviceToHost, st));  // iter, maxiter
         int done = 0;
         WL_CUDA(cudaMemcpyAsync(&done, &d->done, sizeof(int), cudaMemcpyDeviceToHost, st));

@@ -9,7 +9,8 @@
 
 namespace wl {
 
-constexpr int kBlockMax = 16;  // right-hand sides one block CG can carry
+constexpr int kBlockMax = 16;    // right-hand sides one block CG can carry
+constexpr int kBlockChunk = 16;  // iterations per captured graph
 
 struct BCGState;
 
@@ -36,8 +37,8 @@ public:
         int status = 0;  // 0: reduced by delta (or iteration cap), 3: breakdown, 4: NaN/Inf
     };
     Result run(const GaugeField& glo, double kappa, Vec s_in, Vec S, Vec W, Vec Z, Vec T, Vec X,
-               const std::vector<int>& finished, const std::vector<double>& delta, int maxiter, int chunk,
-               bool use_graph, bool reliable, cudaStream_t st);
+               const std::vector<int>& finished, const std::vector<double>& delta, int maxiter, bool reliable,
+               cudaStream_t st);
 
 private:
     void iteration(const GaugeField& glo, double kappa, Vec S, Vec W, Vec Z, Vec T, Vec X, cudaStream_t st);

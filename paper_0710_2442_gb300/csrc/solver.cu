@@ -35,7 +35,7 @@
 //   convergence test, beta; p = r + beta p
 // The iteration is the body of a device-side loop (a conditional graph node, whose
 // condition the last launch sets); the host reads the scalars when the loop has
-// ended.  Without conditional nodes a chunk of iterations is captured and replayed.
+// ended.
 #include <algorithm>
 #include <chrono>
 #include <cmath>
@@ -262,7 +262,7 @@ std::vector<SolveStats> cg_solve_prepared(SpinorField& x, const SpinorField& b, 
     }
     schur_tune(g64, P_F64, vec(q64, 0), vec(x, 0), vec(t64, 1), nr, 0, nullptr, 0, st);
 
-    LoopHandle loop;
+    cudaGraphConditionalHandle loop{};
     auto iteration = [&](cudaStream_t s) {
         const int* skip = &sc->done;
         const RedArgs rq = red.args(slot(2), FIN_PARTIAL, nullptr, nullptr);
@@ -279,54 +279,33 @@ std::vector<SolveStats> cg_solve_prepared(SpinorField& x, const SpinorField& b, 
 
     // The iterations of a correction as one device-side while loop (a
     // conditional graph node, whose condition the p update sets): no iterations
-    // launched after convergence, no host round trip per chunk, and six nodes to
-    // instantiate instead of 96.
+    // launched after convergence, no host round trip on the way, and six nodes to
+    // instantiate.
     cudaGraphExec_t gexec = nullptr;
     cudaGraph_t graph = nullptr;
-    const int chunk = prm.chunk > 0 ? prm.chunk : 16;
-    bool loops = false;
-    if (prm.use_graph && !blk) {
-        WL_CUDA(cudaGraphCreate(&graph, 0));
+    WL_CUDA(cudaGraphCreate(&graph, 0));
+    try {
+        WL_CUDA(cudaGraphConditionalHandleCreate(&loop, graph, 1, cudaGraphCondAssignDefault));
         cudaGraphNodeParams cp = {cudaGraphNodeTypeConditional};
+        cp.conditional.handle = loop;
         cp.conditional.type = cudaGraphCondTypeWhile;
         cp.conditional.size = 1;
         cudaGraphNode_t cnode;
-        if (cudaGraphConditionalHandleCreate(&loop.handle, graph, 1, cudaGraphCondAssignDefault) == cudaSuccess) {
-            cp.conditional.handle = loop.handle;
-            loops = cudaGraphAddNode(&cnode, graph, nullptr, nullptr, 0, &cp) == cudaSuccess;
-        }
-        if (loops) {
-            loop.on = 1;
-            cudaGraph_t out = nullptr;
-            try {
-                WL_CUDA(cudaStreamBeginCaptureToGraph(st, cp.conditional.phGraph_out[0], nullptr, nullptr, 0,
-                                                      cudaStreamCaptureModeThreadLocal));
-                iteration(st);
-            } catch (...) {
-                cudaStreamEndCapture(st, &out);
-                cudaGraphDestroy(graph);
-                throw;
-            }
-            WL_CUDA(cudaStreamEndCapture(st, &out));
-            WL_CUDA(cudaGraphInstantiate(&gexec, graph, 0));
-        } else {  // no conditional nodes here: chunks of captured iterations
-            (void)cudaGetLastError();
-            cudaGraphDestroy(graph);
-            graph = nullptr;
-        }
-    }
-    if (prm.use_graph && !loops) {
-        WL_CUDA(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
+        WL_CUDA(cudaGraphAddNode(&cnode, graph, nullptr, nullptr, 0, &cp));
+        WL_CUDA(cudaStreamBeginCaptureToGraph(st, cp.conditional.phGraph_out[0], nullptr, nullptr, 0,
+                                              cudaStreamCaptureModeThreadLocal));
+        cudaGraph_t out = nullptr;
         try {
-            for (int k = 0; k < chunk; k++) iteration(st);
+            iteration(st);
         } catch (...) {
-            cudaGraph_t junk = nullptr;
-            cudaStreamEndCapture(st, &junk);
-            if (junk) cudaGraphDestroy(junk);
+            cudaStreamEndCapture(st, &out);
             throw;
         }
-        WL_CUDA(cudaStreamEndCapture(st, &graph));
+        WL_CUDA(cudaStreamEndCapture(st, &out));
         WL_CUDA(cudaGraphInstantiate(&gexec, graph, 0));
+    } catch (...) {
+        cudaGraphDestroy(graph);
+        throw;
     }
 
     std::vector<int> total_inner(nr, 0), finished(nr, 0);
@@ -335,7 +314,7 @@ std::vector<SolveStats> cg_solve_prepared(SpinorField& x, const SpinorField& b, 
     bool first = true;
     bool force64 = false;  // the next residual is FP64
     bool f32_off = false;  // no more FP32 residuals in this solve
-    // device time of the inner iterations: events around each chunk's replay
+    // device time of the inner iterations: events around each loop
     cudaEvent_t ev_in0 = nullptr, ev_in1 = nullptr;
     WL_CUDA(cudaEventCreate(&ev_in0));
     WL_CUDA(cudaEventCreate(&ev_in1));
@@ -426,8 +405,7 @@ std::vector<SolveStats> cg_solve_prepared(SpinorField& x, const SpinorField& b, 
                 }
                 const BlockInner::Result br =
                     blk->run(glo, kappa, in.s_in(), vec(in.p, 0), vec(in.q, 0), vec(in.r, 0), vec(in.t, 1),
-                             vec(in.xin, 0), finished, dk, left, chunk, prm.use_graph != 0, prm.reliable != 0,
-                             st);
+                             vec(in.xin, 0), finished, dk, left, prm.reliable != 0, st);
                 hops += 2 + 4 * br.iterations;
                 for (int k = 0; k < nr; k++)
                     if (!finished[k]) total_inner[k] += br.iterations;
@@ -480,25 +458,15 @@ std::vector<SolveStats> cg_solve_prepared(SpinorField& x, const SpinorField& b, 
             else cg_p_update(in.ip, vec(in.p, 0), vec(in.r, 0), g, nr, sc, st);
             first = false;
 
-            while (true) {
-                WL_CUDA(cudaEventRecord(ev_in0, st));
-                if (gexec) {
-                    WL_CUDA(cudaGraphLaunch(gexec, st));
-                } else {
-                    for (int it = 0; it < chunk; it++) iteration(st);
-                }
-                WL_CUDA(cudaEventRecord(ev_in1, st));
-                WL_CUDA(cudaMemcpyAsync(h_sc, sc, sizeof(CGScalars) * nr, cudaMemcpyDeviceToHost, st));
-                WL_CUDA(cudaStreamSynchronize(st));
-                {
-                    float ms = 0.f;
-                    WL_CUDA(cudaEventElapsedTime(&ms, ev_in0, ev_in1));
-                    inner_ms += ms;
-                }
-                bool all = true;
-                for (int k = 0; k < nr; k++) all = all && h_sc[k].done != 0;
-                if (all) break;
-            }
+            WL_CUDA(cudaEventRecord(ev_in0, st));
+            WL_CUDA(cudaGraphLaunch(gexec, st));
+            WL_CUDA(cudaEventRecord(ev_in1, st));
+            WL_CUDA(cudaMemcpyAsync(h_sc, sc, sizeof(CGScalars) * nr, cudaMemcpyDeviceToHost, st));
+            WL_CUDA(cudaStreamSynchronize(st));
+            float ms = 0.f;
+            WL_CUDA(cudaEventElapsedTime(&ms, ev_in0, ev_in1));
+            inner_ms += ms;
+            for (int k = 0; k < nr; k++) WL_REQUIRE(h_sc[k].done != 0, "the device loop ended before its right-hand sides did");
             int most = 0;
             for (int k = 0; k < nr; k++) {
                 if (finished[k]) continue;
@@ -513,14 +481,14 @@ std::vector<SolveStats> cg_solve_prepared(SpinorField& x, const SpinorField& b, 
             axpy(P_F64, vec(x, 0), in.xp, vec(in.xin, 0), 1.0, g, nr, st);
         }
     } catch (...) {
-        if (gexec) cudaGraphExecDestroy(gexec);
-        if (graph) cudaGraphDestroy(graph);
+        cudaGraphExecDestroy(gexec);
+        cudaGraphDestroy(graph);
         cudaEventDestroy(ev_in0);
         cudaEventDestroy(ev_in1);
         throw;
     }
-    if (gexec) cudaGraphExecDestroy(gexec);
-    if (graph) cudaGraphDestroy(graph);
+    cudaGraphExecDestroy(gexec);
+    cudaGraphDestroy(graph);
     cudaEventDestroy(ev_in0);
     cudaEventDestroy(ev_in1);
 

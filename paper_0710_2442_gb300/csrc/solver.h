@@ -19,8 +19,6 @@ struct SolveParams {
     int use_initial_guess = 0;
     int reliable = 1;
     int block_cg = 0;           // several right-hand sides: one block CG instead of lockstep CGs
-    int chunk = 16;           // iterations per captured graph
-    int use_graph = 1;
     int batch_small_vh = 4096;  // batched solves: problems with at most this many sites per parity
                                 // run the CTA-resident solver (0: none)
 };
