@@ -634,10 +634,14 @@ void batch_solve(int n, const wilson_problem* probs, const SolveParams& prm, wil
     WL_CUDA(cudaEventCreateWithFlags(&join, cudaEventDisableTiming));
     WL_CUDA(cudaEventCreateWithFlags(&fork3, cudaEventDisableTiming));
     WL_CUDA(cudaEventCreateWithFlags(&join3, cudaEventDisableTiming));
+    // After an exception work may be left on the side streams (the small problems' solves,
+    // bounded by their budget), and the buffers go back in st's order alone: wait for it.
     struct Cleanup {
         cudaStream_t s[2];
         cudaEvent_t e[4];
         ~Cleanup() {
+            for (cudaStream_t x : s)
+                if (x && cudaStreamSynchronize(x) != cudaSuccess) (void)cudaGetLastError();
             for (cudaStream_t x : s)
                 if (x) cudaStreamDestroy(x);
             for (cudaEvent_t x : e)

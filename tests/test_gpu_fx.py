@@ -250,3 +250,35 @@ def test_component_accuracy(w, oracle_mod, dims, links, field):
     check(host(out), want, bound, "schur")
     got = handle_hop(w, U, even, dims, inputs.DEFAULT_PHASES, w.WILSON_F64, 18, 0, 0, w.WILSON_OP_SCHUR, kappa)
     check(got, want, bound, "schur on handles")
+
+
+def test_captured_handle_operators(w, oracle_mod):
+    """Under stream capture an F64 operator takes no workspace (a captured call allocates
+    nothing), so that its hops of a large lattice run on the other kernel: the same operator."""
+    import torch
+    dims = (14, 14, 12, 18)
+    L = w.lattice(dims, PHASES)
+    U = inputs.gauge_field(dims, "random", seed=435)
+    src = inputs.gaussian_spinor(inputs.volume(dims) // 2, seed=436)
+    g = w.Gauge(U, L, w.WILSON_F64, 18)
+    a, b, c = (w.Spinor(L, w.WILSON_EVEN, w.WILSON_F64) for _ in range(3))
+    d = w.Spinor(L, w.WILSON_ODD, w.WILSON_F64)
+    a.load(dev(src))
+    w.wilson_dslash_h(b, g, a, 0.13, w.WILSON_OP_SCHUR)  # the handle's intermediate field
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        w.wilson_dslash_h(c, g, a, 0.13, w.WILSON_OP_SCHUR)
+        w.wilson_dslash_h(d, g, a, 0.0, w.WILSON_OP_HOP)
+    got = []
+    for _ in range(2):
+        graph.replay()
+        got.append([np.empty_like(src), np.empty_like(src)])
+        for f, x in zip((c, d), got[-1]):
+            out = empty_like_dev(src)
+            f.store(out)
+            x[:] = host(out)
+    for x, y in zip(*got):
+        assert np.array_equal(x, y)
+    assert_parity(got[0][0], oracle_mod.schur(U, src, dims, 0.13, 0, False, PHASES), TOL)
+    assert_parity(got[0][1], oracle_mod.dslash_eo(U, src, dims, 1, PHASES), TOL)
