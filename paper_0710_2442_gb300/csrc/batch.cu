@@ -350,7 +350,7 @@ struct BatchRun {
     void hop(const BOp& o, int dag, cudaStream_t st) const {
         if (o.use64 == 1) {
             WL_REQUIRE(!dag, "the batched FP64 hop is never daggered");
-            launch_bhop_fx(A, o, grid, st);
+            launch_bhop_fx(A, o, st);
         } else if (o.use64 == 2) {
             hop_t<P_F32, P_F32>(o, dag, hop_32, st);
         } else {

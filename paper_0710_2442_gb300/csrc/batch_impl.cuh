@@ -759,7 +759,7 @@ extern template void launch_bhop<P_F32, P_F32>(const BatchArgs&, const BOp&, int
 extern template void launch_bhop<P_F16, P_F16>(const BatchArgs&, const BOp&, int, int, int, int, cudaStream_t);
 extern template void launch_bhop<P_BF16, P_BF16>(const BatchArgs&, const BOp&, int, int, int, int, cudaStream_t);
 // The FP64 hop, dagger = 0 (batch_hop_64.cu).
-void launch_bhop_fx(const BatchArgs& A, const BOp& o, int blocks, cudaStream_t st);
+void launch_bhop_fx(const BatchArgs& A, const BOp& o, cudaStream_t st);
 
 // The CTA-resident solves of nprob small problems (ids: their indices), inner
 // precision IP.  Instantiated one inner precision per translation unit

@@ -671,157 +671,174 @@ __device__ __forceinline__ bool fx_turn_hop(const FxParams& P, FxSlots<TB>& T, F
 // One site on two threads, lanes l and l + 16 of a warp, one per half-spin row: a
 // thread keeps 18 64-bit sums instead of the 24 of a thread with both rows, and half of
 // the half spinor.  Output: doubles, or a fixed-point field (OUTFX; out.p in
-// that form, no xpay or scale).
+// that form, no xpay or scale).  The block's sites are h0 and the next ones, a thread past the end runs site 0 and
+// stores nothing; returns the sites of its warp that are to be done over (bits 0 to 15).
+struct FxDone {
+    double n2;  // this thread's share of the output's squared modulus (RED)
+    unsigned redo;
+};
+template <bool OUTFX, bool RED, int TB>
+__device__ __forceinline__ FxDone fx_sites(const FxParams& P, FxSlots<TB>& T, const char* in, int p, int k, int h0) {
+    const Geom& g = P.g;
+    FxTurn t;
+    t.r = threadIdx.x >> 4 & 1;
+    t.sl = (threadIdx.x >> 5) * 16 + (threadIdx.x & 15);
+    t.S = P.dag ? -1 : 1;
+    t.p = p;
+    double nrm = 0.0;
+    const bool ok = h0 + t.sl < g.Vh;
+    const int h = ok ? h0 + t.sl : 0, r = t.r;
+    t.h = h;
+    bool bad;
+    int spins;  // nonzero ones of the neighbours: bits 0 to 3 in x and y, 4 to 7 in z and t
+    __syncwarp();
+    {
+        // thread r: the forward (0) or backward (1) neighbours
+        const int* ex = fx_exponents(in, g.stride);
+        int c[4], s, top = 0, low = 1 << 30;
+        spins = 0;
+        site_of_half(h, p, g, c, s);
+#pragma unroll
+        for (int mu = 0; mu < 4; mu++) {
+            const int smu = mu == 0 ? 1 : mu == 1 ? g.L[0] : mu == 2 ? g.L[0] * g.L[1] : g.L[0] * g.L[1] * g.L[2];
+            const bool w = c[mu] == (r ? 0 : g.L[mu] - 1);
+            const int step = r ? -smu : smu;
+            const int hn = (w ? s - step * (g.L[mu] - 1) : s + step) >> 1;
+            const int ew = __ldg(ex + hn), e = ew & kFxExpMask;
+            spins |= ew >> 12 << (mu < 2 ? 0 : 4);
+            top = max(top, e);
+            low = min(low, e);
+            T.nb[2 * mu + r][t.sl] = make_int2(hn | (w ? (int)0x80000000 : 0), e);
+        }
+        t.top = max(top, __shfl_xor_sync(0xffffffffu, top, 16));
+        bad = min(low, __shfl_xor_sync(0xffffffffu, low, 16)) == 0;
+        spins |= __shfl_xor_sync(0xffffffffu, spins, 16);
+    }
+    __syncwarp();
+    {
+        const int hn = T.nb[3][t.sl].x & 0x7FFFFFFF;
+        fx_issue_link<TB>(T.l[0], P.u.p, (1 - p) * 4 + 1, hn, r, t.sl, g.stride);
+        fx_issue_spinor<1>(T, in, hn, r, g.stride);
+    }
+    FxSums A;
+#pragma unroll
+    for (int i = 0; i < 3; i++)
+#pragma unroll
+        for (int z = 0; z < 2; z++) A.up[i][z] = A.lo[0][i][z] = A.lo[1][i][z] = 0;
+    bad |= fx_turn_hop<0>(P, T, A, t, in);
+    bad |= fx_turn_hop<1>(P, T, A, t, in);
+    fx_negate_if(A.lo[0], r);
+    bad |= fx_turn_hop<2>(P, T, A, t, in);
+    bad |= fx_turn_hop<3>(P, T, A, t, in);
+    bad |= fx_turn_hop<4>(P, T, A, t, in);
+    bad |= fx_turn_hop<5>(P, T, A, t, in);
+    fx_negate_if(A.lo[1], r);
+    bad |= fx_turn_hop<6>(P, T, A, t, in);
+    bad |= fx_turn_hop<7>(P, T, A, t, in);
+    const int top = t.top;
+    // spin 3 - r: this thread's x and y part, the other's z and t part
+#pragma unroll
+    for (int i = 0; i < 3; i++)
+#pragma unroll
+        for (int z = 0; z < 2; z++) A.lo[0][i][z] += __shfl_xor_sync(0xffffffffu, A.lo[1][i][z], 16);
+    if (P.dag) fx_negate_if(A.lo[0], 1);
+    {
+        // the guard, but for a spin to which only zeros contribute (row q: spin q, and 3 - q in x and y, 2 + q in z and t)
+        bool up = false, lo = false;
+#pragma unroll
+        for (int i = 0; i < 3; i++) {
+            const unsigned zt = fx_swap(A.k[2][i]) + A.k[3][i], zt1 = __shfl_xor_sync(0xffffffffu, zt, 16);
+            up = up || fx_below(A.k[0][i] + A.k[1][i] + A.k[2][i] + A.k[3][i]);
+            lo = lo || fx_below(fx_swap(A.k[0][i]) + A.k[1][i] + zt1);
+        }
+        const int xy = (1 << r | 8 >> r) & spins, zt = (1 << r | 4 << r) & spins >> 4, zt1 = (2 >> r | 8 >> r) & spins >> 4;
+        bad = bad || (up && (xy | zt)) || (lo && (xy | zt1));
+        const int bad2 = __shfl_xor_sync(0xffffffffu, (int)bad, 16);
+        bad = bad || bad2;
+    }
+    if constexpr (OUTFX) {
+        // to 58 bits below the largest component: shift right by sr, left if negative
+        unsigned long long mu = 0, ml = 0;
+#pragma unroll
+        for (int i = 0; i < 3; i++)
+#pragma unroll
+            for (int z = 0; z < 2; z++) {
+                mu |= (unsigned long long)(A.up[i][z] ^ (A.up[i][z] >> 63));
+                ml |= (unsigned long long)(A.lo[0][i][z] ^ (A.lo[0][i][z] >> 63));
+            }
+        unsigned long long m = mu | ml;
+        m |= __shfl_xor_sync(0xffffffffu, m, 16);
+        int nz = (mu ? 1 << r : 0) | (ml ? 8 >> r : 0);
+        nz |= __shfl_xor_sync(0xffffffffu, nz, 16);
+        const int sr = m ? 6 - __clzll((long long)m) : 0;
+        const int eo = m ? top + 2 + sr : kFxEmin;
+        bad = bad || eo < kFxEmin || eo > kFxEmax;
+        if (ok && !bad) {
+            const long long half = sr > 0 ? 1LL << (sr - 1) : 0;
+            char* out = P.out.p + (P.full ? p * P.out.pstep : 0) + k * P.out.rstep;
+            uint4* ob = reinterpret_cast<uint4*>(out) + h;
+#pragma unroll
+            for (int q = 0; q < 6; q++) {
+                long long v[2];
+#pragma unroll
+                for (int z = 0; z < 2; z++) {
+                    v[z] = q < 3 ? A.up[q][z] : A.lo[0][q - 3][z];
+                    v[z] = sr > 0 ? (v[z] + half) >> sr : v[z] << -sr;
+                }
+                ob[(long long)(q < 3 ? 3 * r + q : 6 - 3 * r + q) * g.stride] =
+                    make_uint4((unsigned)(v[0] >> kFxLimb), (unsigned)v[0] & kFxLow, (unsigned)(v[1] >> kFxLimb),
+                               (unsigned)v[1] & kFxLow);
+            }
+            if (r == 0) fx_exponents(out, g.stride)[h] = eo | nz << 12;
+        }
+    } else if (ok && !bad) {
+        const FxBias b = fx_bias(top + 1 - 1023 - 56);
+        int c[4], s;
+        site_of_half(h, p, g, c, s);
+        uint4* out = const_cast<uint4*>(fx_at(P.out, p, k, s));
+        const uint4* x = P.xpay ? fx_at(P.x, p, k, s) : nullptr;
+        double2 v[3];
+#pragma unroll
+        for (int i = 0; i < 3; i++) v[i] = make_double2(fx_double(A.up[i][0], b), fx_double(A.up[i][1], b));
+        fx_finish(P, out, x, 3 * r, v);
+        if (RED) nrm += fx_norm(v);
+#pragma unroll
+        for (int i = 0; i < 3; i++) v[i] = make_double2(fx_double(A.lo[0][i][0], b), fx_double(A.lo[0][i][1], b));
+        fx_finish(P, out, x, 9 - 3 * r, v);
+        if (RED) nrm += fx_norm(v);
+    }
+    return FxDone{nrm, __ballot_sync(0xffffffffu, ok && bad) & 0xFFFFu};
+}
+// For a loop over turns: in line, the call to fx_redo beside it costs the loop 40 registers' spills.
+template <bool RED, int TB>
+__device__ __noinline__ FxDone fx_sites_call(const FxParams& P, FxSlots<TB>& T, const char* in, int p, int k, int h0) {
+    return fx_sites<false, RED>(P, T, in, p, k, h0);
+}
+
 template <bool OUTFX, bool RED, int TB, int MINB>
 __global__ void __launch_bounds__(TB, MINB) hop_kernel_fx1(const __grid_constant__ FxParams P) {
     extern __shared__ __align__(16) unsigned char fx_smem[];
     FxSlots<TB>& T = *reinterpret_cast<FxSlots<TB>*>(fx_smem);
     constexpr int SITES = TB / 2;
-    FxTurn t;
-    t.r = threadIdx.x >> 4 & 1;
-    t.sl = (threadIdx.x >> 5) * 16 + (threadIdx.x & 15);
-    t.S = P.dag ? -1 : 1;
     const int k = blockIdx.x % P.nrhs;
     const int sb = blockIdx.x / P.nrhs;
     const int nb = gridDim.x / P.nrhs;
     const int p = P.full ? (int)blockIdx.y : P.out_parity;
-    t.p = p;
     pdl_wait();
     if (P.skip && __ldcg(P.skip + (size_t)k * P.skip_stride)) return;
-    const Geom& g = P.g;
     const char* in = P.in.p + (P.full && p == 0 ? P.in.pstep : 0) + k * P.in.rstep;
+    const int warp = threadIdx.x >> 5;
+    double2* w = reinterpret_cast<double2*>(&T.s[0][32 * warp]);  // the warp's columns, all of whose copies have arrived
     double nrm = 0.0;
-    // Block-uniform turns (RED; else the grid covers the sites and there is one: a call in the
-    // loop costs 25 registers' spills); a thread past the end runs site 0 and stores nothing.
-    for (int h0 = sb * SITES; h0 < g.Vh; h0 += nb * SITES) {
-        const bool ok = h0 + t.sl < g.Vh;
-        const int h = ok ? h0 + t.sl : 0, r = t.r;
-        t.h = h;
-        bool bad;
-        int spins;  // nonzero ones of the neighbours: bits 0 to 3 in x and y, 4 to 7 in z and t
-        __syncwarp();
-        {
-            // thread r: the forward (0) or backward (1) neighbours
-            const int* ex = fx_exponents(in, g.stride);
-            int c[4], s, top = 0, low = 1 << 30;
-            spins = 0;
-            site_of_half(h, p, g, c, s);
-#pragma unroll
-            for (int mu = 0; mu < 4; mu++) {
-                const int smu = mu == 0 ? 1 : mu == 1 ? g.L[0] : mu == 2 ? g.L[0] * g.L[1] : g.L[0] * g.L[1] * g.L[2];
-                const bool w = c[mu] == (r ? 0 : g.L[mu] - 1);
-                const int step = r ? -smu : smu;
-                const int hn = (w ? s - step * (g.L[mu] - 1) : s + step) >> 1;
-                const int ew = __ldg(ex + hn), e = ew & kFxExpMask;
-                spins |= ew >> 12 << (mu < 2 ? 0 : 4);
-                top = max(top, e);
-                low = min(low, e);
-                T.nb[2 * mu + r][t.sl] = make_int2(hn | (w ? (int)0x80000000 : 0), e);
-            }
-            t.top = max(top, __shfl_xor_sync(0xffffffffu, top, 16));
-            bad = min(low, __shfl_xor_sync(0xffffffffu, low, 16)) == 0;
-            spins |= __shfl_xor_sync(0xffffffffu, spins, 16);
+    if constexpr (RED) {
+        for (int h0 = sb * SITES; h0 < P.g.Vh; h0 += nb * SITES) {
+            const FxDone d = fx_sites_call<RED>(P, T, in, p, k, h0);
+            nrm += d.n2;
+            if (d.redo) nrm += fx_redo_sites(P, w, TB, p, k, h0 + 16 * warp, d.redo, 0, 1, OUTFX);
         }
-        __syncwarp();
-        {
-            const int hn = T.nb[3][t.sl].x & 0x7FFFFFFF;
-            fx_issue_link<TB>(T.l[0], P.u.p, (1 - p) * 4 + 1, hn, r, t.sl, g.stride);
-            fx_issue_spinor<1>(T, in, hn, r, g.stride);
-        }
-        FxSums A;
-#pragma unroll
-        for (int i = 0; i < 3; i++)
-#pragma unroll
-            for (int z = 0; z < 2; z++) A.up[i][z] = A.lo[0][i][z] = A.lo[1][i][z] = 0;
-        bad |= fx_turn_hop<0>(P, T, A, t, in);
-        bad |= fx_turn_hop<1>(P, T, A, t, in);
-        fx_negate_if(A.lo[0], r);
-        bad |= fx_turn_hop<2>(P, T, A, t, in);
-        bad |= fx_turn_hop<3>(P, T, A, t, in);
-        bad |= fx_turn_hop<4>(P, T, A, t, in);
-        bad |= fx_turn_hop<5>(P, T, A, t, in);
-        fx_negate_if(A.lo[1], r);
-        bad |= fx_turn_hop<6>(P, T, A, t, in);
-        bad |= fx_turn_hop<7>(P, T, A, t, in);
-        const int top = t.top;
-        // spin 3 - r: this thread's x and y part, the other's z and t part
-#pragma unroll
-        for (int i = 0; i < 3; i++)
-#pragma unroll
-            for (int z = 0; z < 2; z++) A.lo[0][i][z] += __shfl_xor_sync(0xffffffffu, A.lo[1][i][z], 16);
-        if (P.dag) fx_negate_if(A.lo[0], 1);
-        {
-            // the guard, but for a spin to which only zeros contribute (row q: spin q, and 3 - q in x and y, 2 + q in z and t)
-            bool up = false, lo = false;
-#pragma unroll
-            for (int i = 0; i < 3; i++) {
-                const unsigned zt = fx_swap(A.k[2][i]) + A.k[3][i], zt1 = __shfl_xor_sync(0xffffffffu, zt, 16);
-                up = up || fx_below(A.k[0][i] + A.k[1][i] + A.k[2][i] + A.k[3][i]);
-                lo = lo || fx_below(fx_swap(A.k[0][i]) + A.k[1][i] + zt1);
-            }
-            const int xy = (1 << r | 8 >> r) & spins, zt = (1 << r | 4 << r) & spins >> 4, zt1 = (2 >> r | 8 >> r) & spins >> 4;
-            bad = bad || (up && (xy | zt)) || (lo && (xy | zt1));
-            const int bad2 = __shfl_xor_sync(0xffffffffu, (int)bad, 16);
-            bad = bad || bad2;
-        }
-        if constexpr (OUTFX) {
-            // to 58 bits below the largest component: shift right by sr, left if negative
-            unsigned long long mu = 0, ml = 0;
-#pragma unroll
-            for (int i = 0; i < 3; i++)
-#pragma unroll
-                for (int z = 0; z < 2; z++) {
-                    mu |= (unsigned long long)(A.up[i][z] ^ (A.up[i][z] >> 63));
-                    ml |= (unsigned long long)(A.lo[0][i][z] ^ (A.lo[0][i][z] >> 63));
-                }
-            unsigned long long m = mu | ml;
-            m |= __shfl_xor_sync(0xffffffffu, m, 16);
-            int nz = (mu ? 1 << r : 0) | (ml ? 8 >> r : 0);
-            nz |= __shfl_xor_sync(0xffffffffu, nz, 16);
-            const int sr = m ? 6 - __clzll((long long)m) : 0;
-            const int eo = m ? top + 2 + sr : kFxEmin;
-            bad = bad || eo < kFxEmin || eo > kFxEmax;
-            if (ok && !bad) {
-                const long long half = sr > 0 ? 1LL << (sr - 1) : 0;
-                char* out = P.out.p + (P.full ? p * P.out.pstep : 0) + k * P.out.rstep;
-                uint4* ob = reinterpret_cast<uint4*>(out) + h;
-#pragma unroll
-                for (int q = 0; q < 6; q++) {
-                    long long v[2];
-#pragma unroll
-                    for (int z = 0; z < 2; z++) {
-                        v[z] = q < 3 ? A.up[q][z] : A.lo[0][q - 3][z];
-                        v[z] = sr > 0 ? (v[z] + half) >> sr : v[z] << -sr;
-                    }
-                    ob[(long long)(q < 3 ? 3 * r + q : 6 - 3 * r + q) * g.stride] =
-                        make_uint4((unsigned)(v[0] >> kFxLimb), (unsigned)v[0] & kFxLow, (unsigned)(v[1] >> kFxLimb),
-                                   (unsigned)v[1] & kFxLow);
-                }
-                if (r == 0) fx_exponents(out, g.stride)[h] = eo | nz << 12;
-            }
-        } else if (ok && !bad) {
-            const FxBias b = fx_bias(top + 1 - 1023 - 56);
-            int c[4], s;
-            site_of_half(h, p, g, c, s);
-            uint4* out = const_cast<uint4*>(fx_at(P.out, p, k, s));
-            const uint4* x = P.xpay ? fx_at(P.x, p, k, s) : nullptr;
-            double2 v[3];
-#pragma unroll
-            for (int i = 0; i < 3; i++) v[i] = make_double2(fx_double(A.up[i][0], b), fx_double(A.up[i][1], b));
-            fx_finish(P, out, x, 3 * r, v);
-            if (RED) nrm += fx_norm(v);
-#pragma unroll
-            for (int i = 0; i < 3; i++) v[i] = make_double2(fx_double(A.lo[0][i][0], b), fx_double(A.lo[0][i][1], b));
-            fx_finish(P, out, x, 9 - 3 * r, v);
-            if (RED) nrm += fx_norm(v);
-        }
-        const unsigned redo = __ballot_sync(0xffffffffu, ok && bad) & 0xFFFFu;
-        if (redo) {
-            const int warp = threadIdx.x >> 5;  // the warp's columns of T.s, all of whose copies have arrived
-            const double n2 = fx_redo_sites(P, reinterpret_cast<double2*>(&T.s[0][32 * warp]), TB, p, k, h0 + 16 * warp, redo, 0, 1, OUTFX);
-            if (RED) nrm += n2;
-        }
-        if (!RED) break;
+    } else {  // the grid covers the sites
+        const FxDone d = fx_sites<OUTFX, RED>(P, T, in, p, k, sb * SITES);
+        if (d.redo) fx_redo_sites(P, w, TB, p, k, sb * SITES + 16 * warp, d.redo, 0, 1, OUTFX);
     }
     pdl_trigger();
     if (RED) grid_reduce(nrm, P.red, k, nb * gridDim.y, sb + nb * blockIdx.y);
