@@ -507,8 +507,12 @@ int wilson_gauge_create(wilson_gauge** out, const double* canon, const wilson_la
         }
         DevBuf tmp;
         const double* d = device_view(canon, sizeof(double) * 72 * 2 * (size_t)g.Vh, tmp, st);
-        pack_gauge(h->f, d, st);
-        WL_CUDA(cudaStreamSynchronize(st));
+        if (h->f.fx.p) {
+            if (!pack_gauge_fx(h->f, d, st)) h->f.fx.release();
+        } else {
+            pack_gauge(h->f, d, st);
+            WL_CUDA(cudaStreamSynchronize(st));
+        }
         *out = h.release();
     });
 }

@@ -201,6 +201,9 @@ __host__ __device__ __forceinline__ FxCplx fx_cross(const FxCplx& a, const FxCpl
     fx_mac(i, fx_neg(c.im), d.re);
     return FxCplx{fx_requant(r.hh, r.mid), fx_requant(i.hh, i.mid)};
 }
+// Whether the high limb of such an entry is in the links' range.  A component can reach 6.25, and wraps from 4 on
+// to -4 .. -1.75: still out of it.
+__host__ __device__ __forceinline__ bool fx_limb_fits(int h) { return (unsigned)h + kFxLinkLimb <= 2u * kFxLinkLimb; }
 __host__ __device__ __forceinline__ void fx_recon_row2(FxCplx U[3][3]) {
 #pragma unroll
     for (int q = 0; q < 3; q++) {

@@ -229,10 +229,12 @@ __global__ void pack_gauge_kernel(const double2* __restrict__ canon, char* base,
 }
 
 // F64 links in fixed point (fx.cuh): nine words per link whatever R, the third row
-// rebuilt for R = 12; a link out of range is marked.  DBL: the doubles too.
+// rebuilt for R = 12; a link out of range is marked, and counted if bad is not null.  DBL: the doubles too.
 template <int R, bool DBL>
-__global__ void pack_gauge_fx_kernel(const double2* __restrict__ canon, char* base, uint4* fx, Geom g) {
+__global__ void pack_gauge_fx_kernel(const double2* __restrict__ canon, char* base, uint4* fx, Geom g,
+                                     unsigned long long* bad) {
     const long long V = 2LL * g.Vh;
+    unsigned misfits = 0;
     for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < V; s += (long long)gridDim.x * blockDim.x) {
         const int p = site_parity((int)s, g);
         const int h = (int)(s >> 1);
@@ -256,9 +258,10 @@ __global__ void pack_gauge_fx_kernel(const double2* __restrict__ canon, char* ba
             if (R == 12) {
                 fx_recon_row2(f);  // a third row of rows that are no SU(3) ones can be larger
 #pragma unroll
-                for (int k = 0; k < 3; k++) fits = fits && abs(f[2][k].re.h) <= kFxLinkLimb && abs(f[2][k].im.h) <= kFxLinkLimb;
+                for (int k = 0; k < 3; k++) fits = fits && fx_limb_fits(f[2][k].re.h) && fx_limb_fits(f[2][k].im.h);
             }
             if (!fits) f[0][0].re.h = (int)kFxBadLink;
+            misfits += !fits;
             uint4* b = fx + (size_t)(p * 4 + mu) * 9 * g.stride + h;
 #pragma unroll
             for (int k = 0; k < 9; k++) {
@@ -268,9 +271,23 @@ __global__ void pack_gauge_fx_kernel(const double2* __restrict__ canon, char* ba
             }
         }
     }
+    if (bad) {
+        misfits = __reduce_add_sync(0xffffffffu, misfits);
+        if (misfits && (threadIdx.x & 31) == 0) atomicAdd(bad, (unsigned long long)misfits);
+    }
 }
 
-void pack_gauge(GaugeField& gf, const double* canon, cudaStream_t st) {
+bool pack_gauge_fx(GaugeField& gf, const double* canon, cudaStream_t st) {
+    DevBuf bad(sizeof(unsigned long long));
+    WL_CUDA(cudaMemsetAsync(bad.p, 0, bad.bytes, st));
+    pack_gauge(gf, canon, st, bad.as<unsigned long long>());
+    unsigned long long n = 0;
+    WL_CUDA(cudaMemcpyAsync(&n, bad.p, sizeof(n), cudaMemcpyDeviceToHost, st));
+    WL_CUDA(cudaStreamSynchronize(st));
+    return n * 12 <= 8ULL * gf.g.Vh;
+}
+
+void pack_gauge(GaugeField& gf, const double* canon, cudaStream_t st, unsigned long long* bad) {
     const long long V = 2LL * gf.g.Vh;
     const int block = 256, grid = grid_for(V, block);
     const double2* src = reinterpret_cast<const double2*>(canon);
@@ -279,10 +296,10 @@ void pack_gauge(GaugeField& gf, const double* canon, cudaStream_t st) {
     const int R = gf.recon;
     if (p == P_F64 && gf.fx.p) {
         uint4* fx = gf.fx.as<uint4>();
-        if (R == 18 && base) pack_gauge_fx_kernel<18, true><<<grid, block, 0, st>>>(src, base, fx, gf.g);
-        else if (R == 18) pack_gauge_fx_kernel<18, false><<<grid, block, 0, st>>>(src, base, fx, gf.g);
-        else if (base) pack_gauge_fx_kernel<12, true><<<grid, block, 0, st>>>(src, base, fx, gf.g);
-        else pack_gauge_fx_kernel<12, false><<<grid, block, 0, st>>>(src, base, fx, gf.g);
+        if (R == 18 && base) pack_gauge_fx_kernel<18, true><<<grid, block, 0, st>>>(src, base, fx, gf.g, bad);
+        else if (R == 18) pack_gauge_fx_kernel<18, false><<<grid, block, 0, st>>>(src, base, fx, gf.g, bad);
+        else if (base) pack_gauge_fx_kernel<12, true><<<grid, block, 0, st>>>(src, base, fx, gf.g, bad);
+        else pack_gauge_fx_kernel<12, false><<<grid, block, 0, st>>>(src, base, fx, gf.g, bad);
         WL_LAUNCH_CHECK();
         return;
     }

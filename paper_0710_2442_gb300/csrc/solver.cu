@@ -563,13 +563,22 @@ std::vector<SolveStats> cg_solve_prepared(SpinorField& x, const SpinorField& b, 
 
 std::vector<SolveStats> cg_solve(double* xc, const double* gauge_canon, const double* bc, int nrhs, const Geom& g,
                                  double kappa, const SolveParams& prm, cudaStream_t st) {
+    // F64 links: in fixed point, those out of range read from the canonical ones; as
+    // doubles for the FP64 stencil where too many are
+    auto pack64 = [&](GaugeField& f) {
+        f.fx.alloc(gauge_bytes(P_F64, 18, g.stride));
+        f.canon = gauge_canon;
+        if (pack_gauge_fx(f, gauge_canon, st)) return;
+        f.fx.release();
+        f.canon = nullptr;
+        f.buf.alloc(gauge_bytes(P_F64, f.recon, g.stride));
+        pack_gauge(f, gauge_canon, st);
+    };
     GaugeField g64;
     g64.prec = P_F64;
     g64.recon = 18;
     g64.g = g;
-    g64.fx.alloc(gauge_bytes(P_F64, 18, g.stride));
-    g64.canon = gauge_canon;
-    pack_gauge(g64, gauge_canon, st);
+    pack64(g64);
     GaugeField glo;
     const GaugeField* inner_gauge = &g64;
     if (prm.inner != P_F64 || prm.recon != 18) {
@@ -577,12 +586,11 @@ std::vector<SolveStats> cg_solve(double* xc, const double* gauge_canon, const do
         glo.recon = prm.recon;
         glo.g = g;
         if (prm.inner == P_F64) {
-            glo.fx.alloc(gauge_bytes(P_F64, 18, g.stride));
-            glo.canon = gauge_canon;
+            pack64(glo);
         } else {
             glo.buf.alloc(gauge_bytes(prm.inner, prm.recon, g.stride));
+            pack_gauge(glo, gauge_canon, st);
         }
-        pack_gauge(glo, gauge_canon, st);
         inner_gauge = &glo;
     }
     // FP32 links for the FP32 outer residuals: the inner links when they are FP32

@@ -133,7 +133,7 @@ def test_conversions_agree(w, scale):
 
 
 @pytest.mark.parametrize("dims", [(4, 2, 4, 6), (12, 14, 16, 16)])
-@pytest.mark.parametrize("case", ["mean link", "all entries", "third row"])
+@pytest.mark.parametrize("case", ["mean link", "all entries", "third row", "third row of 4"])
 def test_links_at_the_edge_of_the_range(w, monkeypatch, dims, case):
     """Entries up to 1.25 stay in fixed point: SU(3) over a mean link of 0.8, and links whose every entry is as large
     as it may be, with a field that adds all products up; 12-real links whose third row leaves the range do not.
@@ -147,6 +147,10 @@ def test_links_at_the_edge_of_the_range(w, monkeypatch, dims, case):
     elif case == "all entries":
         U = np.full_like(U, 1.25 - 1.25j)
         src = np.full_like(src, 1.0 + 1.0j)
+    elif case == "third row of 4":  # its limb is 2^31
+        recon = 12
+        U[..., 0, :] = 1.0 + 1.0j
+        U[..., 1, :] = [1.0 - 1.0j, -1.0 + 1.0j, 1.0 - 1.0j]
     else:
         recon = 12
         U[..., 0, :] = 0.95 + 0.95j
@@ -282,3 +286,30 @@ def test_captured_handle_operators(w, oracle_mod):
         assert np.array_equal(x, y)
     assert_parity(got[0][0], oracle_mod.schur(U, src, dims, 0.13, 0, False, PHASES), TOL)
     assert_parity(got[0][1], oracle_mod.dslash_eo(U, src, dims, 1, PHASES), TOL)
+
+
+@pytest.mark.parametrize("dims", [(4, 4, 4, 6), (14, 14, 12, 18)])
+@pytest.mark.parametrize("part", [40, 20, 6, 1])
+def test_links_out_of_range_in_part(w, oracle_mod, dims, part):
+    """Every part-th link twice as large: a few are done over site by site, from a twelfth of them on
+    the handle runs on the FP64 stencil."""
+    U = inputs.gauge_field(dims, "random", seed=437)
+    U.reshape(-1, 3, 3)[::part] *= 2.0
+    src = inputs.gaussian_spinor(inputs.volume(dims) // 2, seed=438)
+    got = handle_hop(w, U, src, dims, PHASES, w.WILSON_F64, 18, 0, 0, w.WILSON_OP_SCHUR, 0.13)
+    assert_parity(got, oracle_mod.schur(U, src, dims, 0.13, 0, False, PHASES), TOL)
+
+
+@pytest.mark.parametrize("inner", ["f64", "f32"])
+def test_solve_with_links_out_of_range(w, oracle_mod, inner):
+    """Links twice as large and half of kappa are the same matrix."""
+    dims, kappa = (4, 4, 4, 8), 0.0675
+    U = 2.0 * inputs.gauge_field(dims, "weak", eps=0.3, seed=439)
+    b = inputs.gaussian_spinor(dims, seed=440)
+    p = w.solver_defaults(w.PREC[inner])
+    p.recon = 18
+    x = dev(np.zeros_like(b))
+    st = w.wilson_cg_solve(x, dev(U), dev(b), w.lattice(dims), kappa, p)
+    assert st["rc"] == 0
+    r = b - oracle_mod.wilson_m(U, host(x), dims, kappa)
+    assert np.linalg.norm(r) <= 1.1e-10 * np.linalg.norm(b)
