@@ -189,6 +189,23 @@ def workload_config(args, cfg, dims, apps, ws):
             "l2": L2_NOTE, "parallelism": "replicas" if ws > 1 else "single"}
 
 
+def timed_spans(steps, step, reset, event):
+    """Runs the steps and returns the (begin, end) events of what is timed: all of
+    them in one span, or with a reset, which runs before each step, each step in its own."""
+    if reset is None:
+        begin = event()
+        for _ in range(steps):
+            step()
+        return [(begin, event())]
+    spans = []
+    for _ in range(steps):
+        reset()
+        begin = event()
+        step()
+        spans.append((begin, event()))
+    return spans
+
+
 def run_ours(args, ws, rank, local, fields):
     import torch
     from paper_0710_2442_gb300 import build, wilson as w
@@ -228,26 +245,24 @@ def run_ours(args, ws, rank, local, fields):
             else:
                 w.wilson_dslash_h(e, g, o, 0.0, w.WILSON_OP_HOP, stream)
 
-    def device_step():
-        if args.prec == "f64":  # from the source again: thousands of hops in a row leave the FP64 range
-            even.load(src_dev, stream)
-        step()
+    # F64 steps begin with the source again, outside the timing: thousands of hops in a row
+    # leave the FP64 range
+    reset = (lambda: even.load(src_dev, stream)) if args.prec == "f64" else None
 
-    for _ in range(args.warmup):
-        device_step()
+    def event():
+        e = torch.cuda.Event(enable_timing=True)
+        e.record(stream)
+        return e
+
+    timed_spans(args.warmup, step, reset, event)
     torch.cuda.synchronize(dev)
-    start = torch.cuda.Event(enable_timing=True)
-    stop = torch.cuda.Event(enable_timing=True)
     with ClockSampler(local) as clk:
         barrier(ws)
         torch.cuda.synchronize(dev)
-        start.record(stream)
-        for _ in range(args.steps):
-            device_step()
-        stop.record(stream)
+        spans = timed_spans(args.steps, step, reset, event)
         torch.cuda.synchronize(dev)
         barrier(ws)
-    ms = start.elapsed_time(stop)
+    ms = sum(a.elapsed_time(b) for a, b in spans)
     ms = max_over_ranks(ms, ws)
     clocks = clk.summary()
     launches = args.steps * apps

@@ -52,3 +52,15 @@ def test_access_pattern_record_arithmetic():
     assert abs(rec["hop_over_access"] - 89.9 / 88.0) < 1e-3
     assert abs(rec["frac"] - byts / 88.0e-6 / 1e9 / 6791.7) < 1e-4
     assert rec["us"] == 88.0 and rec["hop_us"] == 89.9
+
+
+def test_reset_is_outside_the_timed_spans():
+    """A reset before each step takes no part in the time that is reported per launch."""
+    clock = [0]
+
+    def work(t):
+        clock[0] += t
+
+    spans = bench.timed_spans(3, lambda: work(10), lambda: work(7), lambda: clock[0])
+    assert sum(b - a for a, b in spans) == 30 and clock[0] == 51
+    assert bench.timed_spans(3, lambda: work(10), None, lambda: clock[0]) == [(51, 81)]
