@@ -23,15 +23,17 @@ FxField canonical(const void* p, int full) {
 template <bool OUTFX, bool RED>
 void launch_site(const FxParams& P, int blocks, int ny, cudaStream_t st) {
     auto k = hop_kernel_fx1<OUTFX, RED, kSiteThreads, kSiteBlocks>;
-    constexpr int smem = (int)sizeof(FxSlots<kSiteThreads>);
-    static_assert(smem <= 48 * 1024, "fits without the opt-in");
+    // and the turns' masks of sites to be done over (a field of more turns than fit does not fit the device's memory)
+    const int turns = RED ? (int)((P.g.Vh + (long long)blocks * (kSiteThreads / 2) - 1) / ((long long)blocks * (kSiteThreads / 2))) : 0;
+    const int smem = (int)sizeof(FxSlots<kSiteThreads>) + turns * (kSiteThreads / 32) * (int)sizeof(unsigned short);
+    WL_REQUIRE(smem <= 48 * 1024, "too few blocks for a reducing hop of this lattice");
     launch_dep_smem(k, dim3(blocks * P.nrhs, ny), dim3(kSiteThreads), smem, st, P);
 }
 
 template <bool FXL, bool RED>
 void launch_split(const FxParams& P, int tiles, int ny, cudaStream_t st) {
-    // up to one tile per SM, eight warps a tile are faster (8^4: 8.2 against 10.3 us);
-    // beyond, four (16^3 x 32: 43 against 48 us)
+    // up to one tile per SM, eight warps a tile are faster (8^4 with the Python call of then: 8.2
+    // against 10.3 us); beyond, four (16^3 x 32: 43 against 48 us)
     if (tiles * ny * P.nrhs <= device_sm_count())
         launch_dep(hop_kernel_fx<FXL, RED, 8, 2>, dim3(tiles * P.nrhs, ny), dim3(256), st, P);
     else launch_dep(hop_kernel_fx<FXL, RED, 4, kSplitBlocks>, dim3(tiles * P.nrhs, ny), dim3(128), st, P);

@@ -11,9 +11,10 @@
 //  read a site, the links when they are packed, and the Schur operator's intermediate
 //  field never leaves that form.  Two threads per site, one per half-spin row, sum
 //  the eight hops in 64-bit integers, with the next hop's words copied ahead.  About 180 instructions
-//  a thread and hop, bound by their issue (43 % of the slots; IMAD.WIDE at half rate), DRAM
-//  52 % busy.  A hop without the conversion (24^3 x 48 / 32^3 x 64): FP64 stencil 552 / 1648 us,
-//  here 111 / 329 us; with the conversion in every hop 166 / 512 us; with one thread
+//  a thread and hop.  No unit is saturated (16^3 x 32: issue 37 %, DRAM 49 %, L1 48 %, FP64 34 %
+//  busy): bound by the latency of the copies at 16 warps an SM, at 0.7 to 0.75 of the HBM time of what it
+//  reads.  A hop without the conversion (24^3 x 48 / 32^3 x 64): FP64 stencil 552 / 1648 us, here 114 / 333 us
+//  (111 / 329 before the guard of fx.cuh); with the conversion in every hop 166 / 512 us; with one thread
 //  per site and both rows (24 sums, 168 registers) 124 / 353 us.
 //
 //  hop_kernel_fx, small lattices.  A block works on 32 consecutive sites of one parity
@@ -22,7 +23,12 @@
 //  neighbour's components (and the link, if it comes as doubles) to fixed point,
 //  projects, multiplies, and leaves its half spinor as 64-bit integers in shared memory with one
 //  exponent per half-spin row.  After one barrier warp s adds up spin s: the
-//  eight hops aligned to their largest exponent, rounded to FP64 once.  8^4: 8.2 us.
+//  eight hops aligned to their largest exponent, rounded to FP64 once.  8^4: 6.7 us (a call's
+//  34 us on the FP64 stencil), 12^4: 11 us (37).
+//
+//  Both do a site over in FP64 where it is out of range or below the guard (fx_redo).  A lattice all of
+//  whose sites are takes 991 us on 24^3 x 48, 57 us on 12^4 and 25 us on 8^4 (FP64 stencil 552, 37 and 34 us);
+//  a lone site makes its block 2 to 5 us longer.
 #pragma once
 
 #include "dslash_impl.cuh"
@@ -259,7 +265,7 @@ __device__ __forceinline__ void fx_hop(const FxParams& P, FxTile& T, int j, int 
 // in dslash_impl.cuh) aligned to their largest exponent; returns whether a component is below
 // the guard (fx.cuh).  The sums become doubles with integer instructions
 // (INT) where a block is one of several on an SM: 12^4 F64 Schur 24.7 -> 24.0 us; one block of
-// eight warps on an SM is as fast or faster with the FP64 additions (8^4 hop 6.42 against 6.49 us).
+// eight warps on an SM is as fast or faster with the FP64 additions (8^4 hop, before the guard: 6.42 against 6.49 us).
 template <int SPIN, bool INT, int N>
 __device__ __forceinline__ bool fx_spin(const FxTile& T, int c0, int dag, int lane, double2 (&v)[N]) {
     constexpr bool lower = SPIN >= 2;
@@ -809,11 +815,6 @@ __device__ __forceinline__ FxDone fx_sites(const FxParams& P, FxSlots<TB>& T, co
     }
     return FxDone{nrm, __ballot_sync(0xffffffffu, ok && bad) & 0xFFFFu};
 }
-// For a loop over turns: in line, the call to fx_redo beside it costs the loop 40 registers' spills.
-template <bool RED, int TB>
-__device__ __noinline__ FxDone fx_sites_call(const FxParams& P, FxSlots<TB>& T, const char* in, int p, int k, int h0) {
-    return fx_sites<false, RED>(P, T, in, p, k, h0);
-}
 
 template <bool OUTFX, bool RED, int TB, int MINB>
 __global__ void __launch_bounds__(TB, MINB) hop_kernel_fx1(const __grid_constant__ FxParams P) {
@@ -831,11 +832,21 @@ __global__ void __launch_bounds__(TB, MINB) hop_kernel_fx1(const __grid_constant
     double2* w = reinterpret_cast<double2*>(&T.s[0][32 * warp]);  // the warp's columns, all of whose copies have arrived
     double nrm = 0.0;
     if constexpr (RED) {
-        for (int h0 = sb * SITES; h0 < P.g.Vh; h0 += nb * SITES) {
-            const FxDone d = fx_sites_call<RED>(P, T, in, p, k, h0);
+        // Turns, and then the sites to be done over: a call to fx_redo in the loop costs it 40
+        // registers' spills, a call for the turn 28 % of the hop's time.
+        unsigned short* redo = reinterpret_cast<unsigned short*>(fx_smem + sizeof(FxSlots<TB>)) + warp;  // [turn][warp]
+        int n = 0;
+        unsigned any = 0;
+        for (int h0 = sb * SITES; h0 < P.g.Vh; h0 += nb * SITES, n++) {
+            const FxDone d = fx_sites<OUTFX, RED>(P, T, in, p, k, h0);
             nrm += d.n2;
-            if (d.redo) nrm += fx_redo_sites(P, w, TB, p, k, h0 + 16 * warp, d.redo, 0, 1, OUTFX);
+            any |= d.redo;
+            if ((threadIdx.x & 31) == 0) redo[n * (TB / 32)] = (unsigned short)d.redo;
         }
+        __syncwarp();
+        if (any)
+            for (int i = 0; i < n; i++)
+                nrm += fx_redo_sites(P, w, TB, p, k, (sb + i * nb) * SITES + 16 * warp, redo[i * (TB / 32)], 0, 1, OUTFX);
     } else {  // the grid covers the sites
         const FxDone d = fx_sites<OUTFX, RED>(P, T, in, p, k, sb * SITES);
         if (d.redo) fx_redo_sites(P, w, TB, p, k, sb * SITES + 16 * warp, d.redo, 0, 1, OUTFX);

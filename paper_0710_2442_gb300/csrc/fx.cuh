@@ -14,10 +14,11 @@
 // scale (fields graded within a site, sparse or nearly diagonal links) would come out
 // worse than from FP64 arithmetic, whose error follows the terms.  So a hop adds up, for each
 // component, the moduli of its eight contributions, a lower bound of its terms', and where
-// they are below 3/16 of the scale (kFxGuard) the site is done over in FP64.  Between 3/16 and
-// 1/4 the error is 0.85 to 0.95 of the FP64 stencil's (root mean square; the worst inputs tried: unit
+// they are below 5/32 of the scale (kFxGuard) the site is done over in FP64.  Between 5/32 and
+// 3/16 the error is 0.9 to 1.0 of the FP64 stencil's (root mean square; the worst inputs tried: unit
 // links, components graded by up to 2^30), above it smaller, 0.35 to 0.4 where the eight hops
-// contribute alike.  Gaussian fields fall below it at four sites in a million.
+// contribute alike; between 4/32 and 5/32 it would be 1.06 to 1.14.  Gaussian fields fall
+// below the line at one to two sites in a million.
 //
 // Ranges, with the unit of a term at 2^58 = scale: |v.h| <= 2^29, |v.l| < 2^29 for
 // a component, twice that after the projection's one addition; a boundary phase makes the
@@ -47,7 +48,7 @@ static_assert(6 * kFxU * kFx2Sqrt2 + 8 < 32, "hh");
 static_assert(6 * (2 * kFxU + 2) < 32 && 6 * (kFxU + kFx2Sqrt2) < 32, "mid");
 static_assert(8 * 3 * kFxU * kFx2Sqrt2 / 2 * kFx2Sqrt2 < 128, "eight hops");
 // The guard: the contributions' moduli are counted in 256ths of the scale.
-constexpr unsigned kFxGuard = 48;
+constexpr unsigned kFxGuard = 40;
 
 // Right shifts that give 0 for counts of the word length and more.
 __host__ __device__ __forceinline__ unsigned fx_shr32(unsigned v, unsigned s) {
