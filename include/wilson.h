@@ -113,8 +113,10 @@ typedef struct {
 
 /* ---------------------------------------------------------------------- */
 /* Stateless calls on canonical complex128 device fields (Sec. 5, Eq. 3).  */
-/* FP64 results from 18-real links (computed in block fixed point, where    */
-/* that is at least as accurate, else in FP64).  Small lattices read links  */
+/* FP64 results from 18-real links: computed in block fixed point, and site */
+/* by site in FP64 where that is not as accurate for every component (fields */
+/* graded within a site, links above 1.25, exponents out of range; a lattice  */
+/* of such sites takes 1.5 times an FP64 stencil).  Small lattices read links */
 /* and fields as they are; larger ones convert them into workspace taken    */
 /* from a per-device memory pool of the library with stream-ordered         */
 /* allocation on the caller's stream (the pool keeps its memory, so only    */
@@ -304,7 +306,9 @@ int wilson_spinor_export(const wilson_spinor* s, double* canon, void* stream);
  * scheduled while the previous kernel on the stream drains, but they touch
  * no memory before that kernel has completed, so stream order holds for
  * every earlier operation.  The environment variable WILSON_PDL=0 launches
- * plainly. */
+ * plainly.  F64 hops of at least 20,000 output sites take workspace from a pool
+ * of the library on the stream (a field of the input's size); where there is none, and in a captured call, which allocates nothing, they run on the kernel of the
+ * smaller ones: the same accuracy, other last bits, 1.7 times the time. */
 int wilson_dslash_h(wilson_spinor* out, const wilson_gauge* g, const wilson_spinor* in, double kappa,
                     int op, void* stream);
 

@@ -28,7 +28,7 @@
 //
 //  Both do a site over in FP64 where it is out of range or below the guard (fx_redo).  A lattice all of
 //  whose sites are takes 991 us on 24^3 x 48, 57 us on 12^4 and 25 us on 8^4 (FP64 stencil 552, 37 and 34 us);
-//  a lone site makes its block 2 to 5 us longer.
+//  a lone site makes its block about 2 us longer.
 #pragma once
 
 #include "dslash_impl.cuh"

@@ -229,8 +229,9 @@ __global__ void pack_gauge_kernel(const double2* __restrict__ canon, char* base,
 }
 
 // F64 links in fixed point (fx.cuh): nine words per link whatever R, the third row
-// rebuilt for R = 12; a link out of range is marked, and counted if bad is not null.  DBL: the doubles too.
-template <int R, bool DBL>
+// rebuilt for R = 12; a link out of range is marked, and with COUNT counted.  DBL: the doubles too.  (The counter's ten
+// registers in a stateless call's pack would leave three blocks an SM: M on 16^3 x 32 98 -> 103 us.)
+template <int R, bool DBL, bool COUNT>
 __global__ void pack_gauge_fx_kernel(const double2* __restrict__ canon, char* base, uint4* fx, Geom g,
                                      unsigned long long* bad) {
     const long long V = 2LL * g.Vh;
@@ -261,7 +262,7 @@ __global__ void pack_gauge_fx_kernel(const double2* __restrict__ canon, char* ba
                 for (int k = 0; k < 3; k++) fits = fits && fx_limb_fits(f[2][k].re.h) && fx_limb_fits(f[2][k].im.h);
             }
             if (!fits) f[0][0].re.h = (int)kFxBadLink;
-            misfits += !fits;
+            if (COUNT) misfits += !fits;
             uint4* b = fx + (size_t)(p * 4 + mu) * 9 * g.stride + h;
 #pragma unroll
             for (int k = 0; k < 9; k++) {
@@ -271,7 +272,7 @@ __global__ void pack_gauge_fx_kernel(const double2* __restrict__ canon, char* ba
             }
         }
     }
-    if (bad) {
+    if (COUNT) {
         misfits = __reduce_add_sync(0xffffffffu, misfits);
         if (misfits && (threadIdx.x & 31) == 0) atomicAdd(bad, (unsigned long long)misfits);
     }
@@ -296,10 +297,18 @@ void pack_gauge(GaugeField& gf, const double* canon, cudaStream_t st, unsigned l
     const int R = gf.recon;
     if (p == P_F64 && gf.fx.p) {
         uint4* fx = gf.fx.as<uint4>();
-        if (R == 18 && base) pack_gauge_fx_kernel<18, true><<<grid, block, 0, st>>>(src, base, fx, gf.g, bad);
-        else if (R == 18) pack_gauge_fx_kernel<18, false><<<grid, block, 0, st>>>(src, base, fx, gf.g, bad);
-        else if (base) pack_gauge_fx_kernel<12, true><<<grid, block, 0, st>>>(src, base, fx, gf.g, bad);
-        else pack_gauge_fx_kernel<12, false><<<grid, block, 0, st>>>(src, base, fx, gf.g, bad);
+        auto pack = [&](auto RR, auto DBL) {
+            constexpr int r = decltype(RR)::value;
+            constexpr bool d = decltype(DBL)::value;
+            if (bad) pack_gauge_fx_kernel<r, d, true><<<grid, block, 0, st>>>(src, base, fx, gf.g, bad);
+            else pack_gauge_fx_kernel<r, d, false><<<grid, block, 0, st>>>(src, base, fx, gf.g, bad);
+        };
+        using std::bool_constant;
+        using std::integral_constant;
+        if (R == 18 && base) pack(integral_constant<int, 18>{}, bool_constant<true>{});
+        else if (R == 18) pack(integral_constant<int, 18>{}, bool_constant<false>{});
+        else if (base) pack(integral_constant<int, 12>{}, bool_constant<true>{});
+        else pack(integral_constant<int, 12>{}, bool_constant<false>{});
         WL_LAUNCH_CHECK();
         return;
     }
