@@ -23,7 +23,7 @@
 //  neighbour's components (and the link, if it comes as doubles) to fixed point,
 //  projects, multiplies, and leaves its half spinor as 64-bit integers in shared memory with one
 //  exponent per half-spin row.  After one barrier warp s adds up spin s: the
-//  eight hops aligned to their largest exponent, rounded to FP64 once.  8^4: 6.7 us (a call's
+//  eight hops aligned to their largest exponent, rounded to FP64 once.  8^4: 6.6 us (a call's
 //  34 us on the FP64 stencil), 12^4: 11 us (37).
 //
 //  Both do a site over in FP64 where it is out of range or below the guard (fx_redo).  A lattice all of
@@ -874,9 +874,10 @@ __device__ __forceinline__ unsigned fx_tile(const FxParams& P, FxTile& T, int p,
     double2 va[W == 8 ? 2 : 3], vb[1];  // warps 4 to 7: the third colour
     const bool below = warp < 4 ? fx_spin_of<W == 4>(T, spin, 0, P.dag, lane, va) : fx_spin_of<W == 4>(T, spin, 2, P.dag, lane, vb);
     if (below) T.bad[lane] = 1;
-    __syncthreads();
-    const bool bad = T.bad[lane];
-    if (ok && !bad) {
+    // with RED a site that is done over must not be in the sum; else it is stored twice (x is
+    // never the output), which puts the stores before the barrier: 8^4 hop 6.70 -> 6.64 us
+    if (RED) __syncthreads();
+    if (ok && !(RED && T.bad[lane])) {
         uint4* out = const_cast<uint4*>(fx_at(P.out, p, k, s));
         const uint4* x = P.xpay ? fx_at(P.x, p, k, s) : nullptr;
         if (warp < 4) {
@@ -887,7 +888,8 @@ __device__ __forceinline__ unsigned fx_tile(const FxParams& P, FxTile& T, int p,
             if (RED) nrm += fx_norm(vb);
         }
     }
-    return __ballot_sync(0xffffffffu, ok && bad);
+    if (!RED) __syncthreads();
+    return __ballot_sync(0xffffffffu, ok && T.bad[lane]);
 }
 template <int W>
 __device__ __forceinline__ double fx_tile_redo(const FxParams& P, FxTile& T, int p, int k, int h0, unsigned redo) {
